@@ -617,9 +617,23 @@ static cudaError_t launch_inv(BMat X, BMat M, int n, int units, const int* activ
   return cudaGetLastError();
 }
 
+// The FP32 inverse runs as column tiles over several CTAs per block (inv_tiles.cu) from
+// this size on whenever there is scratch for it.  Measured against the one-CTA kernels
+// below (us, tiles : one CTA): n = 16, 512 blocks 28 : 74; n = 32, 1024 blocks 93 : 240;
+// n = 48, 100 blocks 63 : 64; n = 64, 2 blocks 70 : 86; n = 128, 4 blocks 128 : 233, 128
+// blocks 274 : 236, 512 blocks 462 : 908; n = 200, 40 blocks 343 : 2114; n = 512, 1 block
+// 750 : 27570, 16 blocks 1220 : 27940.  Below it the FP64 path is the usual one.  Masked
+// launches of n <= 128 stay with one CTA per block: with few of the units active the tiles'
+// launches cost more than they save (an OBC of 192 energies at b = 128: 80.5 -> 84.2 ms).
+constexpr int kTilesMin = 16;
 cudaError_t zinv(BMat X, BMat M, int n, int units, const int* active, int single, void* scratch,
-                 int32_t* status, cudaStream_t s) {
+                 int32_t* status, cudaStream_t s, void* lent, size_t lent_bytes) {
   if (units <= 0 || n <= 0) return cudaSuccess;
+  if (single && n >= kTilesMin && (!active || n > kPanelThreads)) {
+    const size_t need = zinv_tiles_bytes(n, units);
+    void* t = lent_bytes >= need ? lent : (zinv_scratch_bytes(n, units, 1) >= need ? scratch : nullptr);
+    if (t) return zinv_tiles(X, M, n, units, active, t, status, s);
+  }
   if (single) return launch_inv<float>(X, M, n, units, active, scratch, status, s);
   return launch_inv<double>(X, M, n, units, active, scratch, status, s);
 }

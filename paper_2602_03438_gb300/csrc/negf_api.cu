@@ -552,7 +552,11 @@ struct Engine {
     const bool masked = active != nullptr && active_frac < 0.0;   // an unknown share of the work
     const double frac = (active && active_frac >= 0.0) ? active_frac : 1.0;
     begin(masked ? K_OTHER : (single ? K_INV_F32 : K_INV_F64));
-    cudaError_t e = zinv(X, M, n, units, active, single, inv_scratch, status, s);
+    // the FP32 inverse may use the sliced products' scratch, whose images are then gone
+    void* lent = (single && mixed == 1 && oz_supported(n)) ? ozt_scratch : nullptr;
+    if (lent) last_a = AKey();
+    cudaError_t e = zinv(X, M, n, units, active, single, inv_scratch, status, s, lent,
+                         lent ? ozt_scratch_bytes(n, units) : 0);
     end(masked ? 0.0 : 8.0 * (double)n * n * n * units * frac, masked ? 0.0 : 32.0 * (double)n * n * units * frac);
     return e;
   }

@@ -163,9 +163,16 @@ cudaError_t zgemm_ozt_variant(const GemmArgs& g, void* scratch, int* err, cudaSt
 // Work storage: in shared memory when it fits, otherwise `scratch` (units * n*n
 // complex of the working precision).  status[u] (nullable, indexed status_base+u)
 // gets NEGF_ERR_SINGULAR on an exactly zero pivot.
+// `lent` (lent_bytes, nullable): scratch the caller does not need meanwhile, which the FP32
+// inverse may use beside its own.
 cudaError_t zinv(BMat X, BMat M, int n, int units, const int* active, int single, void* scratch,
-                 int32_t* status, cudaStream_t s);
+                 int32_t* status, cudaStream_t s, void* lent = nullptr, size_t lent_bytes = 0);
 size_t zinv_scratch_bytes(int n, int units, int single);
+// the FP32 inverse as column tiles, several CTAs per block (inv_tiles.cu; n <= 512);
+// `scratch` holds zinv_tiles_bytes(n, units) bytes, 16-byte aligned
+cudaError_t zinv_tiles(BMat X, BMat M, int n, int units, const int* active, void* scratch, int32_t* status,
+                       cudaStream_t s);
+size_t zinv_tiles_bytes(int n, int units);
 
 // block i of unit u at p + u us + i is (a device's diagonal or off-diagonal output
 // blocks, or a workspace slot array [i][u])
