@@ -38,26 +38,6 @@ negf_status fail(Ctx* c, negf_status code, const std::string& msg) {
       return fail(ctx, NEGF_ERR_CUDA, std::string(#call) + ": " + cudaGetErrorString(e_)); \
   } while (0)
 
-// ---------------------------------------------------------------------------
-// one device of the (possibly uneven) batch, as the kernels see it
-// ---------------------------------------------------------------------------
-struct DevView {
-  const zc* Hd;   // block 0 of this device
-  const zc* Hu;
-  const zc* Sd;   // NULL => identity
-  const zc* Su;   // NULL => zero
-  const double* E;
-  double eta;
-  int nb, b;
-};
-
-struct ScatView {
-  const zc* sigR;        // NULL or this device's block 0 (energy 0)
-  const zc* sigL;
-  const double* scale;   // NULL or [ne][nb] of this device
-  long long e_stride;    // elements between energies (0 = shared)
-};
-
 struct Layout {
   int ndev;
   std::vector<long long> off;   // 8*(ndev+1)
@@ -155,14 +135,6 @@ ScatView scat_view(const negf_scattering* sc, const Layout& L, int d, int nb, in
   s.e_stride = sc->per_energy ? (long long)nb * bb : 0;
   return s;
 }
-
-// one device of an uneven batch as the batched sweeps over (device, energy) units see it
-struct UnitDev {
-  DevView dv;
-  ScatView sc;
-  const zc *sigma_L, *sigma_R;   // this device's lead blocks (energy 0)
-  const double *fL, *fR;         // this device's occupations (energy 0), nullable
-};
 
 // ---------------------------------------------------------------------------
 // assembly kernels (row a1 of the hot path): blocks of A = z S - H - Sigma and of
@@ -651,6 +623,7 @@ struct RgfIO {
   int32_t* status;               // device-offset, nullable
   bool lesser;
   bool greater = false;          // also G^> (with `lesser`)
+  bool allow_small = true;       // small blocks in one launch where supported
   const zc* W = nullptr;         // this device's W blocks (asm_w_kernel; Wd, Wu, Wl in turn), nullable
 };
 
@@ -685,7 +658,7 @@ negf_status rgf_chunk(Ctx* ctx, Engine& eng, const DevView& dv, const ScatView& 
   char* p = ws;
   auto slot = [&](int count) { zc* q = (zc*)p; p += blk * (size_t)U * count; return q; };
   // small blocks: the whole sweep in one launch over blocks assembled for every index
-  const bool small = !bp && rgf_small_supported(b, eng.mixed);
+  const bool small = !bp && io.allow_small && rgf_small_supported(b, eng.mixed);
   const int nd = small ? nb : 1, no = small ? std::max(nb - 1, 1) : 1;
   zc* Adiag = slot(nd);
   zc* Aup = slot(no);
@@ -1222,7 +1195,8 @@ size_t rgf_bytes_per_energy(int nb, int b, const RgfIO& io, int mixed) {
   const size_t blk = sizeof(zc) * (size_t)b * b;
   const bool greater = io.lesser && io.greater;
   size_t n = 3 + (io.lesser ? 1 : 0) + (greater ? 1 : 0) + 4 + std::max(nb - 1, 1);
-  if (rgf_small_supported(b, mixed))   // blocks assembled for every index (one launch)
+  const bool small = io.allow_small && rgf_small_supported(b, mixed);
+  if (small)   // blocks assembled for every index (one launch)
     n += (size_t)(nb - 1) * (1 + (io.lesser ? 1 : 0) + (greater ? 1 : 0)) + 2 * (size_t)(std::max(nb - 1, 1) - 1);
   if (!io.GRd) n += nb;
   if (io.lesser && !io.GLd) n += nb;
@@ -1231,7 +1205,7 @@ size_t rgf_bytes_per_energy(int nb, int b, const RgfIO& io, int mixed) {
   size_t bytes = n * blk;
   bytes += zinv_scratch_bytes(b, 1, mixed ? 1 : 0);
   // the sliced products' scratch, and a second one for the 5-digit correction products
-  if (mixed == 1) bytes += 2 * (ozt_scratch_bytes(b, 1) + 1024);
+  if (mixed == 1 && !small) bytes += 2 * (ozt_scratch_bytes(b, 1) + 1024);
   return bytes;
 }
 
@@ -2050,6 +2024,7 @@ negf_status rgf_batched_group(Ctx* ctx, Engine& eng, const negf_system* sys, con
   io.lesser = lesser;
   // per unit: the sweep workspace at the group's largest nb, the tables and two masks
   auto align = [](size_t x) { return (x + 255) & ~(size_t)255; };
+  io.allow_small = false;   // the work list sweeps step by step
   const size_t per = rgf_bytes_per_energy(max_nb, b, io, eng.mixed) + 4 * sizeof(int) + 2 * sizeof(long long) +
                      sizeof(int32_t) + 2 * sizeof(int) * (size_t)max_nb;
   const size_t fixed = align(sizeof(UnitDev) * ud.size()) + 8 * 256 + 2048;
@@ -2164,7 +2139,11 @@ static negf_status rgf_common(Ctx* ctx, const negf_system* sys, negf_precision p
     io.greater = lesser && (GG_diag || GG_low);
     io.status = status ? status + o[2] : nullptr;
     io.lesser = lesser;
-    const size_t per = rgf_bytes_per_energy(dv.nb, dv.b, io, eng.mixed);
+    size_t per = rgf_bytes_per_energy(dv.nb, dv.b, io, eng.mixed);
+    if (per > ctx->ws_bytes) {   // no room for every index's blocks of one energy: step by step
+      io.allow_small = false;
+      per = std::min(per, rgf_bytes_per_energy(dv.nb, dv.b, io, eng.mixed));
+    }
     // the device's W blocks (energy-independent part of A) ahead of the chunk workspace,
     // when there is room for them next to one energy
     const size_t wb = asm_w_bytes(dv.nb, dv.b);
@@ -2563,6 +2542,32 @@ negf_status negf_obc(negf_ctx* c, const negf_system* sys, negf_precision prec, d
       p = (char*)(((uintptr_t)p + 1023) & ~(uintptr_t)1023);
       eng.ozt_scratch = sl ? (void*)p : nullptr;
 
+      // small blocks without a guess: every lead unit's whole solve in one launch, one CTA
+      // per unit (FP64), where the steps below are a few hundred launches of a few
+      // microseconds and a read-back every fourth one (64 energies of blocks of 8: 7.06 -> 0.48 ms)
+      auto lead_at = [&](void* base) {   // nullable output blocks of the chunk's energies
+        if (!base) return BMat{nullptr, 0};
+        if (batched) return BMat{(zc*)base, 0, 0, 0, t_off};
+        return BMat{(zc*)base + o[3] + (long long)e0 * bb, bb};
+      };
+      if (b <= kObcSmallB && !any_warm) {
+        ObcSmall q;
+        q.dv = dv; q.e0 = e0; q.U = U; q.b = b; q.max_iter = max_iter;
+        q.udev = t_udev; q.unit_dev = t_dev; q.unit_e = t_e;
+        q.tol = tol; q.target = target;
+        q.sigma_L = lead_at(sigma_L); q.sigma_R = lead_at(sigma_R);
+        q.gs_L = lead_at(gs_L); q.gs_R = lead_at(gs_R);
+        q.done = done; q.iters = it_arr; q.nsteps = nsteps; q.res = res;
+        ctx->launches += 2;
+        CU(obc_small(q, s));
+        const long long ob = batched ? 0 : o[2] + e0;
+        obc_finish_kernel<<<(U + 127) / 128, 128, 0, s>>>(
+            done, res, it_arr, nsteps, U, status ? status + ob : nullptr, iters ? iters + 2 * ob : nullptr,
+            newton ? newton + 2 * ob : nullptr, accept, t_glob);
+        CU(cudaGetLastError());
+        continue;
+      }
+
       LeadArgs la{dv, e0, U, a00.p, al0.p, be0.p, eps.p, epss.p, al.p, be.p};
       la.udev = t_udev;
       la.unit_dev = t_dev;
@@ -2873,7 +2878,14 @@ negf_status negf_rgf_observables(negf_ctx* c, const negf_system* sys, negf_preci
     // no sweep-internal storage for them; set per chunk)
     io.GRd = io.GRu = io.GRl = io.GLd = io.GLl = (zc*)ctx->ws;
     const int sl = (T && prec == NEGF_MIXED && oz_supported(b)) ? 1 : 0;
-    const size_t per = gblocks * blk + rgf_bytes_per_energy(nb, b, io, eng.mixed) + observables_bytes_per_energy(dv, sl) + 3072;
+    auto bytes = [&]() {
+      return gblocks * blk + rgf_bytes_per_energy(nb, b, io, eng.mixed) + observables_bytes_per_energy(dv, sl) + 3072;
+    };
+    size_t per = bytes();
+    if (per > ctx->ws_bytes) {   // as in rgf_common
+      io.allow_small = false;
+      per = std::min(per, bytes());
+    }
     // the device's W blocks ahead of the chunks, when there is room for them next to one energy
     const size_t wb = asm_w_bytes(nb, b);
     const bool use_w = ctx->ws_bytes >= wb + per;

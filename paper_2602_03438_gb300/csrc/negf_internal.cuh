@@ -20,7 +20,7 @@ namespace negf {
 // is not recorded, so the next call retries it.
 // ---------------------------------------------------------------------------
 enum InitSlot { INIT_OZ = 0, INIT_OZS, INIT_OZP, INIT_OZT, INIT_TC, INIT_MLP, INIT_OZS_LO, INIT_OZP_LO, INIT_OZT_LO,
-                INIT_SMALL,
+                INIT_SMALL, INIT_OBC_SMALL,
                 INIT_NSLOT };
 constexpr int kMaxDevices = 64;
 cudaError_t once_per_device(int slot, const std::function<cudaError_t(int device)>& init);
@@ -181,6 +181,52 @@ struct SBlk {
   long long us, is;
   __host__ __device__ zc* at(int u, int i) const { return p + (long long)u * us + (long long)i * is; }
 };
+// ---------------------------------------------------------------------------
+// one device of the (possibly uneven) batch, as the kernels see it
+// ---------------------------------------------------------------------------
+struct DevView {
+  const zc* Hd;   // block 0 of this device
+  const zc* Hu;
+  const zc* Sd;   // NULL => identity
+  const zc* Su;   // NULL => zero
+  const double* E;
+  double eta;
+  int nb, b;
+};
+
+struct ScatView {
+  const zc* sigR;        // NULL or this device's block 0 (energy 0)
+  const zc* sigL;
+  const double* scale;   // NULL or [ne][nb] of this device
+  long long e_stride;    // elements between energies (0 = shared)
+};
+
+// one device of an uneven batch as the batched sweeps over (device, energy) units see it
+struct UnitDev {
+  DevView dv;
+  ScatView sc;
+  const zc *sigma_L, *sigma_R;   // this device's lead blocks (energy 0)
+  const double *fL, *fR;         // this device's occupations (energy 0), nullable
+};
+
+// the open boundary of blocks of b <= kObcSmallB in one launch, one CTA per lead unit (u < U:
+// the left lead of energy unit u, else the right lead of unit u - U), FP64: decimation to
+// convergence, Newton polishing, Sigma.  Energy unit k is energy e0 + k of `dv`, or energy
+// unit_e[k] of device udev[unit_dev[k]] when udev is given.  done, iters, nsteps, res
+// ([2U]) as the batched path leaves them; gs_L, gs_R nullable.
+constexpr int kObcSmallB = 16;
+struct ObcSmall {
+  DevView dv;
+  int e0, U, b, max_iter;
+  const UnitDev* udev;
+  const int *unit_dev, *unit_e;
+  double tol, target;
+  BMat sigma_L, sigma_R, gs_L, gs_R;
+  int *done, *iters, *nsteps;
+  double* res;
+};
+cudaError_t obc_small(const ObcSmall& a, cudaStream_t s);
+
 // the whole forward and backward sweep of U energies of one device with blocks of b <= 16
 // in one launch (one CTA per energy, FP64).  Ad [nb], Au/Al [nb-1], Sl/Sg [nb] hold the
 // assembled blocks with unit stride b*b and block stride U*b*b; Y: the workspace of the

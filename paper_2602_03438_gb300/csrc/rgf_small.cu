@@ -5,8 +5,10 @@
 //
 // At these sizes every block product is below the smallest tensor-core tile, and the
 // batched per-step launches (about 16 launches per block index) are bound by launch and
-// fill latency rather than by arithmetic: one CTA per energy with one thread per block
-// element does the same FP64 operations with no launch between them.
+// fill latency rather than by arithmetic: one CTA per energy with two threads per block
+// element (one per component, small_block.cuh) does the same FP64 operations with no launch
+// between them, bound by the FP64 pipe.  Measured (GB300): 64 energies of 16 blocks of 8,
+// G^R and G^<, 0.59 -> 0.35 ms against one thread per element.
 //
 // Forward, i = 0 .. nb-1 (Y_{i-1} = A_{i,i-1} g_{i-1}):
 //   g_i = (A_ii - Y_{i-1} A_{i-1,i})^{-1},
@@ -17,238 +19,125 @@
 //   G^x_ii = g^x_i + X P - W + W^H,  G^x_{i+1,i} = -G_{i+1,i+1} Z - P.
 // The block inverse is Gauss-Jordan with partial pivoting (first row of largest
 // modulus), in place, its row interchanges undone as column interchanges.
-#include "negf_internal.cuh"
+#include "small_block.cuh"
 
 namespace negf {
 
 namespace {
 
-constexpr int kSmallB = 16;
-constexpr int kSmallThreads = kSmallB * kSmallB;
 constexpr int kBufs = 13;
 
-// thread (r, c) owns element (r, c) of every b x b block in shared memory (row stride
-// ld = b + 1); a product op(A) op(B) is computed into a register by each owner, and the
-// callers synchronise the CTA before a block that others still read is overwritten
-struct Prod {
-  int b, ld, r, c;
-  bool on;   // this thread owns element (r, c)
-  __device__ zc mul(const zc* A, bool hA, const zc* B, bool hB) const {
-    zc acc = zmake(0.0, 0.0);
-    if (!on) return acc;
-    for (int k = 0; k < b; ++k) {
-      const zc a = hA ? zconj(A[k * ld + r]) : A[r * ld + k];
-      const zc v = hB ? zconj(B[c * ld + k]) : B[k * ld + c];
-      zfma(acc, a, v);
-    }
-    return acc;
-  }
-  __device__ zc get(const zc* A) const { return on ? A[r * ld + c] : zmake(0.0, 0.0); }
-  __device__ void put(zc* D, zc v) const {
-    if (on) D[r * ld + c] = v;
-  }
-};
-
-__device__ __forceinline__ void load_blk(zc* dst, const zc* src, const Prod& t) {
-  if (t.on) dst[t.r * t.ld + t.c] = src[t.r * t.b + t.c];
-}
-__device__ __forceinline__ void store_blk(zc* dst, zc v, const Prod& t) {
-  if (t.on) dst[t.r * t.b + t.c] = v;
-}
-
-// W <- W^{-1} in place (Gauss-Jordan, partial pivoting); returns false (to every thread)
-// when a pivot column is zero or not finite
-__device__ bool gj_inverse(zc* W, const Prod& t, int* piv, zc* s_dinv, int* s_p, int* s_sing) {
-  const int n = t.b, ld = t.ld, tid = threadIdx.x;
-  if (tid == 0) *s_sing = 0;
-  for (int k = 0; k < n; ++k) {
-    if (tid < 32) {
-      double best = -1.0;
-      int bi = n;
-      if (tid >= k && tid < n) {
-        best = zabs2(W[tid * ld + k]);
-        bi = tid;
-      }
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) {
-        const double ob = __shfl_down_sync(0xffffffffu, best, off);
-        const int oi = __shfl_down_sync(0xffffffffu, bi, off);
-        if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
-      }
-      if (tid == 0) {
-        if (!(best > 0.0)) { *s_sing = 1; bi = k; }
-        *s_p = bi;
-        piv[k] = bi;
-        const zc d = W[bi * ld + k];
-        const double den = zabs2(d);
-        *s_dinv = (den > 0.0) ? zmake(d.x / den, -d.y / den) : zmake(0.0, 0.0);
-      }
-    }
-    __syncthreads();
-    const int p = *s_p;
-    const zc dinv = *s_dinv;
-    zc nv = zmake(0.0, 0.0);
-    if (t.on) {
-      // row r of the interchanged matrix is row src of W
-      const int src = (t.r == k) ? p : ((t.r == p) ? k : t.r);
-      const zc prc = zmul(W[p * ld + t.c], dinv);   // the scaled pivot row, column c
-      if (t.r == k) {
-        nv = (t.c == k) ? dinv : prc;
-      } else {
-        const zc f = W[src * ld + k];
-        nv = (t.c == k) ? zmake(-(f.x * dinv.x - f.y * dinv.y), -(f.x * dinv.y + f.y * dinv.x))
-                        : zsub(W[src * ld + t.c], zmul(f, prc));
-      }
-    }
-    __syncthreads();
-    t.put(W, nv);
-    __syncthreads();
-  }
-  // undo the interchanges: swap columns k and piv[k], last pivot first
-  for (int k = n - 1; k >= 0; --k) {
-    const int p = piv[k];
-    if (p != k && tid < n) {
-      const zc a = W[tid * ld + k];
-      W[tid * ld + k] = W[tid * ld + p];
-      W[tid * ld + p] = a;
-    }
-    __syncthreads();
-  }
-  return *s_sing == 0;
-}
-
-__global__ void __launch_bounds__(kSmallThreads) rgf_small_kernel(SmallSweep a) {
+__global__ void __launch_bounds__(small_threads(kSmallB)) rgf_small_kernel(SmallSweep a) {
   const int u = blockIdx.x;
   const int b = a.b, nb = a.nb;
   const long long bb = (long long)b * b;
   const long long step = (long long)a.U * bb;   // stride of the assembled blocks' index
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int ld = b + 1;
   zc* buf[kBufs];
-  for (int q = 0; q < kBufs; ++q) buf[q] = reinterpret_cast<zc*>(smem_raw) + (size_t)q * b * ld;
+  for (int q = 0; q < kBufs; ++q) buf[q] = reinterpret_cast<zc*>(smem_raw) + (size_t)q * small_block_elems(b);
   __shared__ int piv[kSmallB];
-  __shared__ zc s_dinv;
-  __shared__ int s_p, s_sing;
-  Prod t;
-  t.b = b; t.ld = ld;
-  t.r = threadIdx.x / b; t.c = threadIdx.x - t.r * b;
-  t.on = threadIdx.x < bb;
+  const SmallElem t(b);
   bool ok = true;
 
-  // named roles; G/M and the kinds' running blocks swap by index
+  // named roles; G, M and the inverse's second block V swap by pointer
   zc *Al = buf[0], *Au = buf[1], *Yb = buf[2], *T1 = buf[3], *T2 = buf[4], *S = buf[5];
-  zc *X = buf[6], *Gu = buf[7], *P = buf[8];
-  int iG = 9, iM = 10;
+  zc *X = buf[6], *Gu = buf[7], *P = buf[8], *G = buf[9], *M = buf[10];
   zc* K[2] = {buf[11], buf[12]};
   const zc* sigx[2] = {a.Sl, a.Sg};
   const SBlk outx[2] = {a.gL, a.gG};
   const SBlk lowx[2] = {a.Ll, a.Gl};
+  // the adjacent lane's component of the transposed element, from shared memory
+  auto herm = [&](const zc* A) {   // this component of A^H at (r, c)
+    const double v = reinterpret_cast<const double*>(A + t.c * t.ld + t.r)[t.comp];
+    return t.comp ? -v : v;
+  };
 
   // ---------------- forward sweep
   for (int i = 0; i < nb; ++i) {
-    zc* M = buf[iM];
-    zc* G = buf[iG];   // g_{i-1}
-    load_blk(M, a.Ad + i * step + u * bb, t);
+    double m = t.get_g(a.Ad + i * step + u * bb);
     if (i > 0) {
-      load_blk(Al, a.Al + (i - 1) * step + u * bb, t);
-      load_blk(Au, a.Au + (i - 1) * step + u * bb, t);
-    }
-    __syncthreads();
-    if (i > 0) {
-      const zc y = t.mul(Al, false, G, false);   // Y_{i-1} = A_{i,i-1} g_{i-1}
+      t.put(Al, t.get_g(a.Al + (i - 1) * step + u * bb));
+      t.put(Au, t.get_g(a.Au + (i - 1) * step + u * bb));
+      __syncthreads();
+      const double y = t.mul(Al, G);   // Y_{i-1} = A_{i,i-1} g_{i-1}
       t.put(Yb, y);
-      store_blk(a.Y.at(u, i - 1), y, t);
+      t.put_g(a.Y.at(u, i - 1), y);
       __syncthreads();
-      const zc m = zsub(t.get(M), t.mul(Yb, false, Au, false));
-      __syncthreads();
-      t.put(M, m);
-      __syncthreads();
+      m -= t.mul(Yb, Au);
     }
-    ok = gj_inverse(M, t, piv, &s_dinv, &s_p, &s_sing) && ok;   // M <- g_i
-    store_blk(a.gR.at(u, i), t.get(M), t);
+    t.put(M, m);
+    __syncthreads();
+    ok = small_inverse(M, T2, t, piv) && ok;   // M <- g_i
+    t.put_g(a.gR.at(u, i), t.get(M));
     for (int x = 0; x < a.nk; ++x) {
-      load_blk(S, sigx[x] + i * step + u * bb, t);
-      __syncthreads();
-      zc v;
+      double v = t.get_g(sigx[x] + i * step + u * bb);
       if (i > 0) {
-        v = t.mul(Al, false, K[x], false);     // A_{i,i-1} g^x_{i-1}
-        t.put(T1, v);
+        t.put(T1, t.mul(Al, K[x]));               // A_{i,i-1} g^x_{i-1}
         __syncthreads();
-        v = zadd(t.mul(T1, false, Al, true), t.get(S));
-        t.put(T2, v);
-      } else {
-        t.put(T2, t.get(S));
+        v += t.mul<false, true>(T1, Al);
       }
+      t.put(T2, v);
       __syncthreads();
-      v = t.mul(M, false, T2, false);
-      t.put(T1, v);
+      v = t.mul(M, T2);
+      t.put(S, v);
       __syncthreads();
-      v = t.mul(T1, false, M, true);           // g^x_i
+      v = t.mul<false, true>(S, M);               // g^x_i
       t.put(K[x], v);
-      store_blk(outx[x].at(u, i), v, t);
+      t.put_g(outx[x].at(u, i), v);
       __syncthreads();
     }
-    const int sw = iG; iG = iM; iM = sw;   // G <- g_i
+    zc* sw = G; G = M; M = sw;   // G <- g_i
   }
   // ---------------- backward sweep (G holds G_{i+1,i+1}, K[x] G^x_{i+1,i+1})
   for (int i = nb - 2; i >= 0; --i) {
-    zc* G = buf[iG];
-    zc* M = buf[iM];
-    load_blk(Au, a.Au + i * step + u * bb, t);
-    load_blk(Al, a.Al + i * step + u * bb, t);
-    load_blk(M, a.gR.at(u, i), t);    // g_i
-    load_blk(Yb, a.Y.at(u, i), t);
     __syncthreads();
-    zc v = t.mul(M, false, Au, false);  // X = g_i A_{i,i+1}
-    t.put(X, v);
+    t.put(Au, t.get_g(a.Au + i * step + u * bb));
+    t.put(Al, t.get_g(a.Al + i * step + u * bb));
+    t.put(M, t.get_g(a.gR.at(u, i)));    // g_i
+    t.put(Yb, t.get_g(a.Y.at(u, i)));
     __syncthreads();
-    v = t.mul(X, false, G, false);      // G_{i,i+1} = -X G_{i+1,i+1}
-    v = zmake(-v.x, -v.y);
+    t.put(X, t.mul(M, Au));              // X = g_i A_{i,i+1}
+    __syncthreads();
+    double v = -t.mul(X, G);             // G_{i,i+1} = -X G_{i+1,i+1}
     t.put(Gu, v);
-    if (a.Ru.p) store_blk(a.Ru.at(u, i), v, t);
-    if (a.Rl.p) {
-      const zc w = t.mul(G, false, Yb, false);   // G_{i+1,i} = -G_{i+1,i+1} Y_i
-      store_blk(a.Rl.at(u, i), zmake(-w.x, -w.y), t);
-    }
-    __syncthreads();
+    if (a.Ru.p) t.put_g(a.Ru.at(u, i), v);
+    if (a.Rl.p) t.put_g(a.Rl.at(u, i), -t.mul(G, Yb));   // G_{i+1,i} = -G_{i+1,i+1} Y_i
     for (int x = 0; x < a.nk; ++x) {
-      load_blk(T2, outx[x].at(u, i), t);        // g^x_i
+      const double gx = t.get_g(outx[x].at(u, i));   // g^x_i
+      t.put(T2, gx);
       __syncthreads();
-      v = t.mul(Al, false, T2, false);          // Z = A_{i+1,i} g^x_i
-      t.put(T1, v);
-      v = t.mul(K[x], false, X, true);          // P = G^x_{i+1,i+1} X^H
-      t.put(P, v);
+      t.put(T1, t.mul(Al, T2));                 // Z = A_{i+1,i} g^x_i
+      const double pv = t.mul<false, true>(K[x], X);   // P = G^x_{i+1,i+1} X^H
+      t.put(P, pv);
       __syncthreads();
-      if (lowx[x].p) {                          // G^x_{i+1,i} = -G_{i+1,i+1} Z - P
-        const zc w = zadd(t.mul(G, false, T1, false), t.get(P));
-        store_blk(lowx[x].at(u, i), zmake(-w.x, -w.y), t);
-      }
-      v = t.mul(Gu, false, T1, false);          // W = G_{i,i+1} Z
-      t.put(S, v);
+      if (lowx[x].p) t.put_g(lowx[x].at(u, i), -(t.mul(G, T1) + pv));   // G^x_{i+1,i} = -G_{i+1,i+1} Z - P
+      const double w = t.mul(Gu, T1);           // W = G_{i,i+1} Z
+      t.put(S, w);
+      v = gx + t.mul(X, P);
       __syncthreads();
-      // G^x_ii = g^x_i + X P - W + W^H
-      v = zadd(t.get(T2), t.mul(X, false, P, false));
-      if (t.on) v = zadd(zsub(v, S[t.r * ld + t.c]), zconj(S[t.c * ld + t.r]));
-      __syncthreads();
+      v = (v - w) + herm(S);                    // G^x_ii = g^x_i + X P - W + W^H
       t.put(K[x], v);
-      store_blk(outx[x].at(u, i), v, t);
+      t.put_g(outx[x].at(u, i), v);
       __syncthreads();
     }
-    v = zsub(t.get(M), t.mul(Gu, false, Yb, false));   // G_ii = g_i - G_{i,i+1} Y_i
+    if (a.nk == 0) __syncthreads();
+    v = t.get(M) - t.mul(Gu, Yb);               // G_ii = g_i - G_{i,i+1} Y_i
     __syncthreads();
     t.put(M, v);
-    store_blk(a.gR.at(u, i), v, t);
-    __syncthreads();
-    const int sw = iG; iG = iM; iM = sw;   // G <- G_ii
+    t.put_g(a.gR.at(u, i), v);
+    zc* sw = G; G = M; M = sw;   // G <- G_ii
   }
   if (threadIdx.x == 0 && !ok && a.status) a.status[u] = NEGF_ERR_SINGULAR;
 }
 
 }  // namespace
 
-bool rgf_small_supported(int b, int mixed) { return b >= 1 && (b < 16 || (b == 16 && mixed == 0)); }
+// b = 16 reaches the sliced product's smallest tile in NEGF_MIXED, but seven eighths of its
+// 128 rows are padding there: a sweep of 256 energies, 8 blocks and both Keldysh kinds
+// took 8.5 ms step by step and takes 2.0 ms in one launch
+bool rgf_small_supported(int b, int mixed) { return b >= 1 && (b < 16 || (b == 16 && mixed != 2)); }
 
-size_t rgf_small_smem(int b) { return sizeof(zc) * (size_t)kBufs * b * (b + 1); }
+size_t rgf_small_smem(int b) { return sizeof(zc) * (size_t)kBufs * small_block_elems(b); }
 
 cudaError_t rgf_small_sweep(const SmallSweep& a, cudaStream_t s) {
   if (a.U <= 0) return cudaSuccess;
@@ -259,7 +148,7 @@ cudaError_t rgf_small_sweep(const SmallSweep& a, cudaStream_t s) {
                                 (int)rgf_small_smem(kSmallB));
   });
   if (e != cudaSuccess) return e;
-  rgf_small_kernel<<<a.U, kSmallThreads, smem, s>>>(a);
+  rgf_small_kernel<<<a.U, small_threads(a.b), smem, s>>>(a);
   return cudaGetLastError();
 }
 
