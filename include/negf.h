@@ -64,10 +64,10 @@ typedef enum {
 
 typedef enum {
   NEGF_FP64 = 0,       /* every product, inverse and reduction in FP64                      */
-  NEGF_MIXED = 1,      /* block products on the BF16 tensor cores with exact FP32
-                          accumulation of 7-bit digit slices (FP64-class: ~2^-55 of the
-                          row/column scales with the default 8 digits, see
-                          negf_sliced_digits; 16 <= b <= 512, K in exact passes of 256;
+  NEGF_MIXED = 1,      /* block products on the FP16 tensor cores with exact FP32
+                          accumulation of 8-bit digit slices (FP64-class: ~2^-54 of the
+                          row/column scales with the 7 digits of
+                          negf_sliced_digits; 16 <= b <= 512, K in exact passes of 128;
                           FP64 FMA otherwise); block inverses in FP32 + two refinement
                           steps whose residual uses the same product and whose correction
                           a 5-digit one; devices with b < 16 run their sweeps in FP64 (one
@@ -149,8 +149,8 @@ negf_status negf_worklist(const negf_system* sys, int32_t bs, int32_t* count, in
  * NEGF_ERR_NOCONV in status[e].  Sigma_L = a10 g_L a01, Sigma_R = a01 g_R a10.
  * prec: NEGF_FP64 runs every product in FP64; NEGF_MIXED runs the products of the
  * decimation, the residuals and the Newton steps on the digit-sliced BF16 tensor-core
- * path (FP64-class: exact FP32 accumulation of 7-bit slices, ~2^-55 of the row/column
- * scales with 8 digits) when 16 <= b <= 512, with the inverses in FP32 refined twice (twice
+ * path (FP64-class: exact FP32 accumulation of 8-bit slices, ~2^-54 of the row/column
+ * scales) when 16 <= b <= 512, with the inverses in FP32 refined twice (twice
  * more for units whose refinement residual stays above 1e-7) and redone in FP64 for any unit
  * still above it; NEGF_MIXED_TF32 is treated as NEGF_FP64 (a TF32 product is far too coarse
  * for the 1e-10 residual).
@@ -342,7 +342,7 @@ negf_status negf_observables(negf_ctx* ctx, const negf_system* sys, negf_precisi
  * by all units).  op: 0 = as stored, 2 = conjugate transpose.  alpha, beta: host
  * double[2] (re, im).  C may be NULL (beta ignored) or equal to D; D must not
  * overlap A or B.  NEGF_FP64: FP64 FMA; NEGF_MIXED: digit-sliced BF16 tensor-core
- * product for 16 <= n <= 512 (K in exact passes of 256); NEGF_MIXED_TF32: 3-term TF32 split for n >= 16
+ * product for 16 <= n <= 512 (K in exact passes of 128); NEGF_MIXED_TF32: 3-term TF32 split for n >= 16
  * (FP64 FMA outside those ranges). */
 negf_status negf_block_gemm(negf_ctx* ctx, negf_precision prec, int32_t n, int32_t units, int32_t opA,
                             int32_t opB, const double* alpha, const void* A, int64_t a_stride, const void* B,
@@ -391,11 +391,11 @@ negf_status negf_block_gemm_noalloc(int32_t n, int32_t units, int32_t opA, int32
                                     int64_t d_stride, int32_t* status, negf_stream stream);
 
 /* Autotuner of the NEGF_MIXED block products' tile shapes.  Variants:
- *   1 = half-width tiles (128 rows x 16 complex columns, two CTAs per SM; n <= 128),
- *   2 = persistent full-width tiles (128 x 32, the epilogue of one unit overlapping the
- *       next unit's MMAs; n <= 128),
- *   3 = full-width tiles, one CTA per tile (any n, K in exact passes of 256),
- *   0 = the built-in rule (1 for n <= 96, 2 for n <= 128, 3 above).
+ *   1 = tiles of 128 rows x 16 complex columns (n <= 128),
+ *   2 = tiles of 128 x 32 (n <= 128),
+ *   3 = tiles of 128 x 32 (any n, K in exact passes of 128),
+ *   0 = the built-in rule (the narrow tiles where they take fewer or no more rounds of the
+ *       GPU's SMs, else the wide ones).
  * negf_tune_products times every variant that supports n on `units` random n x n
  * products in the context's workspace (1 warm-up + 3 calls each, CUDA events on
  * `stream`), makes the fastest the context's choice for n and returns it in *choice
@@ -407,10 +407,10 @@ negf_status negf_tune_products(negf_ctx* ctx, int32_t n, int32_t units, int32_t*
                                negf_stream stream);
 negf_status negf_set_product_variant(negf_ctx* ctx, int32_t n, int32_t variant);
 
-/* Digits per value of the NEGF_MIXED sliced product in this build (NEGF_OZ_DIGITS at
- * compile time, 6..8; 8 by default): NS digits of 7 bits give an error of ~2^(1 - 7 NS)
- * of the row x column scales and NS (NS + 1) / 2 BF16 slice-pair products per complex
- * product.  Not a paper operation: build introspection for measurement. */
+/* Digits per value of the NEGF_MIXED block product (7, of 8 bits): ND digits give ND (ND +
+ * 1) / 2 FP16 slice products per complex product and an error of ~2^-54 of the row x
+ * column scales.  (negf_block_gemm_noalloc and calls whose workspace holds scales only
+ * use 8 digits of 7 bits in BF16.)  Not a paper operation: introspection for measurement. */
 int32_t negf_sliced_digits(void);
 
 /* Kernel timing (the tracing facility).  When enabled, every launch of the
@@ -420,8 +420,8 @@ int32_t negf_sliced_digits(void);
 negf_status negf_profile_enable(negf_ctx* ctx, int enable);
 /* Accumulated since the last reset: `launches` = all kernels this context has
  * launched; per kernel class k (0 = TF32-split GEMM, 1 = FP64 GEMM, 2 = FP32
- * inverse, 3 = FP64 inverse, 4 = other (masked launches), 5 = sliced BF16 GEMM,
- * 6 = sliced BF16 GEMM with 5 digits, the refinement's correction products)
+ * inverse, 3 = FP64 inverse, 4 = other (masked launches), 5 = sliced GEMM,
+ * 6 = sliced GEMM with 5 digits, the refinement's correction products)
  * the launches, total milliseconds,
  * algorithmic flops (8 n^3 per complex n x n product or inverse, times the
  * units) and algorithmic bytes (16 n^2 per operand read or written).  Each

@@ -426,9 +426,8 @@ struct Engine {
   bool can_slice(int n) const {
     return ozt_scratch ? oz_supported(n) : (oz_scratch != nullptr && oz_inkernel_supported(n));
   }
-  // op(A) of the last 8-digit digitize-once product whose scales and digit images are
-  // still in the scratch (n <= 128: the kernels whose images cover all of K); any other
-  // use of the scratch clears it
+  // op(A) of the last FP64-class product whose scales and digit images are still in the
+  // scratch; any other use of the scratch clears it
   struct AKey {
     const zc* p = nullptr;
     long long us = 0, us2 = 0;
@@ -456,17 +455,15 @@ struct Engine {
       return zgemm_oz(g, oz_scratch, ctx->d_err, s);
     }
     const int v = (g.n >= 0 && g.n <= 512) ? ctx->oz_variant[g.n] : OZ_DEFAULT;
-    const int eff = (v == OZ_DEFAULT) ? (g.n <= 96 ? OZ_HALF : g.n <= 128 ? OZ_PERSISTENT : OZ_FULL) : v;
-    const AKey k = key_of(g, eff, ozt_scratch);
-    const bool keepable = eff != OZ_FULL && g.n <= 128;
-    g.reuse_a = (reuse && keepable && last_a.p && last_a == k) ? 1 : 0;
+    const AKey k = key_of(g, v, ozt_scratch);
+    g.reuse_a = (reuse && last_a.p && last_a == k) ? 1 : 0;
     cudaError_t e = zgemm_ozt_variant(g, ozt_scratch, ctx->d_err, s, v);
     // the images stay valid for the next product unless this one overwrote its own A
-    last_a = (e == cudaSuccess && keepable && g.D.p != g.A.p) ? k : AKey();
+    last_a = (e == cudaSuccess && g.D.p != g.A.p) ? k : AKey();
     return e;
   }
   // a scratch region of the 5-digit product's own (set by the sweeps for their duration),
-  // so that its images leave the 8-digit product's in place; without it both share
+  // so that its images leave the FP64-class product's in place; without it both share
   // ozt_scratch
   void* ozt_scratch_lo = nullptr;
   cudaError_t sliced_lo(const GemmArgs& g) {
@@ -583,8 +580,8 @@ struct Engine {
         // digit images made before they start, and C and D element by element in one
         // thread, so D, A and C may all be X.  I - M X is small (below ~1e-3 when the
         // FP32 inverse is usable at all), so the correction X (I - M X) needs far less
-        // than FP64 class: the 5-digit product (15 slice pairs instead of 36, error
-        // ~2^-34 of |X| |I - M X|; 4 digits measured G^R 9e-8 against FP64 at config 2)
+        // than FP64 class: the 5-digit product (15 slice products instead of 28, error
+        // ~2^-39 of |X| |I - M X|)
         GemmArgs c;
         c.D = X; c.A = X; c.B = T1; c.C = X;
         c.opA = OP_N; c.opB = OP_N; c.alpha = zmake(1.0, 0.0); c.beta = zmake(1.0, 0.0);

@@ -19,8 +19,8 @@ namespace negf {
 // current, under a process-wide lock, at most once per (device, slot); a failed init
 // is not recorded, so the next call retries it.
 // ---------------------------------------------------------------------------
-enum InitSlot { INIT_OZ = 0, INIT_OZS, INIT_OZP, INIT_OZT, INIT_TC, INIT_MLP, INIT_OZS_LO, INIT_OZP_LO, INIT_OZT_LO,
-                INIT_SMALL, INIT_OBC_SMALL,
+enum InitSlot { INIT_OZ = 0, INIT_TC, INIT_MLP, INIT_SMALL, INIT_OBC_SMALL, INIT_OZB, INIT_OZB_LO, INIT_OZB16,
+                INIT_OZB16_LO,
                 INIT_NSLOT };
 constexpr int kMaxDevices = 64;
 cudaError_t once_per_device(int slot, const std::function<cudaError_t(int device)>& init);
@@ -134,26 +134,24 @@ __device__ __forceinline__ void raise_error(int* err, int code) {
 cudaError_t zgemm_f64(const GemmArgs& g, cudaStream_t s);
 // 3-term TF32-split complex GEMM on tcgen05 tensor cores (FP32 accumulate in TMEM)
 cudaError_t zgemm_tc(const GemmArgs& g, int* err, cudaStream_t s);
-// the sliced product with 5 digits per value (error ~2^-34 of the row x column norms),
-// for products whose result is a small correction; scratch as for zgemm_ozt (16 <= n <= 512)
+// the byte-digit product with 5 digits per value (error ~2^-39 of the row x column norms),
+// for products whose result is a small correction; scratch as for zgemm_ozt_variant
 cudaError_t zgemm_ozt_lo(const GemmArgs& g, void* scratch, int* err, cudaStream_t s);
 // one bounded device wait that runs out after limit_ns and raises NEGF_ERR_TIMEOUT on err
 cudaError_t wait_selftest(int* err, unsigned long long limit_ns, cudaStream_t s);
 bool tc_supported(int n);
-// FP64-class complex GEMM on the BF16 tensor cores (exact-accumulation digit slices);
-// `scratch` holds oz_scratch_bytes(n, units) bytes of per-row/column scales
+// FP64-class complex GEMM on the tensor cores by exact accumulation of digit slices, all
+// digits made in the kernel (BF16, 16 <= n <= 256); `scratch` holds oz_scratch_bytes(n,
+// units) bytes of per-row/column scales
 cudaError_t zgemm_oz(const GemmArgs& g, void* scratch, int* err, cudaStream_t s);
-bool oz_supported(int n);            // the digitize-once products (16 <= n <= 512)
-bool oz_inkernel_supported(int n);   // the in-kernel-digit product zgemm_oz (16 <= n <= 256)
+bool oz_inkernel_supported(int n);
 size_t oz_scratch_bytes(int n, int units);
-// the same product with each operand digitized once into global memory and streamed to
-// the tensor cores by bulk copies; `scratch` holds ozt_scratch_bytes(n, units) bytes
-cudaError_t zgemm_ozt(const GemmArgs& g, void* scratch, int* err, cudaStream_t s);
+// the same accuracy from byte digits (FP16, gemm_ozb.cu, 16 <= n <= 512), op(A)'s digits made
+// once into `scratch` (ozt_scratch_bytes(n, units) bytes) and streamed to the tensor cores
+bool oz_supported(int n);
 size_t ozt_scratch_bytes(int n, int units);
-// tile variants of the digitize-once product (the autotuner's choices): the default rule
-// by n, half-width 128 x 16 tiles with two CTAs per SM (n <= 128), persistent full-width
-// 128 x 32 tiles with the epilogue overlapping the next tile (n <= 128), full-width tiles
-// with one CTA per tile (any n)
+// tile variants (the autotuner's choices): the default rule, tiles of 16 complex columns
+// (n <= 128), tiles of 32 (n <= 128), tiles of 32 (any n)
 enum OzVariant { OZ_DEFAULT = 0, OZ_HALF = 1, OZ_PERSISTENT = 2, OZ_FULL = 3, OZ_NVARIANT = 4 };
 bool oz_variant_supported(int n, int variant);
 cudaError_t zgemm_ozt_variant(const GemmArgs& g, void* scratch, int* err, cudaStream_t s, int variant);
