@@ -28,90 +28,55 @@ cudaError_t once_per_device(int slot, const std::function<cudaError_t(int device
 }
 
 // ---------------------------------------------------------------------------
-// FP64 complex GEMM: D = alpha op(A) op(B) + beta C, one grid z-slice per unit.
-// Output tile TM x TM, 256 threads, (TM/16)^2 outputs per thread, K chunks of 16
-// staged through shared memory.  GB300 runs FP64 at ~1/60 of its FP32 rate, so
-// this kernel is bound by the FP64 pipe, not by memory.
+// FP64 complex GEMM: D = alpha op(A) op(B) + beta C, one thread per element of D (32
+// consecutive elements of the row-major block per warp), operands straight from L1/L2.
+// GB300's FP64 pipe takes 64 clocks per instruction and warp in each of an SM's four
+// partitions, so the kernel is bound by 4 n FP64 FMAs per element and nothing else: the
+// one load pair per 256 clocks of the pipe needs no staging, while square tiles spent
+// the pipe on padding.  With C: 96 units of n = 40 206 -> 55 us, 20 of 100 473 -> 149 us, 512 of
+// 8 71 -> 14 us, 128 of 128 2117 -> 1776 us (1.21 TFLOP/s).
 // ---------------------------------------------------------------------------
-template <int TM>
-__global__ void __launch_bounds__(256) zgemm_f64_kernel(GemmArgs g) {
-  const int u = blockIdx.z;
+constexpr int kF64Threads = 128;
+__global__ void __launch_bounds__(kF64Threads) zgemm_f64_kernel(GemmArgs g) {
+  const int u = blockIdx.y;
   if (g.active && !g.active[u]) return;
-  constexpr int KC = 16;
-  constexpr int R = TM / 16;
-  __shared__ zc As[KC][TM + 1];
-  __shared__ zc Bs[KC][TM + 1];
   const int n = g.n;
-  const int m0 = blockIdx.y * TM, n0 = blockIdx.x * TM;
-  const zc* A = g.A.at(u);
-  const zc* B = g.B.at(u);
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  zc acc[R][R];
+  const int e = blockIdx.x * kF64Threads + threadIdx.x;
+  if (e >= n * n) return;
+  const int r = e / n, c = e - r * n;
+  const bool hA = g.opA != OP_N, hB = g.opB != OP_N;
+  const zc* __restrict__ pa = g.A.at(u) + (hA ? r : (size_t)r * n);
+  const zc* __restrict__ pb = g.B.at(u) + (hB ? (size_t)c * n : c);
+  const int sa = hA ? n : 1, sb = hB ? 1 : n;
+  // conjugation by the sign bit (a negation chosen at run time is an FP64 instruction)
+  const int ma = hA ? (int)0x80000000 : 0, mb = hB ? (int)0x80000000 : 0;
+  auto flip = [](double x, int m) { return __hiloint2double(__double2hiint(x) ^ m, __double2loint(x)); };
+  zc acc = zmake(0.0, 0.0);
+  int k = 0;
+  for (; k + 4 <= n; k += 4) {
+    zc a[4], b[4];
 #pragma unroll
-  for (int i = 0; i < R; ++i)
-#pragma unroll
-    for (int j = 0; j < R; ++j) acc[i][j] = zmake(0.0, 0.0);
-
-  for (int k0 = 0; k0 < n; k0 += KC) {
-    for (int idx = threadIdx.x; idx < TM * KC; idx += 256) {
-      int mm, kk;
-      if (g.opA == OP_N) { kk = idx % KC; mm = idx / KC; }
-      else { mm = idx % TM; kk = idx / TM; }
-      const int gm = m0 + mm, gk = k0 + kk;
-      zc v = zmake(0.0, 0.0);
-      if (gm < n && gk < n) v = (g.opA == OP_N) ? A[(size_t)gm * n + gk] : zconj(A[(size_t)gk * n + gm]);
-      As[kk][mm] = v;
+    for (int q = 0; q < 4; ++q) {
+      a[q] = pa[(size_t)(k + q) * sa];
+      b[q] = pb[(size_t)(k + q) * sb];
     }
-    for (int idx = threadIdx.x; idx < TM * KC; idx += 256) {
-      int nn, kk;
-      if (g.opB == OP_N) { nn = idx % TM; kk = idx / TM; }
-      else { kk = idx % KC; nn = idx / KC; }
-      const int gn = n0 + nn, gk = k0 + kk;
-      zc v = zmake(0.0, 0.0);
-      if (gn < n && gk < n) v = (g.opB == OP_N) ? B[(size_t)gk * n + gn] : zconj(B[(size_t)gn * n + gk]);
-      Bs[kk][nn] = v;
-    }
-    __syncthreads();
-#pragma unroll 4
-    for (int kk = 0; kk < KC; ++kk) {
-      zc a[R], b[R];
 #pragma unroll
-      for (int i = 0; i < R; ++i) a[i] = As[kk][ty + 16 * i];
-#pragma unroll
-      for (int j = 0; j < R; ++j) b[j] = Bs[kk][tx + 16 * j];
-#pragma unroll
-      for (int i = 0; i < R; ++i)
-#pragma unroll
-        for (int j = 0; j < R; ++j) zfma(acc[i][j], a[i], b[j]);
-    }
-    __syncthreads();
+    for (int q = 0; q < 4; ++q)
+      zfma(acc, zmake(a[q].x, flip(a[q].y, ma)), zmake(b[q].x, flip(b[q].y, mb)));
   }
-  zc* D = g.D.at(u);
-  const zc* C = g.C.p ? g.C.at(u) : nullptr;
-#pragma unroll
-  for (int i = 0; i < R; ++i) {
-    const int gm = m0 + ty + 16 * i;
-    if (gm >= n) continue;
-#pragma unroll
-    for (int j = 0; j < R; ++j) {
-      const int gn = n0 + tx + 16 * j;
-      if (gn >= n) continue;
-      zc v = zmul(g.alpha, acc[i][j]);
-      if (C) v = zadd(v, zmul(g.beta, C[(size_t)gm * n + gn]));
-      D[(size_t)gm * n + gn] = v;
-    }
+  for (; k < n; ++k) {
+    const zc a = pa[(size_t)k * sa], b = pb[(size_t)k * sb];
+    zfma(acc, zmake(a.x, flip(a.y, ma)), zmake(b.x, flip(b.y, mb)));
   }
+  zc v = zmul(g.alpha, acc);
+  if (g.C.p) v = zadd(v, zmul(g.beta, g.C.at(u)[e]));
+  g.D.at(u)[e] = v;
 }
 
 cudaError_t zgemm_f64(const GemmArgs& g, cudaStream_t s) {
   if (g.units <= 0 || g.n <= 0) return cudaSuccess;
-  if (g.n <= 32) {
-    dim3 grid((g.n + 31) / 32, (g.n + 31) / 32, g.units);
-    zgemm_f64_kernel<32><<<grid, 256, 0, s>>>(g);
-  } else {
-    dim3 grid((g.n + 63) / 64, (g.n + 63) / 64, g.units);
-    zgemm_f64_kernel<64><<<grid, 256, 0, s>>>(g);
-  }
+  const dim3 grid((unsigned)(((long long)g.n * g.n + kF64Threads - 1) / kF64Threads), g.units);
+  zgemm_f64_kernel<<<grid, kF64Threads, 0, s>>>(g);
   return cudaGetLastError();
 }
 
