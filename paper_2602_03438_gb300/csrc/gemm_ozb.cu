@@ -23,9 +23,8 @@
 // [unit][row tile][chunk of 16 k][real, imaginary][digit], each plane 128 rows of 16 FP16
 // (32-byte swizzle); the digits of op(B) are made inside the kernel.  Real and imaginary
 // parts are separate planes (B: real, imaginary, negated imaginary): with A_s fixed,
-//   re += Ar_s Br, im += Ar_s Bi;  im += Ai_s Br, re += Ai_s (-Bi)
-// each over all of B's digit planes t < ND - s as one wide instruction; the A operand
-// stays in the collector for the instructions that share it.
+//   re += Ar_s Br, re += Ai_s (-Bi);  im += Ar_s Bi, im += Ai_s Br
+// each over all of B's digit planes t < ND - s as one wide instruction.
 //
 // One persistent CTA per SM walks (unit, row tile, column tile) in that order, so that the
 // column tiles that share an A image run side by side and read it from L2.  Warps 0-7
@@ -33,17 +32,20 @@
 // issues the MMAs.  All accumulators of a 128 x 32 tile fill the 512 TMEM columns, so the
 // next tile's MMAs wait for the drain: it only combines the groups into 64-bit integers in
 // registers; conversion, C and the stores (through shared memory, so that they are whole
-// 128-byte lines) overlap the next MMAs.
+// 128-byte lines) overlap the next MMAs.  A pass's real accumulators are complete, drained
+// and refilled ahead of its imaginary ones, so that half of a drain overlaps MMAs too.
 //
 // What bounds it (n = 128): shared-memory bandwidth.  A tile's MMAs take 14.3 k clocks of the
-// tensor pipe; their operands are read from shared memory for 10.9 k clocks, A's images
-// and B's digits are written for 5 k, the stores pass through it for 1-2 k; the drain
-// (256 KB of TMEM, 5 k clocks) is not overlapped.  Measured per 1024 units of n = 128 with
-// C, pre-pass included (the pre-pass, HBM bound, takes 140 us): 535 us, against 702 us
-// for 8 digits of 7 bits in BF16 with the drain through shared memory.  On the way:
-// issuing from one lane's branch 620 us (each MMA's descriptors pass between the register
-// files), a 64-bit FP conversion per output in place of the integer one 572 us, spilled
-// registers for want of the register split 624 us, eight producer warps 635 us.
+// tensor pipe, but their operands are read from shared memory for 14 k, A's images and B's
+// digits are written there for 5 k and the stores pass through it for 2 k; with the part of
+// the drain (256 KB of TMEM, 5 k clocks) that nothing overlaps a tile takes 26 k.  Measured
+// per 1024 units of n = 128 with C, pre-pass included (HBM bound, 140 us): 515 us, against
+// 702 us for 8 digits of 7 bits in BF16 with the drain through shared memory; 16 units of
+// n = 512: 425 against 955 us.  On the way (us per 1024 units of 128): issuing from one
+// lane's branch 620 (each MMA's descriptors pass between the register files), a 64-bit FP
+// conversion per output in place of the integer one 572, spilled registers for want of the
+// register split 624, eight producer warps 635, one drain of re and im together and three
+// waits per chunk 535.  A planes kept in the collector for two instructions each: no faster.
 #include <cuda_fp16.h>
 
 #include "negf_internal.cuh"
@@ -64,13 +66,14 @@ struct Cfg {
   static constexpr uint32_t A_PART = ND * A_PL;          // a chunk's real or imaginary planes (28 KB)
   static constexpr uint32_t B_PL = TNC * 32;             // one digit plane of a B part
   static constexpr uint32_t B_CHUNK = 3 * ND * B_PL;     // real, imaginary, negated imaginary planes (21 KB)
-  static constexpr int NA = 4, NB = 3;                   // ring stages (A parts, B chunks)
+  static constexpr uint32_t OFF_B = 2 * A_PART;          // of a stage: both A parts, then B
+  static constexpr uint32_t STAGE = OFF_B + B_CHUNK;
+  static constexpr int NSTG = ND == 7 ? 2 : 3;           // ring stages, one chunk each
   static constexpr int SPLIT = ND == 7 ? 4 : -1;         // the group with a spare accumulator
   static constexpr uint32_t COL_IM = ND * TNC;           // TMEM columns: re groups, im groups, spares
   static constexpr uint32_t COL_SP = 2 * ND * TNC;
   static constexpr uint32_t TMEM_COLS = TNC == 32 ? 512 : 256;
-  static constexpr uint32_t OFF_B = NA * A_PART;
-  static constexpr uint32_t OFF_ST = OFF_B + NB * B_CHUNK;   // per epilogue warp: 32 rows of 128 bytes
+  static constexpr uint32_t OFF_ST = NSTG * STAGE;       // per epilogue warp: 32 rows of 128 bytes
   static constexpr uint32_t OFF_BAR = OFF_ST + 8 * 4096;
   static constexpr uint32_t SMEM = OFF_BAR + 256 + 1024;
 };
@@ -135,8 +138,8 @@ __device__ __forceinline__ void mma_commit(uint64_t* bar, uint32_t el) {
                "r"(el)
                : "memory");
 }
-// the A collector: FILL reads A and keeps it, USE takes the kept one, LAST takes and drops it
-enum Collect { FILL, USE, LAST };
+// the A collector: FILL reads A and keeps it for LAST, which drops it; ONCE keeps nothing
+enum Collect { FILL, LAST, ONCE };
 template <int C>
 __device__ __forceinline__ void mma(uint32_t d, uint64_t a, uint64_t b, uint32_t id, uint32_t acc, uint32_t el) {
 #define NEGF_MMA(Q)                                                                                              \
@@ -145,8 +148,8 @@ __device__ __forceinline__ void mma(uint32_t d, uint64_t a, uint64_t b, uint32_t
                "l"(a), "l"(b), "r"(id), "r"(acc), "r"(el)                                                        \
                : "memory")
   if (C == FILL) NEGF_MMA("fill");
-  else if (C == USE) NEGF_MMA("use");
-  else NEGF_MMA("lastuse");
+  else if (C == LAST) NEGF_MMA("lastuse");
+  else NEGF_MMA("discard");
 #undef NEGF_MMA
 }
 // 1 in the one lane that issues for the warp
@@ -156,29 +159,34 @@ __device__ __forceinline__ uint32_t elect_one() {
   return e;
 }
 
-// One A part (its ND digit planes at `da`) against B's real and imaginary planes.  part 0:
-// re += Ar Br, im += Ar Bi (first: these initialise every accumulator); part 1:
-// im += Ai Br, re += Ai (-Bi).
-template <int ND, int TNC, int PART>
-__device__ __forceinline__ void part_mmas(uint32_t tmem, uint64_t da, uint64_t db, bool first, uint32_t el) {
+// One A part (its ND digit planes at `da`) against one set of B planes: the product goes to
+// the groups' columns from c on (spare accumulator at sp).  first: these MMAs initialise the
+// accumulators.  Rolled loops: a pass's unrolled MMAs are some 25 KB of straight-line code,
+// whose fetch held the issuing warp for a quarter of a tile's time.
+template <int ND, int TNC>
+__device__ __forceinline__ void part_mmas(uint32_t c, uint32_t sp, uint64_t a, uint64_t b, bool first, uint32_t el) {
   using T = Cfg<ND, TNC>;
-  constexpr uint32_t c_br = PART == 0 ? 0u : T::COL_IM, c_bi = PART == 0 ? T::COL_IM : 0u;   // columns of A Br, A Bi
-  constexpr uint32_t b_im = ((PART == 0 ? 1 : 2) * ND * T::B_PL) >> 4;   // Bi or -Bi
-  const uint32_t acc0 = (PART == 0 && first) ? 0u : 1u;
-#pragma unroll
-  for (int s = 0; s < ND; ++s) {
-    const uint64_t a = da + (uint64_t)((s * A_PL) >> 4);
-    if (s == T::SPLIT) {   // its product with t = 0 goes to the spare accumulators
-      constexpr int N1 = (ND - 1 - T::SPLIT) * TNC;
-      constexpr uint32_t sp_br = T::COL_SP + (PART == 0 ? 0 : TNC), sp_bi = T::COL_SP + (PART == 0 ? TNC : 0);
-      mma<FILL>(tmem + sp_br, a, db, idesc(TNC), acc0, el);
-      mma<USE>(tmem + c_br + (s + 1) * TNC, a, db + (T::B_PL >> 4), idesc(N1), 1u, el);
-      mma<USE>(tmem + sp_bi, a, db + b_im, idesc(TNC), acc0, el);
-      mma<LAST>(tmem + c_bi + (s + 1) * TNC, a, db + b_im + (T::B_PL >> 4), idesc(N1), 1u, el);
-    } else {
-      const uint32_t id = idesc((ND - s) * TNC), acc = s == 0 ? acc0 : 1u;
-      mma<FILL>(tmem + c_br + s * TNC, a, db, id, acc, el);
-      mma<LAST>(tmem + c_bi + s * TNC, a, db + b_im, id, acc, el);
+  const uint32_t acc0 = first ? 0u : 1u;
+  constexpr uint32_t STEP = A_PL >> 4, NSTEP = (uint32_t)(TNC >> 3) << 17;
+  uint32_t id = idesc(ND * TNC), acc = acc0;
+  constexpr int S1 = T::SPLIT > 0 ? T::SPLIT : ND;
+#pragma unroll 1
+  for (int s = 0; s < S1; ++s) {
+    mma<ONCE>(c, a, b, id, acc, el);
+    acc = 1u;
+    a += STEP;
+    c += TNC;
+    id -= NSTEP;
+  }
+  if (T::SPLIT > 0) {   // the split digit: its product with t = 0 goes to the spare accumulators
+    mma<FILL>(sp, a, b, idesc(TNC), acc0, el);
+    mma<LAST>(c + TNC, a, b + (T::B_PL >> 4), id - NSTEP, 1u, el);
+#pragma unroll 1
+    for (int s = S1 + 1; s < ND; ++s) {
+      a += STEP;
+      c += TNC;
+      id -= NSTEP;
+      mma<ONCE>(c, a, b, id, 1u, el);
     }
   }
 }
@@ -403,12 +411,16 @@ __device__ __forceinline__ double flip(double x, int mask) {
 template <int ND, int TNC, bool UAB>
 __global__ void __launch_bounds__(NT, 1) ozb_product_kernel(GemmArgs g, ImgArgs im, int* err) {
   using T = Cfg<ND, TNC>;
-  constexpr int NA = T::NA, NB = T::NB;
+  constexpr int NSTG = T::NSTG;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* base = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint64_t* bars = reinterpret_cast<uint64_t*>(base + T::OFF_BAR);
-  uint64_t *fullA = bars, *emptyA = bars + NA, *fullB = bars + 2 * NA, *emptyB = fullB + NB;
-  uint64_t *done = emptyB + NB, *tfree = done + 1, *fin = tfree + 1;
+  // full[s]: a chunk's A images (one expect_tx) and B digits (four warps); emptyR[s], emptyI[s]:
+  // its real and imaginary A planes are read (with the imaginary ones, B too)
+  uint64_t *full = bars, *emptyR = full + NSTG, *emptyI = emptyR + NSTG;
+  uint64_t *doneR = emptyI + NSTG, *doneI = doneR + 1;   // a pass's re, im accumulators are complete
+  uint64_t *freeR = doneI + 1, *freeI = freeR + 1;       // ... are drained
+  uint64_t* fin = freeI + 1;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(fin + 1);
   __shared__ volatile int s_fail;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -417,16 +429,15 @@ __global__ void __launch_bounds__(NT, 1) ozb_product_kernel(GemmArgs g, ImgArgs 
   const long long ntiles = (long long)g.units * per_unit;
 
   if (tid == 0) {
-    for (int i = 0; i < NA; ++i) {
-      mbar_init(&fullA[i], 1);
-      mbar_init(&emptyA[i], 1);
+    for (int i = 0; i < NSTG; ++i) {
+      mbar_init(&full[i], 5);
+      mbar_init(&emptyR[i], 1);
+      mbar_init(&emptyI[i], 1);
     }
-    for (int i = 0; i < NB; ++i) {
-      mbar_init(&fullB[i], 4);
-      mbar_init(&emptyB[i], 1);
-    }
-    mbar_init(done, 1);
-    mbar_init(tfree, 8);
+    mbar_init(doneR, 1);
+    mbar_init(doneI, 1);
+    mbar_init(freeR, 8);
+    mbar_init(freeI, 8);
     mbar_init(fin, 1);
     s_fail = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -452,14 +463,14 @@ __global__ void __launch_bounds__(NT, 1) ozb_product_kernel(GemmArgs g, ImgArgs 
   };
 
   // registers move between the warpgroups (each role's branch begins with its share):
-  // 2 x 184 + 88 + 56 = 512, the launch's 4 x 128 per lane
+  // 2 x 192 + 72 + 56 = 512, the launch's 4 x 128 per lane
   if (warp >= 12) {
    asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
    if (warp == 12) {
-    // ---------------- A: each chunk's real and imaginary planes into the ring.  The tiles of
-    // one image take turns prefetching it into L2, PF parts ahead.
+    // ---------------- A: each chunk's real and imaginary planes into its stage.  The tiles of
+    // one image take turns prefetching it into L2, PF chunks ahead.
     if (lane == 0) {
-      constexpr int PF = 6;
+      constexpr int PF = 3;
       int st = 0, issued = 0;
       uint32_t ph = 0;   // parity of the stage's last release
       bool filled = false;
@@ -467,18 +478,23 @@ __global__ void __launch_bounds__(NT, 1) ozb_product_kernel(GemmArgs g, ImgArgs 
         int u, tm, tn;
         if (!tile_at(i, u, tm, tn)) continue;
         const unsigned char* img = im.a + (size_t)(u * im.tiles_m + tm) * chunks * (2 * T::A_PART);
-        for (int c = 0; c < 2 * chunks; ++c) {
-          if (filled && !mbar_wait(&emptyA[st], ph ^ 1)) { s_fail = 1; break; }
-          mbar_expect_tx(&fullA[st], T::A_PART);
-          bulk_g2s(lbase + st * T::A_PART, img + (size_t)c * T::A_PART, T::A_PART, &fullA[st]);
+        for (int c = 0; c < chunks; ++c) {
+          const unsigned char* src = img + (size_t)c * (2 * T::A_PART);
+          const uint32_t dst = lbase + st * T::STAGE;
+          if (filled && !mbar_wait(&emptyR[st], ph ^ 1)) { s_fail = 1; break; }
+          mbar_expect_tx(&full[st], 2 * T::A_PART);
+          bulk_g2s(dst, src, T::A_PART, &full[st]);
+          if (filled && !mbar_wait(&emptyI[st], ph ^ 1)) s_fail = 1;   // (the copy completes the stage's count)
+          bulk_g2s(dst + T::A_PART, src + T::A_PART, T::A_PART, &full[st]);
           ++issued;
+          if (s_fail) break;
           const int cp = c + PF;
-          if (cp < 2 * chunks && cp % im.tiles_n == tn) prefetch_l2(img + (size_t)cp * T::A_PART, T::A_PART);
-          if (++st == NA) { st = 0; ph ^= 1; filled = true; }
+          if (cp < chunks && cp % im.tiles_n == tn) prefetch_l2(src + (size_t)PF * (2 * T::A_PART), 2 * T::A_PART);
+          if (++st == NSTG) { st = 0; ph ^= 1; filled = true; }
         }
       }
       if (s_fail) {   // a timeout: let the copies in flight land before the CTA ends
-        for (int m = max(0, issued - NA); m < issued; ++m) mbar_wait(&fullA[m % NA], (m / NA) & 1);
+        for (int m = max(0, issued - NSTG); m < issued; ++m) mbar_wait(&full[m % NSTG], (m / NSTG) & 1);
       }
     }
    } else if (warp == 13) {
@@ -487,32 +503,36 @@ __global__ void __launch_bounds__(NT, 1) ozb_product_kernel(GemmArgs g, ImgArgs 
     // between register files), and one elected lane issues
     const uint32_t el = elect_one();
     {
-      int sa = 0, sb = 0;
-      uint32_t pa = 0, pb = 0, passes = 0;
+      const uint32_t re = tmem, imc = tmem + T::COL_IM, spr = tmem + T::COL_SP, spi = spr + TNC;
+      int st = 0;
+      uint32_t ph = 0, passes = 0;
       for (long long i = blockIdx.x; i < ntiles && !s_fail; i += gridDim.x) {
         int u, tm, tn;
         if (!tile_at(i, u, tm, tn)) continue;
         for (int c0 = 0; c0 < chunks && !s_fail; c0 += PASS) {
-          if (passes > 0 && !mbar_wait(tfree, (passes - 1) & 1)) { s_fail = 1; break; }
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
           const int c1 = min(c0 + PASS, chunks);
           for (int c = c0; c < c1; ++c) {
-            if (!mbar_wait(&fullB[sb], pb) || !mbar_wait(&fullA[sa], pa)) { s_fail = 1; break; }
+            if (!mbar_wait(&full[st], ph)) { s_fail = 1; break; }
+            const uint32_t sa = lbase + st * T::STAGE;
+            const uint64_t ar = sdesc32(sa), ai = sdesc32(sa + T::A_PART), br = sdesc32(sa + T::OFF_B);
+            const uint64_t bi = br + ((ND * T::B_PL) >> 4), nbi = br + ((2 * ND * T::B_PL) >> 4);
+            const bool first = c == c0, last = c == c1 - 1;
+            // all of re, then all of im: the drain of one overlaps the MMAs of the other
+            if (first && passes > 0 && !mbar_wait(freeR, (passes - 1) & 1)) { s_fail = 1; break; }
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint64_t db = sdesc32(lbase + T::OFF_B + sb * T::B_CHUNK);
-            part_mmas<ND, TNC, 0>(tmem, sdesc32(lbase + sa * T::A_PART), db, c == c0, el);
-            mma_commit(&emptyA[sa], el);
-            if (++sa == NA) { sa = 0; pa ^= 1; }
-            if (!mbar_wait(&fullA[sa], pa)) { s_fail = 1; break; }
+            part_mmas<ND, TNC>(re, spr, ar, br, first, el);
+            part_mmas<ND, TNC>(re, spr, ai, nbi, false, el);
+            if (last) mma_commit(doneR, el);
+            if (first && passes > 0 && !mbar_wait(freeI, (passes - 1) & 1)) { s_fail = 1; break; }
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            part_mmas<ND, TNC, 1>(tmem, sdesc32(lbase + sa * T::A_PART), db, false, el);
-            mma_commit(&emptyA[sa], el);
-            mma_commit(&emptyB[sb], el);
-            if (++sa == NA) { sa = 0; pa ^= 1; }
-            if (++sb == NB) { sb = 0; pb ^= 1; }
+            part_mmas<ND, TNC>(imc, spi, ar, bi, first, el);
+            mma_commit(&emptyR[st], el);
+            part_mmas<ND, TNC>(imc, spi, ai, br, false, el);
+            mma_commit(&emptyI[st], el);
+            if (last) mma_commit(doneI, el);
+            if (++st == NSTG) { st = 0; ph ^= 1; }
           }
           if (s_fail) break;
-          mma_commit(done, el);
           ++passes;
         }
       }
@@ -523,7 +543,7 @@ __global__ void __launch_bounds__(NT, 1) ozb_product_kernel(GemmArgs g, ImgArgs 
     }
    }
   } else if (warp >= 8) {
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 88;");
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
     // ---------------- B digits: TPC threads per column, KPT consecutive complex k each; the
     // next chunk (of this tile or the next) is loaded while this one is cut
     constexpr int TPC = 128 / TNC, KPT = KC / TPC;
@@ -572,8 +592,8 @@ __global__ void __launch_bounds__(NT, 1) ozb_product_kernel(GemmArgs g, ImgArgs 
         yr[h] = biased_bytes<ND>(v[h].x, eb);
         yi[h] = biased_bytes<ND>(v[h].y, eb);
       }
-      if (filled && !mbar_wait(&emptyB[st], ph ^ 1)) { s_fail = 1; break; }
-      unsigned char* P = base + T::OFF_B + st * T::B_CHUNK + off;
+      if (filled && !mbar_wait(&emptyI[st], ph ^ 1)) { s_fail = 1; break; }
+      unsigned char* P = base + st * T::STAGE + T::OFF_B + off;
 #pragma unroll
       for (int q = 0; q < ND; ++q) {
         const unsigned int r0 = digit_pair<ND>(yr[0], yr[1], q), i0 = digit_pair<ND>(yi[0], yi[1], q);
@@ -592,11 +612,11 @@ __global__ void __launch_bounds__(NT, 1) ozb_product_kernel(GemmArgs g, ImgArgs 
       }
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       __syncwarp();
-      if (lane == 0) mbar_arrive(&fullB[st]);
-      if (++st == NB) { st = 0; ph ^= 1; filled = true; }
+      if (lane == 0) mbar_arrive(&full[st]);
+      if (++st == NSTG) { st = 0; ph ^= 1; filled = true; }
     }
   } else {
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 184;");
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 192;");
     // ---------------- drain and store: TMEM lanes 32 (warp % 4) .., TNC / 2 complex columns
     constexpr int CW = TNC / 2;                 // complex columns per thread
     const int quad = warp & 3, cb = (warp >> 2) * CW;
@@ -608,43 +628,54 @@ __global__ void __launch_bounds__(NT, 1) ozb_product_kernel(GemmArgs g, ImgArgs 
       int u, tm, tn;
       if (!tile_at(i, u, tm, tn)) continue;
       const int m0 = tm * TM + 32 * quad, n0 = tn * TNC + cb;
+      // the scales, long before they are used
+      const int er = (m0 + lane < n) ? im.ea[(size_t)u * n + m0 + lane] - (ND == 7 ? 56 : 48) + xs : 0;
+      int ebj[CW / 8];   // lane j holds column j's
+#pragma unroll
+      for (int h = 0; h < CW / 8; ++h) {
+        const int gcol = n0 + 8 * h + (lane & 7);
+        ebj[h] = gcol < n ? im.eb[(size_t)u * n + gcol] : 0;
+      }
       long long vr[CW], vi[CW];
       for (int c0 = 0; c0 < chunks; c0 += PASS) {
-        if (!__all_sync(0xffffffffu, mbar_wait(done, passes & 1))) { s_fail = 1; break; }
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        // steps of 4 complex columns and one part; the next step's loads fly while this
-        // step's groups are combined
-        uint32_t w[2][8][4];
-        auto fetch = [&](int it, uint32_t (&x)[8][4]) {
-          const int part = it & 1, cc = it >> 1;
+        bool ok = true;
 #pragma unroll
-          for (int d = 0; d < ND; ++d) TC_LD4(lane_base + (uint32_t)(part * T::COL_IM + d * TNC + cb + 4 * cc), x[d]);
-          if (ND == 7) TC_LD4(lane_base + (uint32_t)(T::COL_SP + part * TNC + cb + 4 * cc), x[7]);
-        };
-        fetch(0, w[0]);
+        for (int part = 0; part < 2; ++part) {
+          ok = __all_sync(0xffffffffu, mbar_wait(part ? doneI : doneR, passes & 1));
+          if (!ok) break;
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          // steps of 4 complex columns; the next step's loads fly while this step's groups are
+          // combined
+          uint32_t w[2][8][4];
+          auto fetch = [&](int cc, uint32_t (&x)[8][4]) {
 #pragma unroll
-        for (int it = 0; it < CW / 2; ++it) {
-          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-          if (it + 1 < CW / 2) fetch(it + 1, w[(it + 1) & 1]);
+            for (int d = 0; d < ND; ++d) TC_LD4(lane_base + (uint32_t)(part * T::COL_IM + d * TNC + cb + 4 * cc), x[d]);
+            if (ND == 7) TC_LD4(lane_base + (uint32_t)(T::COL_SP + part * TNC + cb + 4 * cc), x[7]);
+          };
+          fetch(0, w[0]);
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            long long v = combine<ND>(w[it & 1], j);
-            if (ND == 7 && xs > 0) v = (v + (1ll << (xs - 1))) >> xs;
-            long long& o = (it & 1) ? vi[4 * (it >> 1) + j] : vr[4 * (it >> 1) + j];
-            o = (c0 == 0) ? v : o + v;
+          for (int cc = 0; cc < CW / 4; ++cc) {
+            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+            if (cc + 1 < CW / 4) fetch(cc + 1, w[(cc + 1) & 1]);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              long long v = combine<ND>(w[cc & 1], j);
+              if (ND == 7 && xs > 0) v = (v + (1ll << (xs - 1))) >> xs;
+              long long& o = part ? vi[4 * cc + j] : vr[4 * cc + j];
+              o = (c0 == 0) ? v : o + v;
+            }
           }
+          asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+          __syncwarp();
+          if (lane == 0) mbar_arrive(part ? freeI : freeR);
         }
-        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-        __syncwarp();
-        if (lane == 0) mbar_arrive(tfree);
+        if (!ok) { s_fail = 1; break; }
         ++passes;
       }
       if (s_fail) break;
       // rows of this lane -> doubles -> shared memory, then 8 lanes per row: whole lines
       zc* D = g.D.at(u);
       const zc* Cm = (g.C.p && !(UAB && g.beta.x == 0.0)) ? g.C.at(u) : nullptr;
-      const int er = (m0 + lane < n) ? im.ea[(size_t)u * n + m0 + lane] - (ND == 7 ? 56 : 48) + xs : 0;
-      const int* eB = im.eb + (size_t)u * n;
       const int j = lane & 7, r4 = lane >> 3;
       const int neg_a = g.alpha.x < 0.0 ? (int)0x80000000 : 0, neg_b = g.beta.x < 0.0 ? (int)0x80000000 : 0;
 #pragma unroll
@@ -656,12 +687,10 @@ __global__ void __launch_bounds__(NT, 1) ozb_product_kernel(GemmArgs g, ImgArgs 
         for (int k = 0; k < 8; ++k) {
           const int row = m0 + 4 * k + r4;
           cv[k] = (Cm && row < n && gcol < n) ? Cm[(size_t)row * n + gcol] : zmake(0.0, 0.0);
-          if (UAB) cv[k] = zmake(flip(cv[k].x, neg_b), flip(cv[k].y, neg_b));
         }
-        const int ebj = gcol < n ? eB[gcol] : 0;   // lane j holds column j's scale
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
-          const int p = er + __shfl_sync(0xffffffffu, ebj, q);
+          const int p = er + __shfl_sync(0xffffffffu, ebj[h], q);
           const zc v = zmake(ldexp_int(vr[8 * h + q], p), ldexp_int(vi[8 * h + q], p));
           *reinterpret_cast<zc*>(stg + lane * 128 + ((q ^ (lane & 7)) << 4)) = v;
         }
@@ -673,7 +702,7 @@ __global__ void __launch_bounds__(NT, 1) ozb_product_kernel(GemmArgs g, ImgArgs 
           zc v;
           if (UAB) {
             v = zmake(flip(acc.x, neg_a), flip(acc.y, neg_a));
-            if (Cm) v = zadd(v, cv[k]);
+            if (Cm) v = zadd(v, zmake(flip(cv[k].x, neg_b), flip(cv[k].y, neg_b)));
           } else {
             v = zmul(g.alpha, acc);
             if (Cm) v = zadd(v, zmul(g.beta, cv[k]));
