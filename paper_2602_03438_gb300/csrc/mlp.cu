@@ -5,11 +5,11 @@
 //
 //   C[M][N] = A[M][K] * B[N][K]^T      (both operands K-contiguous, BF16)
 //
-// tiles of 128 x 128 per CTA, K in chunks of 64 (one 128-byte swizzle row), operand
-// tiles brought into shared memory by TMA (cp.async.bulk.tensor.2d with a 128-byte
-// swizzle) through a 4-stage mbarrier ring, one thread issuing tcgen05.mma
-// (kind::f16, BF16 x BF16 -> FP32) into a 128-column TMEM accumulator, and four
-// epilogue warps reading TMEM with tcgen05.ld and applying the layer's fused
+// tiles of 128 x 128 (or 128 x 32 where those leave most of the SMs idle) per CTA, K in
+// chunks of 64 (one 128-byte swizzle row), operand tiles brought into shared memory by TMA
+// (cp.async.bulk.tensor.2d with a 128-byte swizzle) through an mbarrier ring, one elected
+// thread issuing tcgen05.mma (kind::f16, BF16 x BF16 -> FP32) into a TMEM accumulator, and
+// four epilogue warps reading TMEM with tcgen05.ld and applying the layer's fused
 // epilogue (bias, relu, relu' mask, BF16 row-major and transposed copies).  Every
 // transposed operand the backward pass needs is produced either by the epilogue
 // that writes it or by a tiled transpose kernel, so that all products take the
@@ -21,6 +21,7 @@
 #include <algorithm>
 #include <mutex>
 #include <string>
+#include <type_traits>
 
 #include "negf_internal.cuh"
 #include "../../include/negf_warmstart.h"
@@ -32,16 +33,18 @@ namespace {
 typedef __nv_bfloat16 bf16;
 
 constexpr int BM = 128, BN = 128, BK = 64;
-constexpr int STAGES = 4;
+constexpr int BN_NARROW = 32;
 constexpr int GEMM_THREADS = 192;   // warp 0 TMA, warp 1 MMA, warps 2-5 epilogue
-constexpr uint32_t TILE_BYTES = BM * BK * 2;            // 16 KB per operand tile
-constexpr uint32_t STAGE_BYTES = 2 * TILE_BYTES;        // A and B
-constexpr uint32_t GEMM_SMEM = STAGES * STAGE_BYTES + 1024 + 256;
+constexpr uint32_t TILE_BYTES = BM * BK * 2;            // 16 KB of A per stage
+__host__ __device__ constexpr uint32_t stage_bytes(int bn) { return TILE_BYTES + bn * BK * 2; }
+__host__ __device__ constexpr int stages(int bn) { return bn == BN ? 6 : 8; }
+__host__ __device__ constexpr uint32_t gemm_smem(int bn) { return stages(bn) * stage_bytes(bn) + 1024 + 256; }
 constexpr unsigned long long kWaitNs = 1000000000ull;   // 1 s bound on every wait
 
-// instruction descriptor: kind::f16, D f32, A/B bf16, both K-major, M = 128, N = 128
-constexpr uint32_t IDESC_BF16 =
-    (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
+// instruction descriptor: kind::f16, D f32, A/B bf16, both K-major, M = 128, N = bn
+__host__ __device__ constexpr uint32_t idesc_bf16(int bn) {
+  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(bn >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
+}
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
@@ -101,16 +104,20 @@ __device__ __forceinline__ uint64_t sdesc(uint32_t saddr) {
   return d;
 }
 
-__device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t acc) {
+// by the lane whose `el` is set: the whole warp walks the loop, so that the descriptors stay
+// in uniform registers
+__device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t id, uint32_t acc, uint32_t el) {
   asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem_d),
-      "l"(a), "l"(b), "r"(IDESC_BF16), "r"(acc)
+      "{\n .reg .pred p, e;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 e, %5, 0;\n"
+      " @e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem_d),
+      "l"(a), "l"(b), "r"(id), "r"(acc), "r"(el)
       : "memory");
 }
 
-__device__ __forceinline__ void mma_commit(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
+__device__ __forceinline__ void mma_commit(uint64_t* bar, uint32_t el) {
+  asm volatile("{\n .reg .pred e;\n setp.ne.b32 e, %1, 0;\n"
+               " @e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(smem_u32(bar)),
+               "r"(el)
                : "memory");
 }
 
@@ -135,9 +142,12 @@ struct Epi {
   int relu;                     // act = relu (else identity)
 };
 
+template <int TN>
 __global__ void __launch_bounds__(GEMM_THREADS, 1)
     bf16_gemm_tn_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, int K,
                         Epi ep, int* err) {
+  constexpr int STAGES = stages(TN);
+  constexpr uint32_t STAGE_BYTES = stage_bytes(TN);
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* base = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint64_t* full = reinterpret_cast<uint64_t*>(base + STAGES * STAGE_BYTES);
@@ -146,7 +156,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
+  const int m0 = blockIdx.y * BM, n0 = blockIdx.x * TN;
   const int nk = K / BK;
 
   if (threadIdx.x == 0) {
@@ -161,7 +171,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
   }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
-                 "r"(BN)
+                 "r"(TN)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
@@ -185,25 +195,26 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {   // MMA issuer
-      bool ok = true;
-      for (int kb = 0; kb < nk; ++kb) {
-        const int s = kb % STAGES;
-        if (!mbar_wait(&full[s], (uint32_t)((kb / STAGES) & 1))) {
-          raise_error(err, NEGF_ERR_TIMEOUT);
-          ok = false;
-          break;
-        }
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t sa = smem_u32(base + s * STAGE_BYTES);
-        const uint64_t da = sdesc(sa), db = sdesc(sa + TILE_BYTES);
-#pragma unroll
-        for (int k = 0; k < BK / 16; ++k)   // 16 BF16 = 32 bytes per MMA: +2 in descriptor units
-          mma_bf16(tmem, da + 2 * k, db + 2 * k, (kb | k) != 0);
-        mma_commit(&empty[s]);
+    // MMA issue
+    uint32_t el;
+    asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(el));
+    bool ok = true;
+    for (int kb = 0; kb < nk; ++kb) {
+      const int s = kb % STAGES;
+      if (!__all_sync(0xffffffffu, mbar_wait(&full[s], (uint32_t)((kb / STAGES) & 1)))) {
+        if (lane == 0) raise_error(err, NEGF_ERR_TIMEOUT);
+        ok = false;
+        break;
       }
-      if (ok) mma_commit(done);
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const uint32_t sa = smem_u32(base + s * STAGE_BYTES);
+      const uint64_t da = sdesc(sa), db = sdesc(sa + TILE_BYTES);
+#pragma unroll
+      for (int k = 0; k < BK / 16; ++k)   // 16 BF16 = 32 bytes per MMA: +2 in descriptor units
+        mma_bf16(tmem, da + 2 * k, db + 2 * k, idesc_bf16(TN), (kb | k) != 0, el);
+      mma_commit(&empty[s], el);
     }
+    if (ok) mma_commit(done, el);
   } else {   // epilogue warps 2..5: TMEM lanes 32 (warp % 4) .. +31
     const int q = warp & 3;
     bool ok = mbar_wait(done, 0);
@@ -212,7 +223,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
     const int row = m0 + 32 * q + lane;
     if (__all_sync(0xffffffffu, ok)) {
 #pragma unroll 1
-      for (int cc = 0; cc < BN / 32; ++cc) {
+      for (int cc = 0; cc < TN / 32; ++cc) {
         uint32_t r[32];
         MLP_LD32(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(cc * 32), r);
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
@@ -257,7 +268,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   if (warp == 1)
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(BN) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TN) : "memory");
 }
 
 // ---------------------------------------------------------------------------
@@ -373,20 +384,24 @@ __global__ void loss_kernel(const float* Y, const zc* G, const int32_t* rows, in
                             double scale, float* dY32, bf16* dYb, double* partial) {
   const int bb = nout / 2;
   double acc = 0.0;
-  const long long total = (long long)np_ * nout;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
-       i += (long long)gridDim.x * blockDim.x) {
-    const int r = (int)(i / nout), c = (int)(i - (long long)r * nout);
-    double d = 0.0;
+  // a block per half row (with a block per row the last rows left half the SMs idle)
+  for (long long hr = blockIdx.x; hr < 2LL * np_; hr += gridDim.x) {
+    const int r = (int)(hr >> 1), c1 = (hr & 1) ? nout : bb;
     const int src = rows ? (r < n ? rows[r] : -1) : r;
-    if (r < n && src >= 0 && src < n_set) {
-      const double t = c < bb ? G[(size_t)src * bb + c].x : G[(size_t)src * bb + c - bb].y;
-      const double res = (double)Y[i] - t;
-      acc += res * res;
-      d = res * scale;
+    const bool in = r < n && src >= 0 && src < n_set;
+    const double* g = reinterpret_cast<const double*>(G + (in ? (size_t)src * bb : 0));
+    const size_t o = (size_t)r * nout;
+#pragma unroll 4
+    for (int c = c1 - bb + threadIdx.x; c < c1; c += blockDim.x) {
+      float d = 0.0f;
+      if (in) {
+        const double res = (double)Y[o + c] - (c < bb ? g[2 * c] : g[2 * (c - bb) + 1]);
+        acc += res * res;
+        d = (float)(res * scale);
+      }
+      dY32[o + c] = d;
+      dYb[o + c] = __float2bfloat16_rn(d);
     }
-    dY32[i] = (float)d;
-    dYb[i] = __float2bfloat16_rn((float)d);
   }
   __shared__ double red[32];
   for (int off = 16; off > 0; off >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, off);
@@ -399,38 +414,59 @@ __global__ void loss_kernel(const float* Y, const zc* G, const int32_t* rows, in
   }
 }
 
-// loss = (sum of the partials, fixed order) / count
+// loss = (sum of the partials, fixed order) / count: one warp, each lane every 32nd partial (a
+// chain of 512 dependent FP64 additions took 30 us; the lanes' chains and the tree 2)
 __global__ void loss_final_kernel(const double* partial, int np, double inv_count, double* loss) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    double t = 0.0;
-    for (int i = 0; i < np; ++i) t += partial[i];
-    *loss = t * inv_count;
+  double t = 0.0;
+  for (int i = threadIdx.x; i < np; i += 32) t += partial[i];
+  for (int off = 16; off > 0; off >>= 1) t += __shfl_down_sync(0xffffffffu, t, off);
+  if (threadIdx.x == 0) *loss = t * inv_count;
+}
+
+// out[c] = sum over rows r < n of A[r][c] (FP64 accumulation, fixed order): 32 columns per CTA,
+// every 16th row per warp, then the 16 partial sums in order.  One thread per column was a
+// chain of n FP64 additions: 43 us for n = 256 whatever N; 8 us so.
+constexpr int CS_WARPS = 16;
+__global__ void __launch_bounds__(32 * CS_WARPS) colsum_kernel(const float* A, int lda, int n, int N, float* out) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, c = blockIdx.x * 32 + lane;
+  __shared__ double part[CS_WARPS][32];
+  double t = 0.0;
+  if (c < N)
+    for (int r = w; r < n; r += CS_WARPS) t += (double)A[(size_t)r * lda + c];
+  part[w][lane] = t;
+  __syncthreads();
+  if (w == 0 && c < N) {
+    for (int q = 1; q < CS_WARPS; ++q) t += part[q][lane];
+    out[c] = (float)t;
   }
 }
 
-// out[c] = sum over rows r < n of A[r][c]  (FP64 accumulation, fixed order)
-__global__ void colsum_kernel(const float* A, int lda, int n, int N, float* out) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= N) return;
-  double t = 0.0;
-  for (int r = 0; r < n; ++r) t += (double)A[(size_t)r * lda + c];
-  out[c] = (float)t;
-}
-
+// V: parameters per load (4 where the vectors are 16-byte aligned)
+template <int V>
 __global__ void adam_kernel(float* theta, float* m, float* v, const float* g, long long count, float lr, float b1,
                             float b2, float eps, float c1, float c2) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < count;
-       i += (long long)gridDim.x * blockDim.x) {
-    const float gi = g[i];
-    const float mi = b1 * m[i] + (1.0f - b1) * gi;
-    const float vi = b2 * v[i] + (1.0f - b2) * gi * gi;
-    m[i] = mi;
-    v[i] = vi;
-    theta[i] -= lr * (mi * c1) / (sqrtf(vi * c2) + eps);
+  typedef typename std::conditional<V == 4, float4, float>::type T;
+  for (long long i = V * (blockIdx.x * (long long)blockDim.x + threadIdx.x); i < count;
+       i += V * (long long)gridDim.x * blockDim.x) {
+    T tg = *reinterpret_cast<const T*>(g + i), tm = *reinterpret_cast<T*>(m + i), tv = *reinterpret_cast<T*>(v + i),
+      tt = *reinterpret_cast<T*>(theta + i);
+    float *pg = reinterpret_cast<float*>(&tg), *pm = reinterpret_cast<float*>(&tm), *pv = reinterpret_cast<float*>(&tv),
+          *pt = reinterpret_cast<float*>(&tt);
+#pragma unroll
+    for (int q = 0; q < V; ++q) {
+      const float gi = pg[q];
+      const float mi = b1 * pm[q] + (1.0f - b1) * gi;
+      const float vi = b2 * pv[q] + (1.0f - b2) * gi * gi;
+      pm[q] = mi;
+      pv[q] = vi;
+      pt[q] -= lr * (mi * c1) / (sqrtf(vi * c2) + eps);
+    }
+    *reinterpret_cast<T*>(m + i) = tm;
+    *reinterpret_cast<T*>(v + i) = tv;
+    *reinterpret_cast<T*>(theta + i) = tt;
   }
 }
 
-// g0[s] = Y[s][0:bb] + i Y[s][bb:2bb]
 __global__ void unpack_kernel(const float* Y, int n, int bb, zc* g0) {
   const long long total = (long long)n * bb;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
@@ -480,15 +516,16 @@ struct Fail {
 #define MLAUNCH() do { ++ctx->launches; MCU(cudaGetLastError()); } while (0)
 
 // a BF16 row-major matrix [rows][cols] with leading dimension ld (elements), tiles
-// of 128 rows x 64 columns, 128-byte swizzle
-negf_status make_map(const Fail& F, CUtensorMap* m, const void* ptr, long long rows, long long cols, long long ld) {
+// of box_rows rows x 64 columns, 128-byte swizzle
+negf_status make_map(const Fail& F, CUtensorMap* m, const void* ptr, long long rows, long long cols, long long ld,
+                     int box_rows) {
   EncodeTiledFn enc = encode_fn();
   if (!enc) return F(NEGF_ERR_CUDA, "cuTensorMapEncodeTiled is not available from the driver");
-  if (((uintptr_t)ptr & 15) || (ld * 2) % 16 || rows % BM || cols % BK)
+  if (((uintptr_t)ptr & 15) || (ld * 2) % 16 || rows % box_rows || cols % BK)
     return F(NEGF_ERR_ARG, "tensor map operand not 16-byte aligned or not tile-shaped");
   const cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
   const cuuint64_t strides[1] = {(cuuint64_t)(ld * 2)};
-  const cuuint32_t box[2] = {(cuuint32_t)BK, (cuuint32_t)BM};
+  const cuuint32_t box[2] = {(cuuint32_t)BK, (cuuint32_t)box_rows};
   const cuuint32_t es[2] = {1, 1};
   CUresult r = enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(ptr), dims, strides, box, es,
                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -503,14 +540,25 @@ negf_status gemm(Ctx* ctx, cudaStream_t s, const bf16* A, long long lda, const b
   const Fail F{ctx};
   if (M % BM || N % BN || K % BK || K <= 0) return F(NEGF_ERR_ARG, "GEMM shape not a multiple of the tiles");
   MCU(once_per_device(INIT_MLP, [](int) {
-    return cudaFuncSetAttribute(bf16_gemm_tn_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GEMM_SMEM);
+    cudaError_t e = cudaFuncSetAttribute(bf16_gemm_tn_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)gemm_smem(BN));
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(bf16_gemm_tn_kernel<BN_NARROW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)gemm_smem(BN_NARROW));
   }));
+  // Narrow tiles where the wide ones would leave most SMs idle: a CTA's time is its K chunks,
+  // and those are bound by what one SM reads (16 KB of A and the B tile per chunk).  n =
+  // 256, hidden 512, K = 12416 (8 wide tiles): 65 -> 39 us; with 64 wide tiles and more
+  // the A tile read four times as often costs more than it gains.
+  const bool narrow = (long long)(N / BN) * (M / BM) <= 32;
+  const int tn = narrow ? BN_NARROW : BN;
   CUtensorMap ma, mb;
   negf_status st;
-  if ((st = make_map(F, &ma, A, M, K, lda)) != NEGF_OK) return st;
-  if ((st = make_map(F, &mb, B, N, K, ldb)) != NEGF_OK) return st;
-  dim3 grid(N / BN, M / BM);
-  bf16_gemm_tn_kernel<<<grid, GEMM_THREADS, GEMM_SMEM, s>>>(ma, mb, K, ep, ctx->d_err);
+  if ((st = make_map(F, &ma, A, M, K, lda, BM)) != NEGF_OK) return st;
+  if ((st = make_map(F, &mb, B, N, K, ldb, tn)) != NEGF_OK) return st;
+  const dim3 grid(N / tn, M / BM);
+  if (narrow) bf16_gemm_tn_kernel<BN_NARROW><<<grid, GEMM_THREADS, gemm_smem(BN_NARROW), s>>>(ma, mb, K, ep, ctx->d_err);
+  else bf16_gemm_tn_kernel<BN><<<grid, GEMM_THREADS, gemm_smem(BN), s>>>(ma, mb, K, ep, ctx->d_err);
   MLAUNCH();
   return NEGF_OK;
 }
@@ -746,7 +794,7 @@ negf_status negf_mlp_train_step(negf_ctx* c, const negf_mlp_dims* dims, float* p
   Epi e = epi0();
   e.c32 = grad + dims->off_W3; e.ldc32 = (int)H;
   if ((st = gemm(ctx, s, B.dYT, np_, B.H2T, np_, (int)NO, (int)H, (int)np_, e)) != NEGF_OK) return st;
-  colsum_kernel<<<(unsigned)((NO + 255) / 256), 256, 0, s>>>(B.dY32, (int)NO, n, (int)NO, grad + dims->off_c3);
+  colsum_kernel<<<(unsigned)((NO + 31) / 32), 32 * CS_WARPS, 0, s>>>(B.dY32, (int)NO, n, (int)NO, grad + dims->off_c3);
   MLAUNCH();
   e = epi0();
   e.c32 = B.dZ2; e.ldc32 = (int)H;
@@ -759,7 +807,7 @@ negf_status negf_mlp_train_step(negf_ctx* c, const negf_mlp_dims* dims, float* p
   e = epi0();
   e.c32 = grad + dims->off_W2; e.ldc32 = (int)H;
   if ((st = gemm(ctx, s, B.dZ2T, np_, B.H1T, np_, (int)H, (int)H, (int)np_, e)) != NEGF_OK) return st;
-  colsum_kernel<<<(unsigned)((H + 255) / 256), 256, 0, s>>>(B.dZ2, (int)H, n, (int)H, grad + dims->off_c2);
+  colsum_kernel<<<(unsigned)((H + 31) / 32), 32 * CS_WARPS, 0, s>>>(B.dZ2, (int)H, n, (int)H, grad + dims->off_c2);
   MLAUNCH();
   e = epi0();
   e.c32 = B.dZ1; e.ldc32 = (int)H;
@@ -771,7 +819,7 @@ negf_status negf_mlp_train_step(negf_ctx* c, const negf_mlp_dims* dims, float* p
   e = epi0();
   e.c32 = grad + dims->off_W1; e.ldc32 = (int)K0;
   if ((st = gemm(ctx, s, B.dZ1T, np_, B.XT, np_, (int)H, (int)K0, (int)np_, e)) != NEGF_OK) return st;
-  colsum_kernel<<<(unsigned)((H + 255) / 256), 256, 0, s>>>(B.dZ1, (int)H, n, (int)H, grad + dims->off_c1);
+  colsum_kernel<<<(unsigned)((H + 31) / 32), 32 * CS_WARPS, 0, s>>>(B.dZ1, (int)H, n, (int)H, grad + dims->off_c1);
   MLAUNCH();
 
   // ---- Adam
@@ -779,8 +827,13 @@ negf_status negf_mlp_train_step(negf_ctx* c, const negf_mlp_dims* dims, float* p
     const double b1 = 0.9, b2 = 0.999;
     const float c1 = (float)(1.0 / (1.0 - pow(b1, (double)step)));
     const float c2 = (float)(1.0 / (1.0 - pow(b2, (double)step)));
-    adam_kernel<<<grid_for(dims->n_params, 256), 256, 0, s>>>(params, adam_m, adam_v, grad, dims->n_params, lr,
-                                                              (float)b1, (float)b2, 1e-8f, c1, c2);
+    auto aligned = [](const void* p) { return ((uintptr_t)p & 15) == 0; };
+    if (dims->n_params % 4 == 0 && aligned(params) && aligned(adam_m) && aligned(adam_v) && aligned(grad))
+      adam_kernel<4><<<grid_for(dims->n_params / 4, 256), 256, 0, s>>>(params, adam_m, adam_v, grad, dims->n_params, lr,
+                                                                       (float)b1, (float)b2, 1e-8f, c1, c2);
+    else
+      adam_kernel<1><<<grid_for(dims->n_params, 256), 256, 0, s>>>(params, adam_m, adam_v, grad, dims->n_params, lr,
+                                                                   (float)b1, (float)b2, 1e-8f, c1, c2);
     MLAUNCH();
   }
   return NEGF_OK;
