@@ -517,15 +517,24 @@ struct Engine {
     end(masked ? 0.0 : flops, masked ? 0.0 : bytes);
     return e;
   }
-  cudaError_t inv(BMat X, BMat M, int n, int units, const int* active, int single, int32_t* status) {
+  // l1, l2: two adjacent blocks per unit that are free meanwhile (nullable), lent to the FP64
+  // inverse as scratch
+  cudaError_t inv(BMat X, BMat M, int n, int units, const int* active, int single, int32_t* status, BMat l1 = BMat{nullptr, 0},
+                  BMat l2 = BMat{nullptr, 0}) {
     const bool masked = active != nullptr && active_frac < 0.0;   // an unknown share of the work
     const double frac = (active && active_frac >= 0.0) ? active_frac : 1.0;
     begin(masked ? K_OTHER : (single ? K_INV_F32 : K_INV_F64));
-    // the FP32 inverse may use the sliced products' scratch, whose images are then gone
-    void* lent = (single && mixed == 1 && oz_supported(n)) ? ozt_scratch : nullptr;
+    // the FP32 inverse of large blocks may use the sliced products' scratch, whose images are
+    // then gone
+    void* lent = (single && n > 128 && mixed == 1 && oz_supported(n)) ? ozt_scratch : nullptr;
+    size_t lent_bytes = lent ? ozt_scratch_bytes(n, units) : 0;
     if (lent) last_a = AKey();
-    cudaError_t e = zinv(X, M, n, units, active, single, inv_scratch, status, s, lent,
-                         lent ? ozt_scratch_bytes(n, units) : 0);
+    const long long nn = (long long)n * n;
+    if (!single && l1.p && l1.plain() && l1.us == nn && l2.p == l1.p + nn * units) {
+      lent = l1.p;
+      lent_bytes = 2 * sizeof(zc) * (size_t)nn * units;
+    }
+    cudaError_t e = zinv(X, M, n, units, active, single, inv_scratch, status, s, lent, lent_bytes);
     end(masked ? 0.0 : 8.0 * (double)n * n * n * units * frac, masked ? 0.0 : 32.0 * (double)n * n * units * frac);
     return e;
   }
@@ -537,7 +546,7 @@ struct Engine {
   cudaError_t inverse(BMat X, BMat M, int n, int units, int32_t* status, BMat T1, BMat T2, int refine = -1,
                       const int* active = nullptr) {
     if (refine < 0) refine = (mixed == 1) ? 2 : 1;
-    cudaError_t e = inv(X, M, n, units, active, mixed ? 1 : 0, status);
+    cudaError_t e = inv(X, M, n, units, active, mixed ? 1 : 0, status, T1, T2);
     if (e != cudaSuccess || !mixed) return e;
     return refine_steps(X, M, n, units, T1, T2, refine, active);
   }
@@ -2612,7 +2621,7 @@ negf_status negf_obc(negf_ctx* c, const negf_system* sys, negf_precision prec, d
       // FP64 precision: FP64 Gauss-Jordan
       auto lead_inverse = [&](BMat X, BMat M, const int* mask) -> negf_status {
         if (!sl) {
-          CU(eng.inv(X, M, b, NU, mask, 0, nullptr));
+          CU(eng.inv(X, M, b, NU, mask, 0, nullptr, T[0], T[1]));
           return NEGF_OK;
         }
         CU(eng.inverse(X, M, b, NU, nullptr, T[0], T[1], 2, mask));
@@ -2674,7 +2683,7 @@ negf_status negf_obc(negf_ctx* c, const negf_system* sys, negf_precision prec, d
       // cnt = the number of units in `mask`.
       auto newton_step = [&](int* mask, BMat gn, int cnt) -> negf_status {
         negf_status sc;
-        CU(eng.inv(T[3], T[1], b, NU, mask, 0, nullptr));                 // K^{-1}
+        CU(eng.inv(T[3], T[1], b, NU, mask, 0, nullptr, T[4], T[5]));     // K^{-1}
         if ((sc = compact(mask, cnt)) != NEGF_OK) return sc;
         CU(lgemm(T[4], T[3], OP_N, al0, OP_N, ONE, NOMAT, ZERO, mask));          // P = K^{-1} al
         CU(lgemm(T[5], be0, OP_N, g, OP_N, ONE, NOMAT, ZERO, mask));             // Q = be g
@@ -3138,8 +3147,11 @@ negf_status negf_block_inverse(negf_ctx* c, negf_precision prec, int32_t n, int3
   if (need > ctx->ws_bytes) return fail(ctx, NEGF_ERR_NOMEM, "workspace too small for this batch of inverses");
   zc* ws = (zc*)ctx->ws;
   Engine eng{ctx, s, mixed, nullptr};
-  BMat T1{ws, bb}, T2{ws + (mixed ? units * bb : 0), bb};
-  eng.inv_scratch = (void*)(ws + (mixed ? 2 * units * bb : 0));
+  // (FP64 needs no slots; where the workspace has room for them they are lent to the inverse)
+  const bool lend = !mixed && need + 2 * sizeof(zc) * (size_t)units * bb <= ctx->ws_bytes;
+  const bool slots = mixed || lend;
+  BMat T1{ws, bb}, T2{ws + (slots ? units * bb : 0), bb};
+  eng.inv_scratch = (void*)(ws + (slots ? 2 * units * bb : 0));
   eng.oz_scratch = (char*)eng.inv_scratch + inv_b;
   {
     char* q = (char*)(((uintptr_t)eng.oz_scratch + 1023) & ~(uintptr_t)1023);

@@ -20,7 +20,7 @@ namespace negf {
 // is not recorded, so the next call retries it.
 // ---------------------------------------------------------------------------
 enum InitSlot { INIT_OZ = 0, INIT_TC, INIT_MLP, INIT_SMALL, INIT_OBC_SMALL, INIT_OZB, INIT_OZB_LO, INIT_OZB16,
-                INIT_OZB16_LO,
+                INIT_OZB16_LO, INIT_INV32, INIT_INV64, INIT_INV96, INIT_INV128,
                 INIT_NSLOT };
 constexpr int kMaxDevices = 64;
 cudaError_t once_per_device(int slot, const std::function<cudaError_t(int device)>& init);
@@ -161,16 +161,17 @@ cudaError_t zgemm_ozt_variant(const GemmArgs& g, void* scratch, int* err, cudaSt
 // Work storage: in shared memory when it fits, otherwise `scratch` (units * n*n
 // complex of the working precision).  status[u] (nullable, indexed status_base+u)
 // gets NEGF_ERR_SINGULAR on an exactly zero pivot.
-// `lent` (lent_bytes, nullable): scratch the caller does not need meanwhile, which the FP32
-// inverse may use beside its own.
+// `lent` (lent_bytes, nullable): 16-byte aligned scratch the caller does not need meanwhile.
 cudaError_t zinv(BMat X, BMat M, int n, int units, const int* active, int single, void* scratch,
                  int32_t* status, cudaStream_t s, void* lent = nullptr, size_t lent_bytes = 0);
 size_t zinv_scratch_bytes(int n, int units, int single);
-// the FP32 inverse as column tiles, several CTAs per block (inv_tiles.cu; n <= 512);
-// `scratch` holds zinv_tiles_bytes(n, units) bytes, 16-byte aligned
-cudaError_t zinv_tiles(BMat X, BMat M, int n, int units, const int* active, void* scratch, int32_t* status,
+// the inverse as column tiles, several CTAs per block (inv_tiles.cu; n <= 512); `scratch`
+// holds zinv_tiles_bytes(n, units, single) bytes, 16-byte aligned
+cudaError_t zinv_tiles(BMat X, BMat M, int n, int units, const int* active, int single, void* scratch, int32_t* status,
                        cudaStream_t s);
-size_t zinv_tiles_bytes(int n, int units);
+size_t zinv_tiles_bytes(int n, int units, int single);
+// FP32, n <= 128: one CTA per block, the matrix in registers, no scratch
+cudaError_t zinv_reg(BMat X, BMat M, int n, int units, const int* active, int32_t* status, cudaStream_t s);
 
 // block i of unit u at p + u us + i is (a device's diagonal or off-diagonal output
 // blocks, or a workspace slot array [i][u])

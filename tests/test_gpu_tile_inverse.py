@@ -1,5 +1,6 @@
-"""The FP32 inverse as column tiles (several CTAs per block), through negf_block_inverse with
-NEGF_MIXED, at the edges of its tiles and thread counts.
+"""The block inverses through negf_block_inverse, at the edges of their tiles and thread counts:
+FP32 with the matrix in registers (n <= 128) or as column tiles over several CTAs, refined
+(NEGF_MIXED), and FP64 as column tiles.
 
 Tolerance: X is FP64-class after the refinement, so I - M X is of the order of the FP64
 product's own error, n 2^-53 |M| |X| per row; 8 n 2^-53 ||M||_F ||X||_F bounds it.
@@ -47,6 +48,33 @@ def test_tile_inverse(P, n, units):
     for u in range(units):
         bound = 8 * n * 2.0 ** -53 * float(M[u].norm()) * float(X[u].norm())
         assert float((eye - M[u] @ X[u]).norm()) <= bound
+
+
+@pytest.mark.parametrize("n,units", [(32, 400), (48, 3), (64, 1), (65, 2), (96, 200), (97, 5), (128, 160)])
+def test_register_inverse_of_many_blocks(P, n, units):
+    test_tile_inverse(P, n, units)
+
+
+@pytest.mark.parametrize("n,units", [(63, 2), (64, 2), (65, 76), (71, 3), (72, 77), (111, 1), (112, 2), (113, 90), (128, 3),
+                                     (200, 2), (257, 1)])
+def test_fp64_inverse(P, n, units):
+    """FP64 Gauss-Jordan: an error of the order of n 2^-53 |M| |X| as well, with pivots that keep
+    the growth of these matrices (a permutation of weight 2 plus noise) near one."""
+    M = _matrix(n, units, 7 * n + units)
+    X = torch.empty_like(M)
+    status = torch.full((units,), 7, dtype=torch.int32, device="cuda")
+    for ws in (1 << 28, 1 << 20):      # with room for the tiles' scratch, and (small n) without
+        ctx = P.Context(0, ws + 16 * n * (n + 1) * units)
+        try:
+            P.negf.negf_block_inverse(ctx, P.FP64, M, X, status)
+            assert ctx.sync() == 0
+        finally:
+            ctx.close()
+        assert int(status.abs().sum()) == 0
+        eye = torch.eye(n, dtype=torch.complex128, device="cuda")
+        for u in range(units):
+            bound = 8 * n * 2.0 ** -53 * float(M[u].norm()) * float(X[u].norm())
+            assert float((eye - M[u] @ X[u]).norm()) <= bound
 
 
 @pytest.mark.parametrize("n,col", [(16, 15), (40, 17), (129, 0), (129, 128), (256, 130), (512, 300)])
