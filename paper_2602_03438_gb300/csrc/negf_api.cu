@@ -1264,9 +1264,49 @@ __global__ void lead_init_kernel(LeadArgs a) {
   }
 }
 
+// The lead solver's bookkeeping reads whole blocks to take one decision per unit.  One SM holds
+// a unit, and the FP64 pipe (64 clocks per warp instruction) is slower there than the memory:
+// so the decisions come from the high words of the entries, and the moduli are formed only
+// where those bounds leave the answer open.  130 active units of b = 128, us before and after:
+// lead_norm 68 -> 17, smith_accum 81 -> 18, balance 105 -> 12 (26 where it scales),
+// refine_check 41 -> 14.
+constexpr unsigned int kBig = 0x5F137489u, kTiny = 0x27074490u;   // high words of about 1e150 and 1e-120
+__device__ __forceinline__ unsigned int abs_key(zc v) {   // the larger component's high word; NaN and infinity on top
+  return max((unsigned int)__double2hiint(v.x) & 0x7fffffffu, (unsigned int)__double2hiint(v.y) & 0x7fffffffu);
+}
+__device__ __forceinline__ double key_lo(unsigned int k) { return __hiloint2double((int)k, 0); }
+__device__ __forceinline__ double key_hi(unsigned int k) { return __hiloint2double((int)k, -1); }
+// the CTA's largest value, to all threads (red: 32 words that the caller has not read since a barrier)
+__device__ __forceinline__ unsigned int cta_max(unsigned int k, unsigned int* red) {
+  k = __reduce_max_sync(0xffffffffu, k);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = k;
+  __syncthreads();
+  const int lane = threadIdx.x & 31;
+  return __reduce_max_sync(0xffffffffu, lane < (int)((blockDim.x + 31) >> 5) ? red[lane] : 0u);
+}
+// the CTA's largest |.|^2 (NaN ignored) of one block, to all threads
+__device__ __noinline__ double cta_max_abs2(const zc* x, long long nn, double* red) {
+  double m = 0.0;
+#pragma unroll 4
+  for (long long i = threadIdx.x; i < nn; i += blockDim.x) m = fmax(m, zabs2(x[i]));
+  for (int off = 16; off > 0; off >>= 1) m = fmax(m, __shfl_down_sync(0xffffffffu, m, off));
+  __syncthreads();   // (red may still be read)
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+  __syncthreads();
+  m = red[0];
+  for (int w = 1; w < (int)(blockDim.x >> 5); ++w) m = fmax(m, red[w]);
+  return m;
+}
+constexpr int kBookUnroll = 4;   // entries of each block in flight per thread
+int book_threads(int n) {        // a CTA per unit, kBookUnroll entries per thread and round
+  const long long t = ((long long)n * n + kBookUnroll - 1) / kBookUnroll;
+  return (int)std::min<long long>(1024, (t + 31) / 32 * 32);
+}
+
 // per unit: m = max(max|al|, max|be|).  mode 0: ref[u] = m.  mode 1: convergence check.
-__global__ void lead_norm_kernel(BMat al, BMat be, int n, int mode, double* ref, int* done, int* live, int* iters,
-                                 int it, double tol, int* n_active, const int* skip = nullptr) {
+__global__ void __launch_bounds__(1024) lead_norm_kernel(BMat al, BMat be, int n, int mode, double* ref, int* done,
+                                                         int* live, int* iters, int it, double tol, int* n_active,
+                                                         const int* skip = nullptr) {
   const int u = blockIdx.x;
   if (mode == 1 && done[u]) return;
   if (mode == 0 && skip && skip[u]) {   // solved by the warm start: no decimation
@@ -1281,33 +1321,42 @@ __global__ void lead_norm_kernel(BMat al, BMat be, int n, int mode, double* ref,
   const long long nn = (long long)n * n;
   const zc* x = al.at(u);
   const zc* y = be.at(u);
-  // the largest |entry|, from the squared moduli (two FP64 operations per entry; one
-  // square root per block)
-  double m = 0.0;
-  for (long long i = threadIdx.x; i < nn; i += blockDim.x) {
-    m = fmax(m, zabs2(x[i]));
-    m = fmax(m, zabs2(y[i]));
-  }
   __shared__ double red[32];
-  for (int off = 16; off > 0; off >>= 1) m = fmax(m, __shfl_down_sync(0xffffffffu, m, off));
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
-  __syncthreads();
+  __shared__ unsigned int redk[32];
+  bool decided = false, small = false;
+  if (mode == 1) {
+    unsigned int k = 0;
+    for (long long i0 = threadIdx.x; i0 < nn; i0 += kBookUnroll * blockDim.x) {
+#pragma unroll
+      for (int q = 0; q < kBookUnroll; ++q) {
+        const long long i = i0 + q * blockDim.x;
+        if (i < nn) k = max(k, max(abs_key(x[i]), abs_key(y[i])));
+      }
+    }
+    k = cta_max(k, redk);
+    // m lies between the largest component and sqrt(2) times it
+    const double thr = tol * ref[u];
+    small = k < kBig && 1.5 * key_hi(k) < thr;
+    decided = small || (k > kTiny && k < kBig && 0.999 * key_lo(k) >= thr);
+  }
+  double m = 0.0;
+  if (!decided) {
+    m = cta_max_abs2(x, nn, red);
+    m = sqrt(fmax(m, cta_max_abs2(y, nn, red)));
+    if (mode == 1) small = m < tol * ref[u] || !isfinite(m);
+  }
   if (threadIdx.x == 0) {
-    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) m = fmax(m, red[w]);
-    m = sqrt(m);
     if (mode == 0) {
       ref[u] = fmax(m, 1e-300);
       done[u] = 0;
       live[u] = 1;
       iters[u] = 0;
-    } else {
-      if (m < tol * ref[u] || !isfinite(m)) {
-        done[u] = isfinite(m) ? 1 : 2;
-        live[u] = 0;
-        iters[u] = it;
-      } else if (n_active) {
-        atomicAdd(n_active, 1);
-      }
+    } else if (small) {
+      done[u] = isfinite(m) ? 1 : 2;
+      live[u] = 0;
+      iters[u] = it;
+    } else if (n_active) {
+      atomicAdd(n_active, 1);
     }
   }
 }
@@ -1351,7 +1400,7 @@ __global__ void residual_kernel(BMat F, int n, double* res, const int* active) {
 // redo[u] = 1 for an active unit whose refined inverse is not FP64-class: the residual
 // R = I - M X left by the last refinement step (the step from X to X + X R leaves an
 // error of the order of |R|^2) has a Frobenius norm above tol, or is not finite
-__global__ void refine_check_kernel(BMat R, int n, const int* active, double tol, int* redo) {
+__global__ void __launch_bounds__(1024) refine_check_kernel(BMat R, int n, const int* active, double tol, int* redo) {
   const int u = blockIdx.x;
   if (active && !active[u]) {
     if (threadIdx.x == 0) redo[u] = 0;
@@ -1359,9 +1408,37 @@ __global__ void refine_check_kernel(BMat R, int n, const int* active, double tol
   }
   const zc* r = R.at(u);
   const int nn = n * n;
+  __shared__ double red[32];
+  __shared__ float redf[32];
+  // in FP32 first, from the entries' high words (within 1e-5; tol^2 is far inside the range)
+  auto high = [](double v) {
+    const unsigned int a = (unsigned int)__double2hiint(v) & 0x7fffffffu;
+    return a < (897u << 20) ? 0.f : a >= (1150u << 20) ? INFINITY : __uint_as_float((a - (896u << 20)) << 3);
+  };
+  float f = 0.f;
+  for (int i0 = threadIdx.x; i0 < nn; i0 += kBookUnroll * blockDim.x) {
+#pragma unroll
+    for (int q = 0; q < kBookUnroll; ++q) {
+      const int i = i0 + q * (int)blockDim.x;
+      if (i < nn) {
+        const zc v = r[i];
+        const float a = high(v.x), b = high(v.y);
+        f = fmaf(a, a, fmaf(b, b, f));
+      }
+    }
+  }
+  for (int off = 16; off > 0; off >>= 1) f += __shfl_xor_sync(0xffffffffu, f, off);
+  if ((threadIdx.x & 31) == 0) redf[threadIdx.x >> 5] = f;
+  __syncthreads();
+  f = redf[0];
+  for (int w = 1; w < (int)(blockDim.x >> 5); ++w) f += redf[w];
+  const float t2 = (float)(tol * tol);
+  if (f < 0.999f * t2 || !(f < 1.001f * t2)) {
+    if (threadIdx.x == 0) redo[u] = (f < t2) ? 0 : 1;
+    return;
+  }
   double s = 0.0;
   for (int i = threadIdx.x; i < nn; i += blockDim.x) s += r[i].x * r[i].x + r[i].y * r[i].y;
-  __shared__ double red[32];
   for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
   __syncthreads();
@@ -1371,63 +1448,95 @@ __global__ void refine_check_kernel(BMat R, int n, const int* active, double tol
   }
 }
 
-// Smith step bookkeeping: S += inc; conv if max|inc| <= tol max|S|; rebalance P, Q
-__global__ void smith_accum_kernel(BMat S, BMat inc, int n, int* act, double tol) {
+// Smith step bookkeeping: S += inc; the unit ends if max|inc| <= tol max|S|
+__global__ void __launch_bounds__(1024) smith_accum_kernel(BMat S, BMat inc, int n, int* act, double tol) {
   const int u = blockIdx.x;
   if (!act[u]) return;
   const long long nn = (long long)n * n;
   zc* s = S.at(u);
   const zc* d = inc.at(u);
-  double mi = 0.0, ms = 0.0;   // squared moduli
-  for (long long i = threadIdx.x; i < nn; i += blockDim.x) {
-    zc v = zadd(s[i], d[i]);
-    s[i] = v;
-    mi = fmax(mi, zabs2(d[i]));
-    ms = fmax(ms, zabs2(v));
+  __shared__ double red[32];
+  __shared__ unsigned int rk[2][32];
+  unsigned int ki = 0, ks = 0;
+  for (long long i0 = threadIdx.x; i0 < nn; i0 += kBookUnroll * blockDim.x) {
+    zc a[kBookUnroll], b[kBookUnroll];
+#pragma unroll
+    for (int q = 0; q < kBookUnroll; ++q) {
+      const long long i = i0 + q * blockDim.x;
+      a[q] = b[q] = zmake(0.0, 0.0);
+      if (i < nn) { a[q] = s[i]; b[q] = d[i]; }
+    }
+#pragma unroll
+    for (int q = 0; q < kBookUnroll; ++q) {
+      const long long i = i0 + q * blockDim.x;
+      a[q] = zadd(a[q], b[q]);
+      if (i < nn) s[i] = a[q];
+      ki = max(ki, abs_key(b[q]));
+      ks = max(ks, abs_key(a[q]));
+    }
   }
-  __shared__ double r1[32], r2[32];
-  for (int off = 16; off > 0; off >>= 1) {
-    mi = fmax(mi, __shfl_down_sync(0xffffffffu, mi, off));
-    ms = fmax(ms, __shfl_down_sync(0xffffffffu, ms, off));
+  ki = cta_max(ki, rk[0]);
+  ks = cta_max(ks, rk[1]);
+  bool end = false, decided = false;
+  if (ks > kTiny && ks < kBig && ki < kBig) {   // each maximum between its largest component and sqrt(2) times it
+    end = 1.5 * key_hi(ki) <= tol * key_lo(ks);
+    decided = end || 0.999 * key_lo(ki) > tol * (1.5 * key_hi(ks));
   }
-  if ((threadIdx.x & 31) == 0) { r1[threadIdx.x >> 5] = mi; r2[threadIdx.x >> 5] = ms; }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) { mi = fmax(mi, r1[w]); ms = fmax(ms, r2[w]); }
-    mi = sqrt(mi);
-    ms = sqrt(ms);
-    if (mi <= tol * fmax(ms, 1e-300) || !isfinite(ms)) act[u] = 0;
+  if (!decided) {
+    const double mi = sqrt(cta_max_abs2(d, nn, red)), ms = sqrt(cta_max_abs2(s, nn, red));
+    end = mi <= tol * fmax(ms, 1e-300) || !isfinite(ms);
   }
+  if (threadIdx.x == 0 && end) act[u] = 0;
 }
 
-__global__ void balance_kernel(BMat P, BMat Q, int n, const int* act) {
+// v 2^e (|e| <= 1022): by the exponent field where v and the result are normal
+__device__ __forceinline__ double scale_pow2(double v, int e) {
+  const int hi = __double2hiint(v), x = (hi >> 20) & 0x7ff;
+  if (x == 0 || x == 0x7ff || x + e <= 0 || x + e >= 0x7ff) return v * __hiloint2double((e + 1023) << 20, 0);
+  return __hiloint2double(hi + e * (1 << 20), __double2loint(v));
+}
+
+// P *= s, Q /= s with the power of two s that brings their largest entries together (within a
+// factor 4): P S Q is what it was, bit for bit
+__global__ void __launch_bounds__(1024) balance_kernel(BMat P, BMat Q, int n, const int* act) {
   const int u = blockIdx.x;
   if (!act[u]) return;
   const long long nn = (long long)n * n;
   zc* p = P.at(u);
   zc* q = Q.at(u);
-  double mp = 0.0, mq = 0.0;   // squared moduli
-  for (long long i = threadIdx.x; i < nn; i += blockDim.x) {
-    mp = fmax(mp, zabs2(p[i]));
-    mq = fmax(mq, zabs2(q[i]));
+  __shared__ unsigned int rk[2][32];   // (two reductions in a row)
+  unsigned int kp = 0, kq = 0;
+  for (long long i0 = threadIdx.x; i0 < nn; i0 += kBookUnroll * blockDim.x) {
+#pragma unroll
+    for (int x = 0; x < kBookUnroll; ++x) {
+      const long long i = i0 + x * blockDim.x;
+      if (i < nn) {
+        kp = max(kp, abs_key(p[i]));
+        kq = max(kq, abs_key(q[i]));
+      }
+    }
   }
-  __shared__ double r1[32], r2[32];
-  __shared__ double sc;
-  for (int off = 16; off > 0; off >>= 1) {
-    mp = fmax(mp, __shfl_down_sync(0xffffffffu, mp, off));
-    mq = fmax(mq, __shfl_down_sync(0xffffffffu, mq, off));
-  }
-  if ((threadIdx.x & 31) == 0) { r1[threadIdx.x >> 5] = mp; r2[threadIdx.x >> 5] = mq; }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) { mp = fmax(mp, r1[w]); mq = fmax(mq, r2[w]); }
-    sc = (mp > 0.0 && mq > 0.0) ? sqrt(sqrt(mq) / sqrt(mp)) : 1.0;
-  }
-  __syncthreads();
-  const double s = sc;
-  for (long long i = threadIdx.x; i < nn; i += blockDim.x) {
-    p[i] = zscale(p[i], s);
-    q[i] = zscale(q[i], 1.0 / s);
+  kp = cta_max(kp, rk[0]) >> 20;
+  kq = cta_max(kq, rk[1]) >> 20;
+  if (kp == 0 || kq == 0 || kp == 0x7ff || kq == 0x7ff) return;
+  const int e = ((int)kq - (int)kp) / 2;
+  if (e == 0) return;
+  for (long long i0 = threadIdx.x; i0 < nn; i0 += kBookUnroll * blockDim.x) {
+    zc a[kBookUnroll], b[kBookUnroll];
+#pragma unroll
+    for (int x = 0; x < kBookUnroll; ++x) {
+      const long long i = i0 + x * blockDim.x;
+      a[x] = b[x] = zmake(0.0, 0.0);
+      if (i < nn) { a[x] = p[i]; b[x] = q[i]; }
+    }
+#pragma unroll
+    for (int x = 0; x < kBookUnroll; ++x) {
+      const long long i = i0 + x * blockDim.x;
+      if (i < nn) {
+        p[i] = zmake(scale_pow2(a[x].x, e), scale_pow2(a[x].y, e));
+        q[i] = zmake(scale_pow2(b[x].x, -e), scale_pow2(b[x].y, -e));
+      }
+    }
   }
 }
 
@@ -2625,12 +2734,12 @@ negf_status negf_obc(negf_ctx* c, const negf_system* sys, negf_precision prec, d
           return NEGF_OK;
         }
         CU(eng.inverse(X, M, b, NU, nullptr, T[0], T[1], 2, mask));
-        refine_check_kernel<<<NU, 256, 0, s>>>(T[0], b, mask, 1e-7, redo);
+        refine_check_kernel<<<NU, book_threads(b), 0, s>>>(T[0], b, mask, 1e-7, redo);
         KCHECK();
         // units whose refinement converges slowly (kappa(eps) up to ~1e7) take two more
         // steps; FP64 Gauss-Jordan for what is left
         CU(eng.refine_steps(X, M, b, NU, T[0], T[1], 2, redo));
-        refine_check_kernel<<<NU, 256, 0, s>>>(T[0], b, redo, 1e-7, redo);
+        refine_check_kernel<<<NU, book_threads(b), 0, s>>>(T[0], b, redo, 1e-7, redo);
         KCHECK();
         CU(eng.inv(X, M, b, NU, redo, 0, nullptr));
         return NEGF_OK;
@@ -2693,13 +2802,13 @@ negf_status negf_obc(negf_ctx* c, const negf_system* sys, negf_precision prec, d
         for (int j = 0; j < 96; ++j) {
           CU(lgemm(W1, Pm, OP_N, Sm, OP_N, ONE, NOMAT, ZERO, act));              // P S
           CU(lgemm(W2, W1, OP_N, Qm, OP_N, ONE, NOMAT, ZERO, act));              // P S Q
-          smith_accum_kernel<<<NU, 256, 0, s>>>(Sm, W2, b, act, 1e-15);
+          smith_accum_kernel<<<NU, book_threads(b), 0, s>>>(Sm, W2, b, act, 1e-15);
           KCHECK();
           CU(lgemm(W1, Pm, OP_N, Pm, OP_N, ONE, NOMAT, ZERO, act));              // P^2
           CU(lgemm(W3, Qm, OP_N, Qm, OP_N, ONE, NOMAT, ZERO, act));              // Q^2
           std::swap(Pm, W1);
           std::swap(Qm, W3);
-          balance_kernel<<<NU, 256, 0, s>>>(Pm, Qm, b, act);
+          balance_kernel<<<NU, book_threads(b), 0, s>>>(Pm, Qm, b, act);
           KCHECK();
           if ((j & 7) == 7) {
             const int c2 = n_set(act);
@@ -2742,7 +2851,7 @@ negf_status negf_obc(negf_ctx* c, const negf_system* sys, negf_precision prec, d
       const int n_cold = any_warm ? n_set(cold) : NU;
       if (n_cold < 0) return fail(ctx, NEGF_ERR_CUDA, "OBC: flag read-back failed");
 
-      lead_norm_kernel<<<NU, 256, 0, s>>>(al, be, b, 0, ref, done, act, it_arr, 0, tol, n_active, keep);
+      lead_norm_kernel<<<NU, book_threads(b), 0, s>>>(al, be, b, 0, ref, done, act, it_arr, 0, tol, n_active, keep);
       KCHECK();
       if (n_cold > 0) {
         // ---- decimation
@@ -2750,7 +2859,7 @@ negf_status negf_obc(negf_ctx* c, const negf_system* sys, negf_precision prec, d
           // counts after the first step (most units end there) and every fourth
           const bool poll = it == 1 || (it & 3) == 3 || it == max_iter;
           if (poll) CU(cudaMemsetAsync(n_active, 0, sizeof(int), s));
-          lead_norm_kernel<<<NU, 256, 0, s>>>(al, be, b, 1, ref, done, act, it_arr, it, tol,
+          lead_norm_kernel<<<NU, book_threads(b), 0, s>>>(al, be, b, 1, ref, done, act, it_arr, it, tol,
                                               poll ? n_active : nullptr);
           KCHECK();
           if (poll) {
