@@ -278,13 +278,13 @@ static cudaError_t launch_inv(BMat X, BMat M, int n, int units, const int* activ
 static bool f64_tiles(int n, int units) { return n >= 112 || (n >= 64 && units <= 76); }
 
 cudaError_t zinv(BMat X, BMat M, int n, int units, const int* active, int single, void* scratch,
-                 int32_t* status, cudaStream_t s, void* lent, size_t lent_bytes) {
+                 int32_t* status, cudaStream_t s, void* lent, size_t lent_bytes, bool few) {
   if (units <= 0 || n <= 0) return cudaSuccess;
   if (single && n <= 128) return zinv_reg(X, M, n, units, active, status, s);
   if (n <= 512 && (single || f64_tiles(n, units))) {
     const size_t need = zinv_tiles_bytes(n, units, single);
     void* t = lent_bytes >= need ? lent : (zinv_scratch_bytes(n, units, single) >= need ? scratch : nullptr);
-    if (t) return zinv_tiles(X, M, n, units, active, single, t, status, s);
+    if (t) return zinv_tiles(X, M, n, units, active, single, t, status, s, few);
   }
   if (single) return launch_inv<float>(X, M, n, units, active, scratch, status, s);
   return launch_inv<double>(X, M, n, units, active, scratch, status, s);

@@ -22,6 +22,7 @@
 // per block: FP32 n = 512, 16 blocks 27.9 -> 1.22 ms; n = 256, 8 blocks 4.01 -> 0.28 ms; FP64
 // n = 128, one block 2.50 -> 0.47 ms, 400 blocks 7.6 -> 6.1 ms; n = 512, 2 blocks 138 -> 5.5 ms.
 // TW: a row's entries fit in 32 registers, and the update reads C once for TW columns.
+#include <algorithm>
 #include <type_traits>
 
 #include "negf_internal.cuh"
@@ -167,7 +168,7 @@ __device__ __forceinline__ void tile_step(const TileInv<typename Tr<R>::C>& g, i
   const size_t prow_n = (size_t)g.units * n;
   const uint16_t* pos_in = g.pos + (size_t)(panel & 1) * prow_n + (size_t)u * n;
   __shared__ __align__(16) C yk[TW][TW];
-  __shared__ __align__(16) C prow[2][NT / 32][TW];
+  __shared__ __align__(16) C prow[2][NT / 32][TW + V];   // the warps' candidates: row and 1 / pivot
   __shared__ uint2 s_key[2][NT / 32];
   __shared__ int s_pos[2][NT / 32];
 
@@ -244,6 +245,8 @@ __device__ __forceinline__ void tile_step(const TileInv<typename Tr<R>::C>& g, i
       unsigned int hi, lo;
       pivot_key(cand, v, hi, lo);
       const bool top = warp_max<R>(hi, lo);
+      C own;   // FP64: every row's 1 / entry beside the search (472 against 488 us at n = 128); only the pivot's is used
+      if constexpr (sizeof(R) == 8) own = cinv(a[0]);
       int p = __reduce_min_sync(0xffffffffu, (cand && top) ? mypos : kMaxN);
       // every warp publishes its own candidate with its row; one barrier, then all
       // threads pick the winner (the buffers alternate: a warp may be one step ahead)
@@ -252,6 +255,7 @@ __device__ __forceinline__ void tile_step(const TileInv<typename Tr<R>::C>& g, i
         s_pos[bf][warp] = p;
 #pragma unroll
         for (int c = 0; c < TW; ++c) prow[bf][warp][c] = a[c];
+        if constexpr (sizeof(R) == 8) prow[bf][warp][TW] = own;
       } else if (lane == 0 && hi == 0u) {
         s_key[bf][warp] = make_uint2(0u, 0u);
         s_pos[bf][warp] = kMaxN;
@@ -265,7 +269,9 @@ __device__ __forceinline__ void tile_step(const TileInv<typename Tr<R>::C>& g, i
       p = __reduce_min_sync(0xffffffffu, wtop ? wp : kMaxN);
       const int ww = __ffs(__ballot_sync(0xffffffffu, wtop && wp == p)) - 1;
       const C* pr = prow[bf][ww];
-      const C di = cinv(pr[0]);   // 0: a zero column, where the first row left stands in for the pivot
+      C di;
+      if constexpr (sizeof(R) == 8) di = pr[TW];
+      else di = cinv(pr[0]);   // 0: a zero column, where the first row left stands in for the pivot
       if (hi <= 1u) sing = true;
       const bool win = has && mypos == p;
       // row r -= f (pivot row / d), with -f / d in place of the pivot column; the pivot
@@ -304,61 +310,128 @@ __device__ __forceinline__ void tile_step(const TileInv<typename Tr<R>::C>& g, i
   }
 }
 
+// the CTA's units of a launch whose blockIdx.y starts at them: the next with its flag set, from u
+// on in steps of gridDim.y (g.units: none left).  Flags are read a warp at a time.
+template <typename C>
+__device__ __forceinline__ int next_unit(const TileInv<C>& g, int u) {
+  if (!g.active) return min(u, g.units);
+  for (; u < g.units; u += 32 * gridDim.y) {
+    const long long x = u + (long long)(threadIdx.x & 31) * gridDim.y;
+    const unsigned int m = __ballot_sync(0xffffffffu, x < g.units && g.active[x]);
+    if (m) return u + (__ffs(m) - 1) * (int)gridDim.y;
+  }
+  return g.units;
+}
+
 template <typename R, int NT>
 __global__ void __launch_bounds__(NT, (sizeof(R) == 4 ? 1024 : 512) / NT)
     inv_tile_kernel(TileInv<typename Tr<R>::C> g, int panel) {
   const int t = blockIdx.x;
   if (t == panel) return;
-  for (int u = blockIdx.y; u < g.units; u += gridDim.y) {
-    if (g.active && !g.active[u]) continue;
+  for (int u = next_unit(g, blockIdx.y); u < g.units; u = next_unit(g, u + gridDim.y)) {
     tile_step<R, NT>(g, panel, t, u);
     __syncthreads();   // the next unit of this CTA reuses the shared buffers
   }
 }
 
-// X[i][c] = W[row at position i][position of row c], in FP64
+// X[i][c] = W[row at position i][position of row c], in FP64, for rows i0 .. i0 + rows - 1 (<= 16)
 constexpr int kOutRows = 16;
 template <typename C>
-__global__ void __launch_bounds__(256) inv_gather_kernel(TileInv<C> g, int last_panel) {
-  const int n = g.n, i0 = blockIdx.x * kOutRows;
+__device__ __forceinline__ void gather_rows(const TileInv<C>& g, int last_panel, int u, int i0, int rows) {
+  const int n = g.n;
   __shared__ int s_pos[kMaxN];
   __shared__ int s_row[kOutRows];
-  for (int u = blockIdx.y; u < g.units; u += gridDim.y) {
-    if (g.active && !g.active[u]) continue;
-    const uint16_t* pos = g.pos + (size_t)(last_panel & 1) * g.units * n + (size_t)u * n;
-    for (int r = threadIdx.x; r < n; r += 256) {
-      const int p = pos[r];
-      s_pos[r] = p;
-      if (p >= i0 && p < i0 + kOutRows) s_row[p - i0] = r;
-    }
-    __syncthreads();
-    const C* W = g.W + (size_t)u * tile_stride(n);
-    zc* X = g.X.at(u);
-    const int rows = min(kOutRows, n - i0);
-    for (int i = threadIdx.x >> 5; i < rows; i += 8) {
-      const int r = s_row[i];
+  const uint16_t* pos = g.pos + (size_t)(last_panel & 1) * g.units * n + (size_t)u * n;
+  for (int r = threadIdx.x; r < n; r += blockDim.x) {
+    const int p = pos[r];
+    s_pos[r] = p;
+    if (p >= i0 && p < i0 + rows) s_row[p - i0] = r;
+  }
+  __syncthreads();
+  const C* W = g.W + (size_t)u * tile_stride(n);
+  zc* X = g.X.at(u);
+  for (int i = threadIdx.x >> 5; i < rows; i += (int)blockDim.x >> 5) {
+    const int r = s_row[i];
 #pragma unroll 4
-      for (int c = threadIdx.x & 31; c < n; c += 32) {
-        X[(size_t)(i0 + i) * n + c] = widen(W[elem<C>(n, r, s_pos[c])]);
-      }
+    for (int c = threadIdx.x & 31; c < n; c += 32) X[(size_t)(i0 + i) * n + c] = widen(W[elem<C>(n, r, s_pos[c])]);
+  }
+  __syncthreads();
+}
+
+template <typename C>
+__global__ void __launch_bounds__(256) inv_gather_kernel(TileInv<C> g, int last_panel) {
+  const int i0 = blockIdx.x * kOutRows;
+  for (int u = next_unit(g, blockIdx.y); u < g.units; u = next_unit(g, u + gridDim.y))
+    gather_rows(g, last_panel, u, i0, min(kOutRows, g.n - i0));
+}
+
+// Up to 16 tiles and few units: one cluster per unit with a CTA per tile, cluster barriers in
+// place of the launches (the tiles still pass through L2).  No gaps between the panels, and
+// a mask without units costs one launch; but a waiting cluster holds its SMs, so many units
+// run better as launches.  Measured (GB300, us, launches : cluster): FP64 n = 128, no unit of
+// 384 set 110 : 6, 1 472 : 415, 8 472 : 598 (the CTAs of a cluster share SMs and their FP64
+// pipes), 32 1142 : 808, 48 1173 : 1329, 400 6103 : 8883; n = 72, 1 261 : 232, 24 327 : 460; n = 64,
+// 8 236 : 205.  FP32 n = 200, 1 254 : 196, 24 286 : 280, 40 371 : 452; n = 256, 32 537 : 361;
+// n = 140, 8 180 : 164, 40 218 : 310.
+constexpr int kMaxCluster = 16;   // more than 8 CTAs: opted in, every GPC has room for them
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+template <typename R, int NT>
+__global__ void __launch_bounds__(NT, (sizeof(R) == 4 ? 1024 : 512) / NT)
+    inv_cluster_kernel(TileInv<typename Tr<R>::C> g, int tiles) {
+  const int t = blockIdx.x, per = (g.n + gridDim.x - 1) / gridDim.x, i0 = t * per;
+  // (the CTAs of a cluster share blockIdx.y and so take the same units)
+  for (int u = next_unit(g, blockIdx.y); u < g.units; u = next_unit(g, u + gridDim.y)) {
+    for (int panel = -1; panel < tiles; ++panel) {
+      if (t < tiles && t != panel) tile_step<R, NT>(g, panel, t, u);
+      cluster_barrier();
     }
-    __syncthreads();
+    gather_rows(g, tiles - 1, u, i0, max(0, min(per, g.n - i0)));
   }
 }
 
 template <typename R, int NT>
 cudaError_t launch_tiles(const TileInv<typename Tr<R>::C>& g, int tiles, int rows, cudaStream_t s) {
   for (int panel = -1; panel < tiles; ++panel) {
-    if (panel == 0 && tiles == 1) break;   // no other tile to update
     inv_tile_kernel<R, NT><<<dim3(tiles, rows), NT, 0, s>>>(g, panel);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
-  return cudaSuccess;
+  inv_gather_kernel<<<dim3((g.n + kOutRows - 1) / kOutRows, rows), 256, 0, s>>>(g, tiles - 1);
+  return cudaGetLastError();
+}
+
+template <typename R, int NT>
+cudaError_t launch_cluster(const TileInv<typename Tr<R>::C>& g, int tiles, int rows, int slot, cudaStream_t s) {
+  const int cs = tiles <= 8 ? 8 : kMaxCluster;
+  cudaError_t e = once_per_device(slot, [](int) {
+    return cudaFuncSetAttribute(inv_cluster_kernel<R, NT>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  });
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(cs, rows);
+  cfg.blockDim = dim3(NT);
+  cfg.stream = s;
+  cudaLaunchAttribute at = {};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = cs;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, inv_cluster_kernel<R, NT>, g, tiles);
+}
+
+template <typename R, int NT>
+cudaError_t launch_inv(const TileInv<typename Tr<R>::C>& g, int tiles, int rows, bool cluster, int slot, cudaStream_t s) {
+  if constexpr (NT <= kMaxCluster * Tr<R>::TW)
+    if (cluster) return launch_cluster<R, NT>(g, tiles, rows, slot, s);
+  return launch_tiles<R, NT>(g, tiles, rows, s);
 }
 
 template <typename R>
-cudaError_t run(BMat X, BMat M, int n, int units, const int* active, void* scratch, int32_t* status, cudaStream_t s) {
+cudaError_t run(BMat X, BMat M, int n, int units, const int* active, bool few, void* scratch, int32_t* status,
+                cudaStream_t s) {
   typedef typename Tr<R>::C C;
   TileInv<C> g;
   g.M = M; g.X = X; g.n = n; g.units = units; g.active = active;
@@ -366,13 +439,14 @@ cudaError_t run(BMat X, BMat M, int n, int units, const int* active, void* scrat
   g.pos = (uint16_t*)(g.W + tile_stride(n) * units);
   g.status = status;
   const int tiles = (n + Tr<R>::TW - 1) / Tr<R>::TW;
-  const int rows = active && units > kMaskedUnits ? kMaskedUnits : units;
-  cudaError_t e = n <= 64 ? launch_tiles<R, 64>(g, tiles, rows, s)
-                : n <= 128 ? launch_tiles<R, 128>(g, tiles, rows, s)
-                : n <= 256 ? launch_tiles<R, 256>(g, tiles, rows, s) : launch_tiles<R, 512>(g, tiles, rows, s);
-  if (e != cudaSuccess) return e;
-  inv_gather_kernel<C><<<dim3((n + kOutRows - 1) / kOutRows, rows), 256, 0, s>>>(g, tiles - 1);
-  return cudaGetLastError();
+  const int rows = std::min(units, active ? kMaskedUnits : 65535);
+  const bool cluster = active ? few : units * (tiles <= 8 ? 1 : 2) <= (sizeof(R) == 4 ? 48 : 8);
+  if constexpr (sizeof(R) == 8) {   // (FP32 blocks up to 128: zinv_reg)
+    if (n <= 64) return launch_inv<R, 64>(g, tiles, rows, cluster, INIT_INVC_D64, s);
+    if (n <= 128) return launch_inv<R, 128>(g, tiles, rows, cluster, INIT_INVC_D128, s);
+  }
+  return n <= 256 ? launch_inv<R, 256>(g, tiles, rows, cluster, INIT_INVC_F256, s)
+                  : launch_inv<R, 512>(g, tiles, rows, false, 0, s);
 }
 
 // ---------------------------------------------------------------------------
@@ -683,11 +757,11 @@ size_t zinv_tiles_bytes(int n, int units, int single) {
 }
 
 cudaError_t zinv_tiles(BMat X, BMat M, int n, int units, const int* active, int single, void* scratch, int32_t* status,
-                       cudaStream_t s) {
+                       cudaStream_t s, bool few) {
   if (units <= 0 || n <= 0) return cudaSuccess;
   if (!scratch || n > kMaxN) return cudaErrorInvalidValue;
-  return single ? run<float>(X, M, n, units, active, scratch, status, s)
-                : run<double>(X, M, n, units, active, scratch, status, s);
+  return single ? run<float>(X, M, n, units, active, few, scratch, status, s)
+                : run<double>(X, M, n, units, active, few, scratch, status, s);
 }
 
 }  // namespace negf

@@ -518,9 +518,9 @@ struct Engine {
     return e;
   }
   // l1, l2: two adjacent blocks per unit that are free meanwhile (nullable), lent to the FP64
-  // inverse as scratch
+  // inverse as scratch; few: some tens of the mask's units at most
   cudaError_t inv(BMat X, BMat M, int n, int units, const int* active, int single, int32_t* status, BMat l1 = BMat{nullptr, 0},
-                  BMat l2 = BMat{nullptr, 0}) {
+                  BMat l2 = BMat{nullptr, 0}, bool few = false) {
     const bool masked = active != nullptr && active_frac < 0.0;   // an unknown share of the work
     const double frac = (active && active_frac >= 0.0) ? active_frac : 1.0;
     begin(masked ? K_OTHER : (single ? K_INV_F32 : K_INV_F64));
@@ -534,7 +534,7 @@ struct Engine {
       lent = l1.p;
       lent_bytes = 2 * sizeof(zc) * (size_t)nn * units;
     }
-    cudaError_t e = zinv(X, M, n, units, active, single, inv_scratch, status, s, lent, lent_bytes);
+    cudaError_t e = zinv(X, M, n, units, active, single, inv_scratch, status, s, lent, lent_bytes, few);
     end(masked ? 0.0 : 8.0 * (double)n * n * n * units * frac, masked ? 0.0 : 32.0 * (double)n * n * units * frac);
     return e;
   }
@@ -2741,7 +2741,7 @@ negf_status negf_obc(negf_ctx* c, const negf_system* sys, negf_precision prec, d
         CU(eng.refine_steps(X, M, b, NU, T[0], T[1], 2, redo));
         refine_check_kernel<<<NU, book_threads(b), 0, s>>>(T[0], b, redo, 1e-7, redo);
         KCHECK();
-        CU(eng.inv(X, M, b, NU, redo, 0, nullptr));
+        CU(eng.inv(X, M, b, NU, redo, 0, nullptr, BMat{nullptr, 0}, BMat{nullptr, 0}, true));
         return NEGF_OK;
       };
       auto residual = [&](BMat X, double* out, const int* mask) -> negf_status {
@@ -2792,7 +2792,7 @@ negf_status negf_obc(negf_ctx* c, const negf_system* sys, negf_precision prec, d
       // cnt = the number of units in `mask`.
       auto newton_step = [&](int* mask, BMat gn, int cnt) -> negf_status {
         negf_status sc;
-        CU(eng.inv(T[3], T[1], b, NU, mask, 0, nullptr, T[4], T[5]));     // K^{-1}
+        CU(eng.inv(T[3], T[1], b, NU, mask, 0, nullptr, T[4], T[5], cnt <= 40));     // K^{-1}
         if ((sc = compact(mask, cnt)) != NEGF_OK) return sc;
         CU(lgemm(T[4], T[3], OP_N, al0, OP_N, ONE, NOMAT, ZERO, mask));          // P = K^{-1} al
         CU(lgemm(T[5], be0, OP_N, g, OP_N, ONE, NOMAT, ZERO, mask));             // Q = be g

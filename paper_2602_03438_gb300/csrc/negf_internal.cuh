@@ -21,7 +21,7 @@ namespace negf {
 // ---------------------------------------------------------------------------
 enum InitSlot { INIT_OZ = 0, INIT_TC, INIT_MLP, INIT_SMALL, INIT_OBC_SMALL, INIT_OZB, INIT_OZB_LO, INIT_OZB16,
                 INIT_OZB16_LO, INIT_INV32, INIT_INV64, INIT_INV96, INIT_INV128,
-                INIT_NSLOT };
+                INIT_INVC_F256, INIT_INVC_D64, INIT_INVC_D128, INIT_NSLOT };
 constexpr int kMaxDevices = 64;
 cudaError_t once_per_device(int slot, const std::function<cudaError_t(int device)>& init);
 
@@ -162,13 +162,14 @@ cudaError_t zgemm_ozt_variant(const GemmArgs& g, void* scratch, int* err, cudaSt
 // complex of the working precision).  status[u] (nullable, indexed status_base+u)
 // gets NEGF_ERR_SINGULAR on an exactly zero pivot.
 // `lent` (lent_bytes, nullable): 16-byte aligned scratch the caller does not need meanwhile.
+// few: some tens of the mask's units are set at most.
 cudaError_t zinv(BMat X, BMat M, int n, int units, const int* active, int single, void* scratch,
-                 int32_t* status, cudaStream_t s, void* lent = nullptr, size_t lent_bytes = 0);
+                 int32_t* status, cudaStream_t s, void* lent = nullptr, size_t lent_bytes = 0, bool few = false);
 size_t zinv_scratch_bytes(int n, int units, int single);
 // the inverse as column tiles, several CTAs per block (inv_tiles.cu; n <= 512); `scratch`
 // holds zinv_tiles_bytes(n, units, single) bytes, 16-byte aligned
 cudaError_t zinv_tiles(BMat X, BMat M, int n, int units, const int* active, int single, void* scratch, int32_t* status,
-                       cudaStream_t s);
+                       cudaStream_t s, bool few = false);
 size_t zinv_tiles_bytes(int n, int units, int single);
 // FP32, n <= 128: one CTA per block, the matrix in registers, no scratch
 cudaError_t zinv_reg(BMat X, BMat M, int n, int units, const int* active, int32_t* status, cudaStream_t s);

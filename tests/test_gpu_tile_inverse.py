@@ -94,3 +94,8 @@ def test_zero_column_is_reported(P, n, col):
     for u in (0, 2):
         bound = 8 * n * 2.0 ** -53 * float(M[u].norm()) * float(X[u].norm())
         assert float((eye - M[u] @ X[u]).norm()) <= bound
+
+
+@pytest.mark.parametrize("n,units", [(129, 24), (129, 25), (240, 26), (256, 24), (256, 25)])
+def test_tiles_of_few_and_many_blocks(P, n, units):   # one cluster per block up to 24 of them
+    test_tile_inverse(P, n, units)
