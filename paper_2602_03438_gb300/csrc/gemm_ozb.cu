@@ -272,6 +272,7 @@ struct PreArgs {
 constexpr int PRE = 32;
 template <int ND, bool HOLD, class ARGS>
 __global__ void __launch_bounds__(256) ozb_prepass_kernel(ARGS g, ImgArgs im, int a_blocks) {
+  pdl_begin();
   const int u = blockIdx.y;
   if (g.active && !g.active[u]) return;
   const int n = g.n, tid = threadIdx.x;
@@ -451,6 +452,7 @@ __global__ void __launch_bounds__(NT, 1) ozb_product_kernel(GemmArgs g, ImgArgs 
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  pdl_begin();
   const uint32_t tmem = *tmem_slot;
   const uint32_t lbase = smem_u32(base);
   // a tile's unit, row tile and column tile; every role walks the same tiles
@@ -756,20 +758,19 @@ cudaError_t launch(const GemmArgs& g, void* scratch, int* err, cudaStream_t s, i
   const dim3 pre(ab + blocks, g.units);
   if (g.A.plain() && g.B.plain()) {
     PreArgs a{Plain{g.A.p, g.A.us}, Plain{g.B.p, g.B.us}, g.opA, g.opB, n, g.active};
-    if (im.chunks <= PASS) ozb_prepass_kernel<ND, true><<<pre, 256, 0, s>>>(a, im, ab);
-    else ozb_prepass_kernel<ND, false><<<pre, 256, 0, s>>>(a, im, ab);
+    if (im.chunks <= PASS) e = launch_pdl(ozb_prepass_kernel<ND, true, PreArgs>, pre, 256, 0, s, a, im, ab);
+    else e = launch_pdl(ozb_prepass_kernel<ND, false, PreArgs>, pre, 256, 0, s, a, im, ab);
   } else {
-    if (im.chunks <= PASS) ozb_prepass_kernel<ND, true><<<pre, 256, 0, s>>>(g, im, ab);
-    else ozb_prepass_kernel<ND, false><<<pre, 256, 0, s>>>(g, im, ab);
+    if (im.chunks <= PASS) e = launch_pdl(ozb_prepass_kernel<ND, true, GemmArgs>, pre, 256, 0, s, g, im, ab);
+    else e = launch_pdl(ozb_prepass_kernel<ND, false, GemmArgs>, pre, 256, 0, s, g, im, ab);
   }
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  if (e != cudaSuccess) return e;
   const bool uab = (g.alpha.y == 0.0 && (g.alpha.x == 1.0 || g.alpha.x == -1.0)) &&
                    (!g.C.p || (g.beta.y == 0.0 && (g.beta.x == 0.0 || g.beta.x == 1.0 || g.beta.x == -1.0)));
   const long long tiles = (long long)g.units * im.tiles_m * im.tiles_n;
   const int grid = (int)(tiles < g_sms[dev] ? tiles : g_sms[dev]);
-  if (uab) ozb_product_kernel<ND, TNC, true><<<grid, NT, T::SMEM, s>>>(g, im, err);
-  else ozb_product_kernel<ND, TNC, false><<<grid, NT, T::SMEM, s>>>(g, im, err);
-  return cudaGetLastError();
+  return uab ? launch_pdl(ozb_product_kernel<ND, TNC, true>, grid, NT, T::SMEM, s, g, im, err)
+             : launch_pdl(ozb_product_kernel<ND, TNC, false>, grid, NT, T::SMEM, s, g, im, err);
 }
 
 }  // namespace

@@ -326,6 +326,7 @@ __device__ __forceinline__ int next_unit(const TileInv<C>& g, int u) {
 template <typename R, int NT>
 __global__ void __launch_bounds__(NT, (sizeof(R) == 4 ? 1024 : 512) / NT)
     inv_tile_kernel(TileInv<typename Tr<R>::C> g, int panel) {
+  pdl_begin();
   const int t = blockIdx.x;
   if (t == panel) return;
   for (int u = next_unit(g, blockIdx.y); u < g.units; u = next_unit(g, u + gridDim.y)) {
@@ -360,6 +361,7 @@ __device__ __forceinline__ void gather_rows(const TileInv<C>& g, int last_panel,
 
 template <typename C>
 __global__ void __launch_bounds__(256) inv_gather_kernel(TileInv<C> g, int last_panel) {
+  pdl_begin();
   const int i0 = blockIdx.x * kOutRows;
   for (int u = next_unit(g, blockIdx.y); u < g.units; u = next_unit(g, u + gridDim.y))
     gather_rows(g, last_panel, u, i0, min(kOutRows, g.n - i0));
@@ -380,6 +382,7 @@ __device__ __forceinline__ void cluster_barrier() {
 template <typename R, int NT>
 __global__ void __launch_bounds__(NT, (sizeof(R) == 4 ? 1024 : 512) / NT)
     inv_cluster_kernel(TileInv<typename Tr<R>::C> g, int tiles) {
+  pdl_begin();
   const int t = blockIdx.x, per = (g.n + gridDim.x - 1) / gridDim.x, i0 = t * per;
   // (the CTAs of a cluster share blockIdx.y and so take the same units)
   for (int u = next_unit(g, blockIdx.y); u < g.units; u = next_unit(g, u + gridDim.y)) {
@@ -394,12 +397,10 @@ __global__ void __launch_bounds__(NT, (sizeof(R) == 4 ? 1024 : 512) / NT)
 template <typename R, int NT>
 cudaError_t launch_tiles(const TileInv<typename Tr<R>::C>& g, int tiles, int rows, cudaStream_t s) {
   for (int panel = -1; panel < tiles; ++panel) {
-    inv_tile_kernel<R, NT><<<dim3(tiles, rows), NT, 0, s>>>(g, panel);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_pdl(inv_tile_kernel<R, NT>, dim3(tiles, rows), NT, 0, s, g, panel);
     if (e != cudaSuccess) return e;
   }
-  inv_gather_kernel<<<dim3((g.n + kOutRows - 1) / kOutRows, rows), 256, 0, s>>>(g, tiles - 1);
-  return cudaGetLastError();
+  return launch_pdl(inv_gather_kernel<typename Tr<R>::C>, dim3((g.n + kOutRows - 1) / kOutRows, rows), 256, 0, s, g, tiles - 1);
 }
 
 template <typename R, int NT>
@@ -413,12 +414,14 @@ cudaError_t launch_cluster(const TileInv<typename Tr<R>::C>& g, int tiles, int r
   cfg.gridDim = dim3(cs, rows);
   cfg.blockDim = dim3(NT);
   cfg.stream = s;
-  cudaLaunchAttribute at = {};
-  at.id = cudaLaunchAttributeClusterDimension;
-  at.val.clusterDim.x = cs;
-  at.val.clusterDim.y = at.val.clusterDim.z = 1;
-  cfg.attrs = &at;
-  cfg.numAttrs = 1;
+  cudaLaunchAttribute at[2] = {};
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = cs;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 2;
   return cudaLaunchKernelEx(&cfg, inv_cluster_kernel<R, NT>, g, tiles);
 }
 
@@ -593,6 +596,7 @@ __device__ __forceinline__ void reg_update(float2 (&b)[RP], const float2* fr, co
 template <int NR>
 __global__ void __launch_bounds__(NR * (NR / RC), NR == 128 ? 1 : NR == 96 ? 2 : NR == 64 ? 4 : 8)
     inv_reg_kernel(BMat X, BMat M, int n, const int* active, int32_t* status) {
+  pdl_begin();
   const int u = blockIdx.x;
   if (active && !active[u]) return;
   constexpr int NQ = NR / RC, NT = NR * NQ, NW = NR / 32;
@@ -738,8 +742,7 @@ cudaError_t launch_reg(BMat X, BMat M, int n, int units, const int* active, int3
     return cudaFuncSetAttribute(inv_reg_kernel<NR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)reg_smem<NR>());
   });
   if (e != cudaSuccess) return e;
-  inv_reg_kernel<NR><<<units, NR * (NR / RC), reg_smem<NR>(), s>>>(X, M, n, active, status);
-  return cudaGetLastError();
+  return launch_pdl(inv_reg_kernel<NR>, units, NR * (NR / RC), reg_smem<NR>(), s, X, M, n, active, status);
 }
 
 }  // namespace

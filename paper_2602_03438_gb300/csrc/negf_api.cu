@@ -206,6 +206,7 @@ constexpr int ASM_T = 32;
 // compiler does not merge the two forms' arithmetic into one predicated sequence
 template <bool USE_W>
 __global__ void __launch_bounds__(256) assemble_kernel(AsmArgs a) {
+  pdl_begin();
   const int u = blockIdx.y;
   int e;
   if (a.udev) {   // the unit's own device
@@ -363,15 +364,12 @@ cudaError_t assemble(const AsmArgs& a, cudaStream_t s) {
   if (a.units <= 0) return cudaSuccess;
   const int nt = (a.dv.b + ASM_T - 1) / ASM_T;
   const dim3 grid((unsigned)(nt * nt), a.units, a.all_blocks ? a.dv.nb : 1);
-  if (a.Wd)
-    assemble_kernel<true><<<grid, dim3(ASM_T, 8), 0, s>>>(a);
-  else
-    assemble_kernel<false><<<grid, dim3(ASM_T, 8), 0, s>>>(a);
-  return cudaGetLastError();
+  return launch_pdl(a.Wd ? assemble_kernel<true> : assemble_kernel<false>, grid, dim3(ASM_T, 8), 0, s, a);
 }
 
 // D = D - W + W^H   (the anti-Hermitian completion of G^<_ii)
 __global__ void antiherm_update_kernel(BMat D, BMat W, int n, const int* act) {
+  pdl_begin();
   const int u = blockIdx.y;
   if (act && !act[u]) return;
   const long long nn = (long long)n * n;
@@ -388,12 +386,12 @@ cudaError_t antiherm_update(BMat D, BMat W, int n, int units, cudaStream_t s, co
   if (units <= 0) return cudaSuccess;
   const long long nn = (long long)n * n;
   dim3 grid((unsigned)std::min<long long>((nn + 255) / 256, 1024), units);
-  antiherm_update_kernel<<<grid, 256, 0, s>>>(D, W, n, act);
-  return cudaGetLastError();
+  return launch_pdl(antiherm_update_kernel, grid, 256, 0, s, D, W, n, act);
 }
 
 // D = A + B on the masked units
 __global__ void add_kernel(BMat D, BMat A, BMat B, int n, const int* act) {
+  pdl_begin();
   const int u = blockIdx.y;
   if (act && !act[u]) return;
   const long long nn = (long long)n * n;
@@ -606,8 +604,7 @@ struct Engine {
           cudaSuccess)
         return e;                                                          // X (I - M X)
       ++ctx->launches;
-      add_kernel<<<grid, 256, 0, s>>>(X, X, T2, n, active);
-      if ((e = cudaGetLastError()) != cudaSuccess) return e;
+      if ((e = launch_pdl(add_kernel, grid, 256, 0, s, X, X, T2, n, active)) != cudaSuccess) return e;
     }
     return cudaSuccess;
   }
@@ -855,6 +852,7 @@ negf_status rgf_chunk(Ctx* ctx, Engine& eng, const DevView& dv, const ScatView& 
 
 // dst[u] = src[u] (units of any BMat layout)
 __global__ void bcopy_kernel(BMat dst, BMat src, int n) {
+  pdl_begin();
   const int u = blockIdx.y;
   const long long nn = (long long)n * n;
   zc* d = dst.at(u);
@@ -866,8 +864,7 @@ __global__ void bcopy_kernel(BMat dst, BMat src, int n) {
 cudaError_t bcopy(BMat dst, BMat src, int n, int units, cudaStream_t s) {
   if (units <= 0) return cudaSuccess;
   const long long nn = (long long)n * n;
-  bcopy_kernel<<<dim3((unsigned)std::min<long long>((nn + 255) / 256, 1024), units), 256, 0, s>>>(dst, src, n);
-  return cudaGetLastError();
+  return launch_pdl(bcopy_kernel, dim3((unsigned)std::min<long long>((nn + 255) / 256, 1024), units), 256, 0, s, dst, src, n);
 }
 
 // status[e] = the worst (most negative) code of the units e*P .. e*P+P-1
@@ -983,8 +980,8 @@ negf_status rgf_partitioned_chunk(Ctx* ctx, Engine& eng, const DevView& dv, cons
     if (r + 1 < P) {                                                        // + dD_a of partition r+1
       ++ctx->launches;
       const long long nn = bb;
-      add_kernel<<<dim3((unsigned)std::min<long long>((nn + 255) / 256, 1024), U), 256, 0, s>>>(
-          S1(T0), ofP(D, r), ofP(dDa, r + 1), b, nullptr);
+      launch_pdl(add_kernel, dim3((unsigned)std::min<long long>((nn + 255) / 256, 1024), U), 256, 0, s,
+                 S1(T0), ofP(D, r), ofP(dDa, r + 1), b, nullptr);
       CU(cudaGetLastError());
       M = S1(T0);
     }
@@ -1166,7 +1163,7 @@ negf_status rgf_arrowhead_chunk(Ctx* ctx, Engine& eng, const DevView& dv, const 
   }
   // ---------------- the tip: G_tt = (A_tt + dD_t)^{-1}
   ++ctx->launches;
-  add_kernel<<<eg, 256, 0, s>>>(S1(T0), S1(Att), S1(dDt), b, nullptr);
+  launch_pdl(add_kernel, eg, 256, 0, s, S1(T0), S1(Att), S1(dDt), b, nullptr);
   CU(cudaGetLastError());
   CU(eng.inverse(Gtt, S1(T0), b, U, st, S1(T1), S1(T2)));
   // ---------------- reconstruction from the last block up
@@ -1307,6 +1304,7 @@ int book_threads(int n) {        // a CTA per unit, kBookUnroll entries per thre
 __global__ void __launch_bounds__(1024) lead_norm_kernel(BMat al, BMat be, int n, int mode, double* ref, int* done,
                                                          int* live, int* iters, int it, double tol, int* n_active,
                                                          const int* skip = nullptr) {
+  pdl_begin();
   const int u = blockIdx.x;
   if (mode == 1 && done[u]) return;
   if (mode == 0 && skip && skip[u]) {   // solved by the warm start: no decimation
@@ -1363,6 +1361,7 @@ __global__ void __launch_bounds__(1024) lead_norm_kernel(BMat al, BMat be, int n
 
 // eps_s -= agb; eps -= agb + bga
 __global__ void lead_update_kernel(BMat eps, BMat epss, BMat agb, BMat bga, int n, const int* done) {
+  pdl_begin();
   const int u = blockIdx.y;
   if (done[u]) return;
   const long long nn = (long long)n * n;
@@ -1401,6 +1400,7 @@ __global__ void residual_kernel(BMat F, int n, double* res, const int* active) {
 // R = I - M X left by the last refinement step (the step from X to X + X R leaves an
 // error of the order of |R|^2) has a Frobenius norm above tol, or is not finite
 __global__ void __launch_bounds__(1024) refine_check_kernel(BMat R, int n, const int* active, double tol, int* redo) {
+  pdl_begin();
   const int u = blockIdx.x;
   if (active && !active[u]) {
     if (threadIdx.x == 0) redo[u] = 0;
@@ -1450,6 +1450,7 @@ __global__ void __launch_bounds__(1024) refine_check_kernel(BMat R, int n, const
 
 // Smith step bookkeeping: S += inc; the unit ends if max|inc| <= tol max|S|
 __global__ void __launch_bounds__(1024) smith_accum_kernel(BMat S, BMat inc, int n, int* act, double tol) {
+  pdl_begin();
   const int u = blockIdx.x;
   if (!act[u]) return;
   const long long nn = (long long)n * n;
@@ -1499,6 +1500,7 @@ __device__ __forceinline__ double scale_pow2(double v, int e) {
 // P *= s, Q /= s with the power of two s that brings their largest entries together (within a
 // factor 4): P S Q is what it was, bit for bit
 __global__ void __launch_bounds__(1024) balance_kernel(BMat P, BMat Q, int n, const int* act) {
+  pdl_begin();
   const int u = blockIdx.x;
   if (!act[u]) return;
   const long long nn = (long long)n * n;
@@ -2734,12 +2736,12 @@ negf_status negf_obc(negf_ctx* c, const negf_system* sys, negf_precision prec, d
           return NEGF_OK;
         }
         CU(eng.inverse(X, M, b, NU, nullptr, T[0], T[1], 2, mask));
-        refine_check_kernel<<<NU, book_threads(b), 0, s>>>(T[0], b, mask, 1e-7, redo);
+        launch_pdl(refine_check_kernel, NU, book_threads(b), 0, s, T[0], b, mask, 1e-7, redo);
         KCHECK();
         // units whose refinement converges slowly (kappa(eps) up to ~1e7) take two more
         // steps; FP64 Gauss-Jordan for what is left
         CU(eng.refine_steps(X, M, b, NU, T[0], T[1], 2, redo));
-        refine_check_kernel<<<NU, book_threads(b), 0, s>>>(T[0], b, redo, 1e-7, redo);
+        launch_pdl(refine_check_kernel, NU, book_threads(b), 0, s, T[0], b, redo, 1e-7, redo);
         KCHECK();
         CU(eng.inv(X, M, b, NU, redo, 0, nullptr, BMat{nullptr, 0}, BMat{nullptr, 0}, true));
         return NEGF_OK;
@@ -2802,13 +2804,13 @@ negf_status negf_obc(negf_ctx* c, const negf_system* sys, negf_precision prec, d
         for (int j = 0; j < 96; ++j) {
           CU(lgemm(W1, Pm, OP_N, Sm, OP_N, ONE, NOMAT, ZERO, act));              // P S
           CU(lgemm(W2, W1, OP_N, Qm, OP_N, ONE, NOMAT, ZERO, act));              // P S Q
-          smith_accum_kernel<<<NU, book_threads(b), 0, s>>>(Sm, W2, b, act, 1e-15);
+          launch_pdl(smith_accum_kernel, NU, book_threads(b), 0, s, Sm, W2, b, act, 1e-15);
           KCHECK();
           CU(lgemm(W1, Pm, OP_N, Pm, OP_N, ONE, NOMAT, ZERO, act));              // P^2
           CU(lgemm(W3, Qm, OP_N, Qm, OP_N, ONE, NOMAT, ZERO, act));              // Q^2
           std::swap(Pm, W1);
           std::swap(Qm, W3);
-          balance_kernel<<<NU, book_threads(b), 0, s>>>(Pm, Qm, b, act);
+          launch_pdl(balance_kernel, NU, book_threads(b), 0, s, Pm, Qm, b, act);
           KCHECK();
           if ((j & 7) == 7) {
             const int c2 = n_set(act);
@@ -2818,7 +2820,7 @@ negf_status negf_obc(negf_ctx* c, const negf_system* sys, negf_precision prec, d
           }
         }
         ncomp = 0;
-        add_kernel<<<eg, 256, 0, s>>>(gn, g, Sm, b, mask);                                  // g + D
+        launch_pdl(add_kernel, eg, 256, 0, s, gn, g, Sm, b, mask);   // g + D
         KCHECK();
         return residual(gn, resn, mask);
       };
@@ -2851,7 +2853,8 @@ negf_status negf_obc(negf_ctx* c, const negf_system* sys, negf_precision prec, d
       const int n_cold = any_warm ? n_set(cold) : NU;
       if (n_cold < 0) return fail(ctx, NEGF_ERR_CUDA, "OBC: flag read-back failed");
 
-      lead_norm_kernel<<<NU, book_threads(b), 0, s>>>(al, be, b, 0, ref, done, act, it_arr, 0, tol, n_active, keep);
+      launch_pdl(lead_norm_kernel, NU, book_threads(b), 0, s, al, be, b, 0, ref, done, act, it_arr, 0, tol, n_active,
+                 keep);
       KCHECK();
       if (n_cold > 0) {
         // ---- decimation
@@ -2859,8 +2862,8 @@ negf_status negf_obc(negf_ctx* c, const negf_system* sys, negf_precision prec, d
           // counts after the first step (most units end there) and every fourth
           const bool poll = it == 1 || (it & 3) == 3 || it == max_iter;
           if (poll) CU(cudaMemsetAsync(n_active, 0, sizeof(int), s));
-          lead_norm_kernel<<<NU, book_threads(b), 0, s>>>(al, be, b, 1, ref, done, act, it_arr, it, tol,
-                                              poll ? n_active : nullptr);
+          launch_pdl(lead_norm_kernel, NU, book_threads(b), 0, s, al, be, b, 1, ref, done, act, it_arr, it,
+                     tol, poll ? n_active : nullptr, nullptr);
           KCHECK();
           if (poll) {
             CU(cudaMemcpyAsync(ctx->h_pinned, n_active, sizeof(int), cudaMemcpyDeviceToHost, s));
@@ -2878,7 +2881,7 @@ negf_status negf_obc(negf_ctx* c, const negf_system* sys, negf_precision prec, d
           CU(lgemm(T[1], be, OP_N, g, OP_N, ONE, NOMAT, ZERO, act));              // be g
           CU(lgemm(T[3], T[1], OP_N, al, OP_N, ONE, NOMAT, ZERO, act));           // be g al
           CU(lgemm(T[5], T[1], OP_N, be, OP_N, MONE, NOMAT, ZERO, act, true));    // -be g be
-          lead_update_kernel<<<eg, 256, 0, s>>>(eps, epss, T[2], T[3], b, done);
+          launch_pdl(lead_update_kernel, eg, 256, 0, s, eps, epss, T[2], T[3], b, done);
           KCHECK();
           std::swap(al, T[4]);
           std::swap(be, T[5]);
