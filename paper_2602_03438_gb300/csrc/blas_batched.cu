@@ -38,6 +38,7 @@ cudaError_t once_per_device(int slot, const std::function<cudaError_t(int device
 // ---------------------------------------------------------------------------
 constexpr int kF64Threads = 128;
 __global__ void __launch_bounds__(kF64Threads) zgemm_f64_kernel(GemmArgs g) {
+  pdl_begin();
   const int u = blockIdx.y;
   if (g.active && !g.active[u]) return;
   const int n = g.n;
@@ -76,7 +77,7 @@ __global__ void __launch_bounds__(kF64Threads) zgemm_f64_kernel(GemmArgs g) {
 cudaError_t zgemm_f64(const GemmArgs& g, cudaStream_t s) {
   if (g.units <= 0 || g.n <= 0) return cudaSuccess;
   const dim3 grid((unsigned)(((long long)g.n * g.n + kF64Threads - 1) / kF64Threads), g.units);
-  zgemm_f64_kernel<<<grid, kF64Threads, 0, s>>>(g);
+  launch_pdl(zgemm_f64_kernel, grid, kF64Threads, 0, s, g);
   return cudaGetLastError();
 }
 
@@ -106,6 +107,7 @@ constexpr int kInvThreads = 1024;
 template <typename R, bool SMEM>
 __global__ void __launch_bounds__(kInvThreads) zinv_kernel(BMat X, BMat M, int n, const int* active,
                                                            typename CT<R>::T* scratch, int32_t* status) {
+  pdl_begin();
   typedef typename CT<R>::T C;
   const int u = blockIdx.x;
   if (active && !active[u]) return;
@@ -261,11 +263,11 @@ static cudaError_t launch_inv(BMat X, BMat M, int n, int units, const int* activ
     cudaError_t e = cudaFuncSetAttribute(zinv_kernel<R, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)full);
     if (e != cudaSuccess) return e;
-    zinv_kernel<R, true><<<units, kInvThreads, full, s>>>(X, M, n, active, nullptr, status);
+    launch_pdl(zinv_kernel<R, true>, units, kInvThreads, full, s, X, M, n, active, nullptr, status);
   } else {
     if (!scratch) return cudaErrorInvalidValue;
     const size_t t = inv_tail_bytes(n, sizeof(C));
-    zinv_kernel<R, false><<<units, kInvThreads, t, s>>>(X, M, n, active, (C*)scratch, status);
+    launch_pdl(zinv_kernel<R, false>, units, kInvThreads, t, s, X, M, n, active, (C*)scratch, status);
   }
   return cudaGetLastError();
 }

@@ -146,6 +146,7 @@ template <int TN>
 __global__ void __launch_bounds__(GEMM_THREADS, 1)
     bf16_gemm_tn_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, int K,
                         Epi ep, int* err) {
+  pdl_begin();
   constexpr int STAGES = stages(TN);
   constexpr uint32_t STAGE_BYTES = stage_bytes(TN);
   extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -292,6 +293,7 @@ constexpr int N_FREQ = 32;   // sine/cosine pairs of the energy encoding
 
 __global__ void pack_kernel(int b, int n, int nlead, const zc* H00, const zc* H01, const int32_t* lead,
                             const double* E, unsigned short* X, int k0p, int* err) {
+  pdl_begin();
   // 2^(k/4), k = 0..3: the frequencies w_m = 2^(m div 4) 2^((m mod 4)/4) are exact products
   const double roots2[4] = {1.0, 1.189207115002721, 1.4142135623730951, 1.6817928305074290};
   const int r = blockIdx.x;
@@ -341,6 +343,7 @@ __global__ void pack_kernel(int b, int n, int nlead, const zc* H00, const zc* H0
 }
 
 __global__ void cvt_bf16_kernel(const float* in, bf16* out, long long count) {
+  pdl_begin();
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < count;
        i += (long long)gridDim.x * blockDim.x)
     out[i] = __float2bfloat16_rn(in[i]);
@@ -348,6 +351,7 @@ __global__ void cvt_bf16_kernel(const float* in, bf16* out, long long count) {
 
 // out[c][r] = bf16(in[r][c]) for an R x C FP32 matrix (R, C multiples of 32)
 __global__ void cvt_transpose_kernel(const float* in, bf16* out, int R, int C) {
+  pdl_begin();
   __shared__ float t[32][33];
   const int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
   for (int k = threadIdx.y; k < 32; k += blockDim.y) t[k][threadIdx.x] = in[(size_t)(r0 + k) * C + c0 + threadIdx.x];
@@ -358,6 +362,7 @@ __global__ void cvt_transpose_kernel(const float* in, bf16* out, int R, int C) {
 
 // out[c][r] = in[r][c] for an R x C BF16 matrix (R, C multiples of 32)
 __global__ void transpose_bf16_kernel(const bf16* in, bf16* out, int R, int C) {
+  pdl_begin();
   __shared__ bf16 t[32][34];
   const int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
   for (int k = threadIdx.y; k < 32; k += blockDim.y) t[k][threadIdx.x] = in[(size_t)(r0 + k) * C + c0 + threadIdx.x];
@@ -368,6 +373,7 @@ __global__ void transpose_bf16_kernel(const bf16* in, bf16* out, int R, int C) {
 // Xg[r] = X[rows[r]] for r < n (zeros below and for indices outside [0, n_set))
 __global__ void gather_rows_kernel(const uint4* X, const int32_t* rows, int n, int n_set, int row_u4, uint4* Xg,
                                    int* err) {
+  pdl_begin();
   const int r = blockIdx.x;
   const int src = r < n ? rows[r] : -1;
   const bool ok = src >= 0 && src < n_set;
@@ -382,6 +388,7 @@ constexpr int LOSS_BLOCKS = 512;
 // partial sums of (Y - T)^2 in FP64
 __global__ void loss_kernel(const float* Y, const zc* G, const int32_t* rows, int n_set, int n, int np_, int nout,
                             double scale, float* dY32, bf16* dYb, double* partial) {
+  pdl_begin();
   const int bb = nout / 2;
   double acc = 0.0;
   // a block per half row (with a block per row the last rows left half the SMs idle)
@@ -417,6 +424,7 @@ __global__ void loss_kernel(const float* Y, const zc* G, const int32_t* rows, in
 // loss = (sum of the partials, fixed order) / count: one warp, each lane every 32nd partial (a
 // chain of 512 dependent FP64 additions took 30 us; the lanes' chains and the tree 2)
 __global__ void loss_final_kernel(const double* partial, int np, double inv_count, double* loss) {
+  pdl_begin();
   double t = 0.0;
   for (int i = threadIdx.x; i < np; i += 32) t += partial[i];
   for (int off = 16; off > 0; off >>= 1) t += __shfl_down_sync(0xffffffffu, t, off);
@@ -428,6 +436,7 @@ __global__ void loss_final_kernel(const double* partial, int np, double inv_coun
 // chain of n FP64 additions: 43 us for n = 256 whatever N; 8 us so.
 constexpr int CS_WARPS = 16;
 __global__ void __launch_bounds__(32 * CS_WARPS) colsum_kernel(const float* A, int lda, int n, int N, float* out) {
+  pdl_begin();
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, c = blockIdx.x * 32 + lane;
   __shared__ double part[CS_WARPS][32];
   double t = 0.0;
@@ -445,6 +454,7 @@ __global__ void __launch_bounds__(32 * CS_WARPS) colsum_kernel(const float* A, i
 template <int V>
 __global__ void adam_kernel(float* theta, float* m, float* v, const float* g, long long count, float lr, float b1,
                             float b2, float eps, float c1, float c2) {
+  pdl_begin();
   typedef typename std::conditional<V == 4, float4, float>::type T;
   for (long long i = V * (blockIdx.x * (long long)blockDim.x + threadIdx.x); i < count;
        i += V * (long long)gridDim.x * blockDim.x) {
@@ -468,6 +478,7 @@ __global__ void adam_kernel(float* theta, float* m, float* v, const float* g, lo
 }
 
 __global__ void unpack_kernel(const float* Y, int n, int bb, zc* g0) {
+  pdl_begin();
   const long long total = (long long)n * bb;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
        i += (long long)gridDim.x * blockDim.x) {
@@ -557,8 +568,8 @@ negf_status gemm(Ctx* ctx, cudaStream_t s, const bf16* A, long long lda, const b
   if ((st = make_map(F, &ma, A, M, K, lda, BM)) != NEGF_OK) return st;
   if ((st = make_map(F, &mb, B, N, K, ldb, tn)) != NEGF_OK) return st;
   const dim3 grid(N / tn, M / BM);
-  if (narrow) bf16_gemm_tn_kernel<BN_NARROW><<<grid, GEMM_THREADS, gemm_smem(BN_NARROW), s>>>(ma, mb, K, ep, ctx->d_err);
-  else bf16_gemm_tn_kernel<BN><<<grid, GEMM_THREADS, gemm_smem(BN), s>>>(ma, mb, K, ep, ctx->d_err);
+  if (narrow) launch_pdl(bf16_gemm_tn_kernel<BN_NARROW>, grid, GEMM_THREADS, gemm_smem(BN_NARROW), s, ma, mb, K, ep, ctx->d_err);
+  else launch_pdl(bf16_gemm_tn_kernel<BN>, grid, GEMM_THREADS, gemm_smem(BN), s, ma, mb, K, ep, ctx->d_err);
   MLAUNCH();
   return NEGF_OK;
 }
@@ -641,11 +652,11 @@ negf_status forward_pass(Ctx* ctx, cudaStream_t s, const negf_mlp_dims* d, const
                          long long np_, const MlpBuffers& B, bool keep) {
   const Fail F{ctx};
   const long long H = d->hidden, K0 = d->k0p, NO = d->nout;
-  cvt_bf16_kernel<<<grid_for(H * K0, 256), 256, 0, s>>>(params + d->off_W1, B.W1b, H * K0);
+  launch_pdl(cvt_bf16_kernel, grid_for(H * K0, 256), 256, 0, s, params + d->off_W1, B.W1b, H * K0);
   MLAUNCH();
-  cvt_bf16_kernel<<<grid_for(H * H, 256), 256, 0, s>>>(params + d->off_W2, B.W2b, H * H);
+  launch_pdl(cvt_bf16_kernel, grid_for(H * H, 256), 256, 0, s, params + d->off_W2, B.W2b, H * H);
   MLAUNCH();
-  cvt_bf16_kernel<<<grid_for(NO * H, 256), 256, 0, s>>>(params + d->off_W3, B.W3b, NO * H);
+  launch_pdl(cvt_bf16_kernel, grid_for(NO * H, 256), 256, 0, s, params + d->off_W3, B.W3b, NO * H);
   MLAUNCH();
   negf_status st;
   Epi e = epi0();
@@ -709,7 +720,7 @@ negf_status negf_mlp_pack(negf_ctx* c, int32_t b, int32_t n, int32_t nlead, cons
   if (!H00 || !H01 || !lead || !E || !X) return F(NEGF_ERR_ARG, "NULL pointer argument");
   MCU(cudaSetDevice(ctx->device));
   const long long np_ = round_up(n, BM);
-  pack_kernel<<<(unsigned)np_, 256, 0, (cudaStream_t)stream>>>(b, n, nlead, (const zc*)H00, (const zc*)H01, lead,
+  launch_pdl(pack_kernel, (unsigned)np_, 256, 0, (cudaStream_t)stream, b, n, nlead, (const zc*)H00, (const zc*)H01, lead,
                                                                 E, (unsigned short*)X, d.k0p, ctx->d_err);
   MLAUNCH();
   return NEGF_OK;
@@ -732,7 +743,7 @@ negf_status negf_mlp_forward(negf_ctx* c, const negf_mlp_dims* dims, const float
   cudaStream_t s = (cudaStream_t)stream;
   if ((st = forward_pass(ctx, s, dims, params, (const bf16*)X, np_, B, false)) != NEGF_OK) return st;
   const long long bb = (long long)dims->b * dims->b;
-  unpack_kernel<<<grid_for(n * bb, 256), 256, 0, s>>>(B.Y, n, (int)bb, (zc*)g0);
+  launch_pdl(unpack_kernel, grid_for(n * bb, 256), 256, 0, s, B.Y, n, (int)bb, (zc*)g0);
   MLAUNCH();
   return NEGF_OK;
 }
@@ -762,7 +773,7 @@ negf_status negf_mlp_train_step(negf_ctx* c, const negf_mlp_dims* dims, float* p
   dim3 tb(32, 8);
   const bf16* Xb = (const bf16*)X;
   if (rows) {   // the minibatch rows of a larger sample set
-    gather_rows_kernel<<<(unsigned)np_, 256, 0, s>>>((const uint4*)X, rows, n, n_set, (int)(K0 / 8), (uint4*)B.Xg,
+    launch_pdl(gather_rows_kernel, (unsigned)np_, 256, 0, s, (const uint4*)X, rows, n, n_set, (int)(K0 / 8), (uint4*)B.Xg,
                                                      ctx->d_err);
     MLAUNCH();
     Xb = B.Xg;
@@ -770,23 +781,23 @@ negf_status negf_mlp_train_step(negf_ctx* c, const negf_mlp_dims* dims, float* p
 
   // ---- forward (keeping Z1, Z2 and the transposed activations)
   if ((st = forward_pass(ctx, s, dims, params, Xb, np_, B, true)) != NEGF_OK) return st;
-  transpose_bf16_kernel<<<dim3((unsigned)(K0 / 32), (unsigned)(np_ / 32)), tb, 0, s>>>(Xb, B.XT, (int)np_, (int)K0);
+  launch_pdl(transpose_bf16_kernel, dim3((unsigned)(K0 / 32), (unsigned)(np_ / 32)), tb, 0, s, Xb, B.XT, (int)np_, (int)K0);
   MLAUNCH();
-  cvt_transpose_kernel<<<dim3((unsigned)(H / 32), (unsigned)(H / 32)), tb, 0, s>>>(params + dims->off_W2, B.W2T,
+  launch_pdl(cvt_transpose_kernel, dim3((unsigned)(H / 32), (unsigned)(H / 32)), tb, 0, s, params + dims->off_W2, B.W2T,
                                                                                    (int)H, (int)H);
   MLAUNCH();
-  cvt_transpose_kernel<<<dim3((unsigned)(H / 32), (unsigned)(NO / 32)), tb, 0, s>>>(params + dims->off_W3, B.W3T,
+  launch_pdl(cvt_transpose_kernel, dim3((unsigned)(H / 32), (unsigned)(NO / 32)), tb, 0, s, params + dims->off_W3, B.W3T,
                                                                                     (int)NO, (int)H);
   MLAUNCH();
 
   // ---- loss and dY = 2 (Y - T) / (n NOUT)
   const double count = (double)n * (double)NO;
-  loss_kernel<<<LOSS_BLOCKS, 256, 0, s>>>(B.Y, (const zc*)g_target, rows, rows ? n_set : n, n, (int)np_, (int)NO,
+  launch_pdl(loss_kernel, LOSS_BLOCKS, 256, 0, s, B.Y, (const zc*)g_target, rows, rows ? n_set : n, n, (int)np_, (int)NO,
                                           2.0 / count, B.dY32, B.dYb, B.partial);
   MLAUNCH();
-  loss_final_kernel<<<1, 32, 0, s>>>(B.partial, LOSS_BLOCKS, 1.0 / count, loss);
+  launch_pdl(loss_final_kernel, 1, 32, 0, s, B.partial, LOSS_BLOCKS, 1.0 / count, loss);
   MLAUNCH();
-  transpose_bf16_kernel<<<dim3((unsigned)(NO / 32), (unsigned)(np_ / 32)), tb, 0, s>>>(B.dYb, B.dYT, (int)np_,
+  launch_pdl(transpose_bf16_kernel, dim3((unsigned)(NO / 32), (unsigned)(np_ / 32)), tb, 0, s, B.dYb, B.dYT, (int)np_,
                                                                                        (int)NO);
   MLAUNCH();
 
@@ -794,7 +805,7 @@ negf_status negf_mlp_train_step(negf_ctx* c, const negf_mlp_dims* dims, float* p
   Epi e = epi0();
   e.c32 = grad + dims->off_W3; e.ldc32 = (int)H;
   if ((st = gemm(ctx, s, B.dYT, np_, B.H2T, np_, (int)NO, (int)H, (int)np_, e)) != NEGF_OK) return st;
-  colsum_kernel<<<(unsigned)((NO + 31) / 32), 32 * CS_WARPS, 0, s>>>(B.dY32, (int)NO, n, (int)NO, grad + dims->off_c3);
+  launch_pdl(colsum_kernel, (unsigned)((NO + 31) / 32), 32 * CS_WARPS, 0, s, B.dY32, (int)NO, n, (int)NO, grad + dims->off_c3);
   MLAUNCH();
   e = epi0();
   e.c32 = B.dZ2; e.ldc32 = (int)H;
@@ -807,7 +818,7 @@ negf_status negf_mlp_train_step(negf_ctx* c, const negf_mlp_dims* dims, float* p
   e = epi0();
   e.c32 = grad + dims->off_W2; e.ldc32 = (int)H;
   if ((st = gemm(ctx, s, B.dZ2T, np_, B.H1T, np_, (int)H, (int)H, (int)np_, e)) != NEGF_OK) return st;
-  colsum_kernel<<<(unsigned)((H + 31) / 32), 32 * CS_WARPS, 0, s>>>(B.dZ2, (int)H, n, (int)H, grad + dims->off_c2);
+  launch_pdl(colsum_kernel, (unsigned)((H + 31) / 32), 32 * CS_WARPS, 0, s, B.dZ2, (int)H, n, (int)H, grad + dims->off_c2);
   MLAUNCH();
   e = epi0();
   e.c32 = B.dZ1; e.ldc32 = (int)H;
@@ -819,7 +830,7 @@ negf_status negf_mlp_train_step(negf_ctx* c, const negf_mlp_dims* dims, float* p
   e = epi0();
   e.c32 = grad + dims->off_W1; e.ldc32 = (int)K0;
   if ((st = gemm(ctx, s, B.dZ1T, np_, B.XT, np_, (int)H, (int)K0, (int)np_, e)) != NEGF_OK) return st;
-  colsum_kernel<<<(unsigned)((H + 31) / 32), 32 * CS_WARPS, 0, s>>>(B.dZ1, (int)H, n, (int)H, grad + dims->off_c1);
+  launch_pdl(colsum_kernel, (unsigned)((H + 31) / 32), 32 * CS_WARPS, 0, s, B.dZ1, (int)H, n, (int)H, grad + dims->off_c1);
   MLAUNCH();
 
   // ---- Adam
@@ -829,10 +840,10 @@ negf_status negf_mlp_train_step(negf_ctx* c, const negf_mlp_dims* dims, float* p
     const float c2 = (float)(1.0 / (1.0 - pow(b2, (double)step)));
     auto aligned = [](const void* p) { return ((uintptr_t)p & 15) == 0; };
     if (dims->n_params % 4 == 0 && aligned(params) && aligned(adam_m) && aligned(adam_v) && aligned(grad))
-      adam_kernel<4><<<grid_for(dims->n_params / 4, 256), 256, 0, s>>>(params, adam_m, adam_v, grad, dims->n_params, lr,
+      launch_pdl(adam_kernel<4>, grid_for(dims->n_params / 4, 256), 256, 0, s, params, adam_m, adam_v, grad, dims->n_params, lr,
                                                                        (float)b1, (float)b2, 1e-8f, c1, c2);
     else
-      adam_kernel<1><<<grid_for(dims->n_params, 256), 256, 0, s>>>(params, adam_m, adam_v, grad, dims->n_params, lr,
+      launch_pdl(adam_kernel<1>, grid_for(dims->n_params, 256), 256, 0, s, params, adam_m, adam_v, grad, dims->n_params, lr,
                                                                    (float)b1, (float)b2, 1e-8f, c1, c2);
     MLAUNCH();
   }

@@ -175,6 +175,7 @@ struct AsmArgs {
 // (then z S - H = E S + W for z = E + i eta, and the conjugate transpose of E S_up + Wl
 // is z S_up^H - H_up^H)
 __global__ void asm_w_kernel(DevView dv, zc* Wd, zc* Wu, zc* Wl) {
+  pdl_begin();
   const int i = blockIdx.y, b = dv.b, nb = dv.nb;
   const int bb = b * b;
   const double eta = dv.eta;
@@ -401,6 +402,7 @@ __global__ void add_kernel(BMat D, BMat A, BMat B, int n, const int* act) {
 
 // R = I - R  (R holds M X on entry)
 __global__ void one_minus_kernel(BMat R, int n, const int* act) {
+  pdl_begin();
   const int u = blockIdx.y;
   if (act && !act[u]) return;
   const long long nn = (long long)n * n;
@@ -579,7 +581,7 @@ struct Engine {
       if (e != cudaSuccess) return e;
       if (!fused) {
         ++ctx->launches;
-        one_minus_kernel<<<grid, 256, 0, s>>>(T1, n, active);             // I - M X
+        launch_pdl(one_minus_kernel, grid, 256, 0, s, T1, n, active);             // I - M X
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
       }
       if (mixed == 1 && ozt_scratch && oz_supported(n)) {
@@ -869,6 +871,7 @@ cudaError_t bcopy(BMat dst, BMat src, int n, int units, cudaStream_t s) {
 
 // status[e] = the worst (most negative) code of the units e*P .. e*P+P-1
 __global__ void status_merge_kernel(int32_t* status, const int32_t* st_units, int U, int P) {
+  pdl_begin();
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= U) return;
   int32_t w = status[e];
@@ -1038,7 +1041,7 @@ negf_status rgf_partitioned_chunk(Ctx* ctx, Engine& eng, const DevView& dv, cons
   }
   if (st) {
     ++ctx->launches;
-    status_merge_kernel<<<(U + 127) / 128, 128, 0, s>>>(st, st_units, U, P);
+    launch_pdl(status_merge_kernel, (U + 127) / 128, 128, 0, s, st, st_units, U, P);
     CU(cudaGetLastError());
   }
   return NEGF_OK;
@@ -1059,6 +1062,7 @@ negf_status rgf_partitioned_chunk(Ctx* ctx, Engine& eng, const DevView& dv, cons
 //   G_kk = g_k - (Wt_k G_tk + X_k G_jk)      (the j terms absent for the last block).
 // ---------------------------------------------------------------------------
 __global__ void tip_assemble_kernel(BMat Att, const zc* H_tip, const double* E, double eta, int e0, int n) {
+  pdl_begin();
   const int u = blockIdx.y;
   const zc z = zmake(E[e0 + u], eta);
   const long long nn = (long long)n * n;
@@ -1073,6 +1077,7 @@ __global__ void tip_assemble_kernel(BMat Att, const zc* H_tip, const double* E, 
 
 // the arrow's blocks of A, shared by all energies: row[i] = -H_(t,i), col[i] = -H_(t,i)^H
 __global__ void arrow_blocks_kernel(zc* row, zc* col, const zc* H, int n) {
+  pdl_begin();
   const int i = blockIdx.y;
   const long long nn = (long long)n * n;
   for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < nn; k += (long long)gridDim.x * blockDim.x) {
@@ -1140,7 +1145,7 @@ negf_status rgf_arrowhead_chunk(Ctx* ctx, Engine& eng, const DevView& dv, const 
   CU(cudaMemsetAsync(dDt, 0, blk * (size_t)U, s));
   CU(bcopy(S1(Ft), shared(Arow, 0), b, U, s));                                // F_t0 = A_t0
   CU(bcopy(S1(Fc), shared(Acol, 0), b, U, s));                                // F_0t = A_0t
-  tip_assemble_kernel<<<eg, 256, 0, s>>>(S1(Att), ar.H_tip, dv.E, dv.eta, e0, b);
+  launch_pdl(tip_assemble_kernel, eg, 256, 0, s, S1(Att), ar.H_tip, dv.E, dv.eta, e0, b);
   CU(cudaGetLastError());
   // ---------------- elimination of every device block, the tip kept
   for (int k = 0; k < nb; ++k) {
@@ -1228,6 +1233,7 @@ struct LeadArgs {
 
 // unit u < U: left lead of energy e0+u; u >= U: right lead of energy e0+u-U
 __global__ void lead_init_kernel(LeadArgs a) {
+  pdl_begin();
   const int u = blockIdx.y;
   const bool left = u < a.U;
   const int k = left ? u : u - a.U;   // the energy unit
@@ -1374,6 +1380,7 @@ __global__ void lead_update_kernel(BMat eps, BMat epss, BMat agb, BMat bga, int 
 
 // F = KG - I (in place), res[u] = ||F||_F / sqrt(n); mode 1 stores into resn instead
 __global__ void residual_kernel(BMat F, int n, double* res, const int* active) {
+  pdl_begin();
   const int u = blockIdx.x;
   if (active && !active[u]) return;
   const long long nn = (long long)n * n;
@@ -1545,6 +1552,7 @@ __global__ void __launch_bounds__(1024) balance_kernel(BMat P, BMat Q, int n, co
 // Newton acceptance: if resn < res: g = gn, res = resn
 __global__ void newton_accept_kernel(BMat g, BMat gn, int n, double* res, const double* resn, int* need,
                                      double target, int* steps) {
+  pdl_begin();
   const int u = blockIdx.x;
   if (!need[u]) return;
   const bool take = resn[u] < res[u];
@@ -1564,6 +1572,7 @@ __global__ void newton_accept_kernel(BMat g, BMat gn, int n, double* res, const 
 // attempt (res = inf, so that the retarded-root test rejects it)
 __global__ void newton_take_kernel(BMat g, BMat gn, int n, double* res, const double* resn, int* need,
                                    double target, int* steps) {
+  pdl_begin();
   const int u = blockIdx.x;
   if (!need[u]) return;
   const bool fin = isfinite(resn[u]);
@@ -1587,6 +1596,7 @@ __global__ void newton_take_kernel(BMat g, BMat gn, int n, double* res, const do
 // g[u] = the guess of its side (left units u < U, right units u >= U), warm[u] = 1 when given
 __global__ void guess_init_kernel(BMat g, const zc* g0L, const zc* g0R, int U, int n, int* warm,
                                   const long long* off = nullptr) {
+  pdl_begin();
   const int u = blockIdx.y;
   const bool left = u < U;
   const zc* src = left ? g0L : g0R;
@@ -1600,6 +1610,7 @@ __global__ void guess_init_kernel(BMat g, const zc* g0L, const zc* g0R, int U, i
 }
 
 __global__ void need_warm_kernel(const int* warm, const double* res, int* need, int units, double target) {
+  pdl_begin();
   const int u = blockIdx.x * blockDim.x + threadIdx.x;
   if (u < units) need[u] = (warm[u] && res[u] > target) ? 1 : 0;
 }
@@ -1610,6 +1621,7 @@ __global__ void need_warm_kernel(const int* warm, const double* res, int* need, 
 // skipped).  A is factorised in place in the scratch block W.
 __global__ void retarded_check_kernel(BMat g, BMat W, int n, const int* warm, const double* res, double accept,
                                       double tol, int* keep) {
+  pdl_begin();
   const int u = blockIdx.x;
   if (!warm[u] || !(res[u] <= accept)) {
     if (threadIdx.x == 0) keep[u] = 0;
@@ -1657,6 +1669,7 @@ __global__ void retarded_check_kernel(BMat g, BMat W, int n, const int* warm, co
 }
 
 __global__ void not_kernel(const int* a, int* out, int units) {
+  pdl_begin();
   const int u = blockIdx.x * blockDim.x + threadIdx.x;
   if (u < units) out[u] = a[u] ? 0 : 1;
 }
@@ -1664,6 +1677,7 @@ __global__ void not_kernel(const int* a, int* out, int units) {
 // off[0 .. c-1] = u * bb for the c units with mask[u] != 0, in increasing u (one CTA
 // of 1024 threads: ballots within warps, a scan of the warp counts per tile of 1024)
 __global__ void __launch_bounds__(1024) compact_kernel(const int* mask, int units, long long bb, long long* off) {
+  pdl_begin();
   __shared__ int wsum[32];
   __shared__ int s_base;
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
@@ -1695,6 +1709,7 @@ __global__ void __launch_bounds__(1024) compact_kernel(const int* mask, int unit
 }
 
 __global__ void count_kernel(const int* flags, int units, int* out) {
+  pdl_begin();
   int c = 0;
   for (int u = threadIdx.x; u < units; u += blockDim.x) c += flags[u] != 0;
   for (int off = 16; off > 0; off >>= 1) c += __shfl_down_sync(0xffffffffu, c, off);
@@ -1708,6 +1723,7 @@ __global__ void count_kernel(const int* flags, int units, int* out) {
 }
 
 __global__ void set_need_kernel(const double* res, int* need, int units, double target, const int* only) {
+  pdl_begin();
   const int u = blockIdx.x * blockDim.x + threadIdx.x;
   if (u < units) need[u] = (only[u] && res[u] > target) ? 1 : 0;
 }
@@ -1715,6 +1731,7 @@ __global__ void set_need_kernel(const double* res, int* need, int units, double 
 __global__ void obc_finish_kernel(const int* done, const double* res, const int* iters, const int* nsteps, int U,
                                   int32_t* status, int32_t* iters_out, int32_t* newton_out, double accept,
                                   const int* glob = nullptr) {
+  pdl_begin();
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= U) return;
   const int ge = glob ? glob[e] : e;   // the energy's index in the outputs
@@ -1748,6 +1765,7 @@ __device__ __forceinline__ double block_sum(double v, double* red) {
 
 // Gamma = i (Sigma - Sigma^H)
 __global__ void gamma_kernel(BMat G, BMat Sg, int n) {
+  pdl_begin();
   const int u = blockIdx.y;
   const long long nn = (long long)n * n;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < nn; i += (long long)gridDim.x * blockDim.x) {
@@ -1766,6 +1784,7 @@ __host__ __device__ __forceinline__ int row_tiles(int b) { return (b + TR - 1) /
 
 // out[u nk + o] = scale * sum_k part[(u nk + o) count + k], o < nk: one thread per (u, o)
 __global__ void sum_parts_kernel(const double* part, int nk, int count, int U, double scale, double* out) {
+  pdl_begin();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= U * nk) return;
   double t = 0.0;
@@ -1777,6 +1796,7 @@ __global__ void sum_parts_kernel(const double* part, int nk, int count, int U, d
 // T = Re( Tr[Gam i (G - G^H)] - sum_pq K1_pq conj(K2_pq) ),  K1 = Gam G, K2 = G Gam: the share of
 // rows p of one tile, G's transposed elements through shared memory
 __global__ void __launch_bounds__(256) transmission_kernel(BMat Gam, BMat G, BMat K1, BMat K2, int n, double* part) {
+  pdl_begin();
   const int u = blockIdx.y, r0 = blockIdx.x * TR;
   const zc *gm = Gam.at(u), *g = G.at(u), *k1 = K1.at(u), *k2 = K2.at(u);
   __shared__ zc sm[32][33];
@@ -1845,6 +1865,7 @@ __device__ __forceinline__ double warp_sum(double v) {
 // (G_ii S_ii and, below the last block, G_{i,i+1} S_{i+1,i} + G_{i+1,i} S_{i,i+1}), by row tiles
 __global__ void __launch_bounds__(256) dos_part_kernel(DevView dv, const zc* GRd, const zc* GRu, const zc* GRl, int e0,
                                                        int eg, double* part) {
+  pdl_begin();
   const int nb = dv.nb, b = dv.b, nt = row_tiles(b);
   const int i = blockIdx.x / nt, r0 = (blockIdx.x - i * nt) * TR, u = blockIdx.y;
   const int eb = e0 + u - eg;   // the energy's place in the G buffers
@@ -1881,6 +1902,7 @@ __global__ void __launch_bounds__(256) dos_part_kernel(DevView dv, const zc* GRd
 
 // J_i(E) = 2 Re Tr[(H_{i,i+1} - z S_{i,i+1}) G^<_{i+1,i}], by row tiles of G^<
 __global__ void __launch_bounds__(256) current_kernel(DevView dv, const zc* GLl, int e0, int eg, double* part) {
+  pdl_begin();
   const int nb = dv.nb, b = dv.b, nt = row_tiles(b);
   const int i = blockIdx.x / nt, r0 = (blockIdx.x - i * nt) * TR, u = blockIdx.y, e = e0 + u;
   const long long bb = (long long)b * b;
@@ -1908,6 +1930,7 @@ __global__ void __launch_bounds__(256) current_kernel(DevView dv, const zc* GLl,
 // nb*b, by row tiles
 __global__ void __launch_bounds__(256) density_energy_kernel(DevView dv, const zc* GLd, const zc* GLl, int e0, int eg,
                                                              double* nE) {
+  pdl_begin();
   const int nb = dv.nb, b = dv.b, nt = row_tiles(b);
   const int i = blockIdx.x / nt, r0 = (blockIdx.x - i * nt) * TR, u = blockIdx.y;
   const int e = e0 + u - eg;   // the energy's place in the G buffers
@@ -1948,6 +1971,7 @@ __global__ void __launch_bounds__(256) density_energy_kernel(DevView dv, const z
 
 // density[k] += sum_u w[e0+u] nE[u][k]  (fixed order over u)
 __global__ void density_accum_kernel(const double* nE, const double* w, int e0, int U, long long N, double* dens) {
+  pdl_begin();
   for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < N; k += (long long)gridDim.x * blockDim.x) {
     double acc = dens[k];
 #pragma unroll 8
@@ -1987,39 +2011,39 @@ negf_status observables_chunk(Ctx* ctx, Engine& eng, const DevView& dv, const Ob
     BMat Sg{(zc*)ob.sigma_L + (long long)e0 * bb, bb};
     BMat G00{(zc*)ob.GRd + (long long)(e0 - eg) * nb * bb, (long long)nb * bb};
     dim3 grid((unsigned)std::min<long long>((bb + 255) / 256, 1024), U);
-    gamma_kernel<<<grid, 256, 0, s>>>(Gam, Sg, b);
+    launch_pdl(gamma_kernel, grid, 256, 0, s, Gam, Sg, b);
     KCHECK();
     CU(eng.gemm(K1, Gam, OP_N, G00, OP_N, ONE, NOMAT, ZERO, b, U));
     CU(eng.gemm(K2, G00, OP_N, Gam, OP_N, ONE, NOMAT, ZERO, b, U));
     // the shares after the three blocks of every unit (the products are done with their scratch)
     double* part = (double*)(p + 3LL * U * bb);
     double* T = ob.T + e0;
-    transmission_kernel<<<dim3(nt, U), 256, 0, s>>>(Gam, G00, K1, K2, b, nt > 1 ? part : T);
+    launch_pdl(transmission_kernel, dim3(nt, U), 256, 0, s, Gam, G00, K1, K2, b, nt > 1 ? part : T);
     KCHECK();
     if (nt > 1) {
-      sum_parts_kernel<<<(U + 63) / 64, 64, 0, s>>>(part, 1, nt, U, 1.0, T);
+      launch_pdl(sum_parts_kernel, (U + 63) / 64, 64, 0, s, part, 1, nt, U, 1.0, T);
       KCHECK();
     }
   }
   if (ob.dos) {
     double* part = (double*)ws;   // [U][nb nt] shares (ws holds >= N = nb b doubles per energy)
-    dos_part_kernel<<<dim3(nb * nt, U), 256, 0, s>>>(dv, ob.GRd, ob.GRu, ob.GRl, e0, eg, part);
+    launch_pdl(dos_part_kernel, dim3(nb * nt, U), 256, 0, s, dv, ob.GRd, ob.GRu, ob.GRl, e0, eg, part);
     KCHECK();
-    sum_parts_kernel<<<(U + 63) / 64, 64, 0, s>>>(part, 1, nb * nt, U, -1.0 / M_PI, ob.dos + e0);
+    launch_pdl(sum_parts_kernel, (U + 63) / 64, 64, 0, s, part, 1, nb * nt, U, -1.0 / M_PI, ob.dos + e0);
     KCHECK();
   }
   if (ob.current && nb > 1) {
     double* part = (double*)ws;   // [U][nb - 1][nt]
-    current_kernel<<<dim3((nb - 1) * nt, U), 256, 0, s>>>(dv, ob.GLl, e0, eg, part);
+    launch_pdl(current_kernel, dim3((nb - 1) * nt, U), 256, 0, s, dv, ob.GLl, e0, eg, part);
     KCHECK();
-    sum_parts_kernel<<<(U * (nb - 1) + 63) / 64, 64, 0, s>>>(part, nb - 1, nt, U, 2.0, ob.current + (long long)e0 * (nb - 1));
+    launch_pdl(sum_parts_kernel, (U * (nb - 1) + 63) / 64, 64, 0, s, part, nb - 1, nt, U, 2.0, ob.current + (long long)e0 * (nb - 1));
     KCHECK();
   }
   if (ob.density) {
     double* nE = (double*)ws;
-    density_energy_kernel<<<dim3(nb * nt, U), 256, 0, s>>>(dv, ob.GLd, ob.GLl, e0, eg, nE);
+    launch_pdl(density_energy_kernel, dim3(nb * nt, U), 256, 0, s, dv, ob.GLd, ob.GLl, e0, eg, nE);
     KCHECK();
-    density_accum_kernel<<<(unsigned)std::min<long long>((N + 255) / 256, 1024), 256, 0, s>>>(nE, ob.w, e0, U, N,
+    launch_pdl(density_accum_kernel, (unsigned)std::min<long long>((N + 255) / 256, 1024), 256, 0, s, nE, ob.w, e0, U, N,
                                                                                                 ob.density);
     KCHECK();
   }
@@ -2127,6 +2151,7 @@ negf_status negf_layout(const negf_system* sys, int64_t* out) {
 
 // status[glob[u]] = st_units[u]
 __global__ void status_scatter_kernel(int32_t* status, const int32_t* st_units, const int* glob, int U) {
+  pdl_begin();
   const int u = blockIdx.x * blockDim.x + threadIdx.x;
   if (u < U) status[glob[u]] = st_units[u];
 }
@@ -2223,7 +2248,7 @@ negf_status rgf_batched_group(Ctx* ctx, Engine& eng, const negf_system* sys, con
     if (st != NEGF_OK) return st;
     if (status) {
       ++ctx->launches;
-      status_scatter_kernel<<<(U + 127) / 128, 128, 0, s>>>(status, bp.st_units, glob, U);
+      launch_pdl(status_scatter_kernel, (U + 127) / 128, 128, 0, s, status, bp.st_units, glob, U);
       CU(cudaGetLastError());
     }
   }
@@ -2305,7 +2330,7 @@ static negf_status rgf_common(Ctx* ctx, const negf_system* sys, negf_precision p
       zc* W = (zc*)ctx->ws;
       const long long bb = (long long)dv.b * dv.b;
       ++ctx->launches;
-      asm_w_kernel<<<dim3((unsigned)std::min<long long>((bb + 255) / 256, 1024), dv.nb), 256, 0, s>>>(
+      launch_pdl(asm_w_kernel, dim3((unsigned)std::min<long long>((bb + 255) / 256, 1024), dv.nb), 256, 0, s, 
           dv, W, W + dv.nb * bb, W + (2LL * dv.nb - 1) * bb);
       CU(cudaGetLastError());
       io.W = W;
@@ -2552,7 +2577,7 @@ negf_status negf_rgf_arrowhead(negf_ctx* c, const negf_system* sys, negf_precisi
       return fail(ctx, NEGF_ERR_NOMEM, "workspace too small: one energy of this device needs " + std::to_string(per) + " bytes");
     chunk = std::min(chunk, ne);
     ++ctx->launches;
-    arrow_blocks_kernel<<<dim3((unsigned)std::min<long long>((bb + 255) / 256, 1024), nb), 256, 0, s>>>(
+    launch_pdl(arrow_blocks_kernel, dim3((unsigned)std::min<long long>((bb + 255) / 256, 1024), nb), 256, 0, s, 
         Arow, Acol, ar.H_arrow, b);
     CU(cudaGetLastError());
     for (int e0 = 0; e0 < ne; e0 += chunk) {
@@ -2708,7 +2733,7 @@ negf_status negf_obc(negf_ctx* c, const negf_system* sys, negf_precision prec, d
         ctx->launches += 2;
         CU(obc_small(q, s));
         const long long ob = batched ? 0 : o[2] + e0;
-        obc_finish_kernel<<<(U + 127) / 128, 128, 0, s>>>(
+        launch_pdl(obc_finish_kernel, (U + 127) / 128, 128, 0, s, 
             done, res, it_arr, nsteps, U, status ? status + ob : nullptr, iters ? iters + 2 * ob : nullptr,
             newton ? newton + 2 * ob : nullptr, accept, t_glob);
         CU(cudaGetLastError());
@@ -2720,7 +2745,7 @@ negf_status negf_obc(negf_ctx* c, const negf_system* sys, negf_precision prec, d
       la.unit_dev = t_dev;
       la.unit_e = t_e;
       dim3 eg((unsigned)std::min<long long>((bb + 255) / 256, 1024), NU);
-      lead_init_kernel<<<eg, 256, 0, s>>>(la);
+      launch_pdl(lead_init_kernel, eg, 256, 0, s, la);
       KCHECK();
       CU(cudaMemsetAsync(nsteps, 0, sizeof(int) * NU, s));
       CU(cudaMemsetAsync(keep, 0, sizeof(int) * NU, s));
@@ -2750,7 +2775,7 @@ negf_status negf_obc(negf_ctx* c, const negf_system* sys, negf_precision prec, d
         CU(eng.gemm(T[0], al0, OP_N, X, OP_N, ONE, NOMAT, ZERO, b, NU, mask));               // al X
         CU(eng.gemm(T[1], T[0], OP_N, be0, OP_N, MONE, a00, ONE, b, NU, mask));              // K = a00 - al X be
         CU(eng.gemm(T[2], T[1], OP_N, X, OP_N, ONE, NOMAT, ZERO, b, NU, mask));              // K X
-        residual_kernel<<<NU, 256, 0, s>>>(T[2], b, out, mask);                              // F = K X - I
+        launch_pdl(residual_kernel, NU, 256, 0, s, T[2], b, out, mask);                              // F = K X - I
         KCHECK();
         return NEGF_OK;
       };
@@ -2763,7 +2788,7 @@ negf_status negf_obc(negf_ctx* c, const negf_system* sys, negf_precision prec, d
         ncomp = 0;
         if (cnt <= 0 || 2 * cnt > NU) return NEGF_OK;
         ++ctx->launches;
-        compact_kernel<<<1, 1024, 0, s>>>(mask, NU, bb, coff);
+        launch_pdl(compact_kernel, 1, 1024, 0, s, mask, NU, bb, coff);
         CU(cudaGetLastError());
         ncomp = cnt;
         return NEGF_OK;
@@ -2781,7 +2806,7 @@ negf_status negf_obc(negf_ctx* c, const negf_system* sys, negf_precision prec, d
       };
       auto n_set = [&](const int* flags) -> int {
         ++ctx->launches;
-        count_kernel<<<1, 256, 0, s>>>(flags, NU, n_active);
+        launch_pdl(count_kernel, 1, 256, 0, s, flags, NU, n_active);
         cudaError_t e = cudaGetLastError();
         if (e == cudaSuccess) e = cudaMemcpyAsync(ctx->h_pinned, n_active, sizeof(int), cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
@@ -2830,25 +2855,25 @@ negf_status negf_obc(negf_ctx* c, const negf_system* sys, negf_precision prec, d
         const long long gb = batched ? 0 : o[3] + (long long)e0 * bb;   // batched: per-unit offsets
         const zc* gl = g0_L ? (const zc*)g0_L + gb : nullptr;
         const zc* gr = g0_R ? (const zc*)g0_R + gb : nullptr;
-        guess_init_kernel<<<eg, 256, 0, s>>>(g, gl, gr, U, b, warm, t_off);
+        launch_pdl(guess_init_kernel, eg, 256, 0, s, g, gl, gr, U, b, warm, t_off);
         KCHECK();
         if ((st = residual(g, res, warm)) != NEGF_OK) return st;
-        need_warm_kernel<<<(NU + 255) / 256, 256, 0, s>>>(warm, res, need, NU, target);
+        launch_pdl(need_warm_kernel, (NU + 255) / 256, 256, 0, s, warm, res, need, NU, target);
         KCHECK();
         for (int step = 0; step < 8; ++step) {
           const int cnt = n_set(need);
           if (cnt < 0) return fail(ctx, NEGF_ERR_CUDA, "OBC: flag read-back failed");
           if (cnt == 0) break;
           if ((st = newton_step(need, eps, cnt)) != NEGF_OK) return st;   // eps is free until the decimation
-          newton_take_kernel<<<NU, 256, 0, s>>>(g, eps, b, res, resn, need, target, nsteps);
+          launch_pdl(newton_take_kernel, NU, 256, 0, s, g, eps, b, res, resn, need, target, nsteps);
           KCHECK();
         }
-        retarded_check_kernel<<<NU, 256, 0, s>>>(g, T[0], b, warm, res, accept, 1e-12, keep);
+        launch_pdl(retarded_check_kernel, NU, 256, 0, s, g, T[0], b, warm, res, accept, 1e-12, keep);
         KCHECK();
-        lead_init_kernel<<<eg, 256, 0, s>>>(la);   // restore the decimation slots
+        launch_pdl(lead_init_kernel, eg, 256, 0, s, la);   // restore the decimation slots
         KCHECK();
       }
-      not_kernel<<<(NU + 255) / 256, 256, 0, s>>>(keep, cold, NU);
+      launch_pdl(not_kernel, (NU + 255) / 256, 256, 0, s, keep, cold, NU);
       KCHECK();
       const int n_cold = any_warm ? n_set(cold) : NU;
       if (n_cold < 0) return fail(ctx, NEGF_ERR_CUDA, "OBC: flag read-back failed");
@@ -2891,7 +2916,7 @@ negf_status negf_obc(negf_ctx* c, const negf_system* sys, negf_precision prec, d
         if ((st = lead_inverse(g, epss, any_warm ? cold : nullptr)) != NEGF_OK) return st;
         if ((st = residual(g, res, any_warm ? cold : nullptr)) != NEGF_OK) return st;
         // ---- Newton polishing of the decimation result above the target
-        set_need_kernel<<<(NU + 255) / 256, 256, 0, s>>>(res, need, NU, target, cold);
+        launch_pdl(set_need_kernel, (NU + 255) / 256, 256, 0, s, res, need, NU, target, cold);
         KCHECK();
         BMat gn = eps;   // decimation slots are free now
         for (int step = 0; step < 3; ++step) {
@@ -2899,7 +2924,7 @@ negf_status negf_obc(negf_ctx* c, const negf_system* sys, negf_precision prec, d
           if (cnt < 0) return fail(ctx, NEGF_ERR_CUDA, "OBC: flag read-back failed");
           if (cnt == 0) break;
           if ((st = newton_step(need, gn, cnt)) != NEGF_OK) return st;
-          newton_accept_kernel<<<NU, 256, 0, s>>>(g, gn, b, res, resn, need, target, nsteps);
+          launch_pdl(newton_accept_kernel, NU, 256, 0, s, g, gn, b, res, resn, need, target, nsteps);
           KCHECK();
           // units that took the step continue from T1/T2 (K, F of the accepted g)
         }
@@ -2918,7 +2943,7 @@ negf_status negf_obc(negf_ctx* c, const negf_system* sys, negf_precision prec, d
       CU(eng.gemm(lead_out(sigma_R), BMat{T[0].p + (long long)U * bb, bb}, OP_N,
                   BMat{be0.p + (long long)U * bb, bb}, OP_N, ONE, NOMAT, ZERO, b, U));
       const long long ob = batched ? 0 : o[2] + e0;   // batched: per-unit energy indices
-      obc_finish_kernel<<<(U + 127) / 128, 128, 0, s>>>(
+      launch_pdl(obc_finish_kernel, (U + 127) / 128, 128, 0, s, 
           done, res, it_arr, nsteps, U, status ? status + ob : nullptr, iters ? iters + 2 * ob : nullptr,
           newton ? newton + 2 * ob : nullptr, accept, t_glob);
       KCHECK();
@@ -3045,7 +3070,7 @@ negf_status negf_rgf_observables(negf_ctx* c, const negf_system* sys, negf_preci
     if (use_w) {
       zc* W = (zc*)ctx->ws;
       ++ctx->launches;
-      asm_w_kernel<<<dim3((unsigned)std::min<long long>((bb + 255) / 256, 1024), nb), 256, 0, s>>>(
+      launch_pdl(asm_w_kernel, dim3((unsigned)std::min<long long>((bb + 255) / 256, 1024), nb), 256, 0, s, 
           dv, W, W + nb * bb, W + (2LL * nb - 1) * bb);
       CU(cudaGetLastError());
       io.W = W;

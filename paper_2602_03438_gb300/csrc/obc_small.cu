@@ -40,6 +40,7 @@ __device__ __forceinline__ double cta_reduce(double v, double* red) {
 }
 
 __global__ void __launch_bounds__(small_threads(kObcSmallB)) obc_small_kernel(ObcSmall a) {
+  pdl_begin();
   const int u = blockIdx.x, b = a.b;
   const bool left = u < a.U;
   const int k = left ? u : u - a.U;   // the energy unit
@@ -216,7 +217,7 @@ cudaError_t obc_small(const ObcSmall& a, cudaStream_t s) {
                                 (int)obc_small_smem(kObcSmallB));
   });
   if (e != cudaSuccess) return e;
-  obc_small_kernel<<<2 * a.U, small_threads(a.b), obc_small_smem(a.b), s>>>(a);
+  launch_pdl(obc_small_kernel, 2 * a.U, small_threads(a.b), obc_small_smem(a.b), s, a);
   return cudaGetLastError();
 }
 

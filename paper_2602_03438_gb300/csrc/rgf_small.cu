@@ -28,6 +28,7 @@ namespace {
 constexpr int kBufs = 13;
 
 __global__ void __launch_bounds__(small_threads(kSmallB)) rgf_small_kernel(SmallSweep a) {
+  pdl_begin();
   const int u = blockIdx.x;
   const int b = a.b, nb = a.nb;
   const long long bb = (long long)b * b;
@@ -148,7 +149,7 @@ cudaError_t rgf_small_sweep(const SmallSweep& a, cudaStream_t s) {
                                 (int)rgf_small_smem(kSmallB));
   });
   if (e != cudaSuccess) return e;
-  rgf_small_kernel<<<a.U, small_threads(a.b), smem, s>>>(a);
+  launch_pdl(rgf_small_kernel, a.U, small_threads(a.b), smem, s, a);
   return cudaGetLastError();
 }
 

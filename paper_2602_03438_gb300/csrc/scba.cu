@@ -25,6 +25,7 @@ __device__ __forceinline__ zc cmul(zc a, zc b) { return zmake(a.x * b.x - a.y * 
 
 // spectrum of the wrapped kernel: Wh[k] = sum_m w_m exp(-2 pi i k m / N)
 __global__ void kernel_spectrum_kernel(const double* w, int M, int N, zc* Wh) {
+  pdl_begin();
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= N) return;
   double re = 0.0, im = 0.0;
@@ -44,6 +45,7 @@ __global__ void kernel_spectrum_kernel(const double* w, int M, int N, zc* Wh) {
 // one CTA: TE elements (columns) x N energies (rows) in shared memory
 __global__ void __launch_bounds__(256) energy_conv_kernel(const zc* __restrict__ X, zc* __restrict__ Y, long long ld,
                                                           int nelem, int ne, int logn, int TE, const zc* __restrict__ Wh) {
+  pdl_begin();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int N = 1 << logn;
   zc* a = reinterpret_cast<zc*>(smem_raw);      // [TE][N]
@@ -112,6 +114,7 @@ __device__ __forceinline__ void atomic_max_nonneg(double* addr, double v) {
 // SR = (SG - SL) / 2
 __global__ void scba_mix_kernel(zc* SL, zc* SG, zc* SR, const zc* SLn, const zc* SGn, long long n, double mix,
                                 double* stats) {
+  pdl_begin();
   double dl = 0.0, dg = 0.0, sc = 0.0;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
     const zc l = SL[i], g = SG[i], ln = SLn[i], gn = SGn[i];
@@ -151,14 +154,14 @@ cudaError_t energy_convolution(const zc* X, zc* Y, long long ld, int nelem, int 
   const int logn = conv_log2_size(ne, M);
   const int N = 1 << logn;
   if (logn > 13) return cudaErrorInvalidValue;   // N <= 8192: one column fits shared memory
-  kernel_spectrum_kernel<<<(N + 255) / 256, 256, 0, s>>>(w_dev, M, N, Wh);
+  launch_pdl(kernel_spectrum_kernel, (N + 255) / 256, 256, 0, s, w_dev, M, N, Wh);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const int TE = std::max(1, std::min(8, 8192 / N));
   const size_t smem = sizeof(zc) * ((size_t)TE * N + N / 2);
   e = cudaFuncSetAttribute(energy_conv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  energy_conv_kernel<<<(nelem + TE - 1) / TE, 256, smem, s>>>(X, Y, ld, nelem, ne, logn, TE, Wh);
+  launch_pdl(energy_conv_kernel, (nelem + TE - 1) / TE, 256, smem, s, X, Y, ld, nelem, ne, logn, TE, Wh);
   return cudaGetLastError();
 }
 
@@ -167,7 +170,7 @@ cudaError_t scba_mix(zc* SL, zc* SG, zc* SR, const zc* SLn, const zc* SGn, long 
   cudaError_t e = cudaMemsetAsync(stats, 0, 3 * sizeof(double), s);
   if (e != cudaSuccess || n <= 0) return e;
   const int blocks = (int)std::min<long long>((n + 255) / 256, 4096);
-  scba_mix_kernel<<<blocks, 256, 0, s>>>(SL, SG, SR, SLn, SGn, n, mix, stats);
+  launch_pdl(scba_mix_kernel, blocks, 256, 0, s, SL, SG, SR, SLn, SGn, n, mix, stats);
   return cudaGetLastError();
 }
 
