@@ -60,3 +60,31 @@ def test_lead_solver_scales_with_powers_of_two(P, b):
                 assert np.abs(x / f - y).max() <= 1e-12 * np.abs(y).max(), k
     finally:
         ctx.close()
+
+
+@pytest.mark.parametrize("b,ne", [(17, 2), (17, 300), (17, 1030), (40, 260)])
+def test_masked_products_of_many_units(P, b, ne):
+    """Mixed precision against FP64: the products under a mask take a list of its units, in one
+    round of 512 flags, in several, and (more than 2048 units) by skipping.  Both sides meet
+    the residual target of 1e-13 that the fixed point amplifies by at most 1 / eta^2 = 1e4."""
+    dev = W.banded_device(2, b, ne, b, overlap=False)
+    rng = np.random.default_rng(b)
+    dev.H_up = dev.H_up + 0.3 / np.sqrt(b) * (rng.normal(size=dev.H_up.shape) + 1j * rng.normal(size=dev.H_up.shape))
+    dev.eta = 1e-2
+    sys_ = P.upload([dev])
+    out = []
+    ctx = P.Context(0, 3 << 30)
+    try:
+        for prec in (P.FP64, P.MIXED):
+            z = lambda: torch.empty(ne * b * b, dtype=torch.complex128, device="cuda")
+            sL, sR = z(), z()
+            status = torch.full((ne,), 9, dtype=torch.int32, device="cuda")
+            iters = torch.zeros(2 * ne, dtype=torch.int32, device="cuda")
+            P.negf_obc(ctx, sys_, sL, sR, iters, status, prec=prec)
+            assert ctx.sync() == 0
+            assert int(status.abs().sum()) == 0
+            out.append(torch.stack([sL, sR]).view(2, ne, -1))
+    finally:
+        ctx.close()
+    size = out[0].abs().amax(dim=2, keepdim=True)
+    assert float(((out[1] - out[0]).abs() / size).max()) <= 2e-9
