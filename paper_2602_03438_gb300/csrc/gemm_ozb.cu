@@ -39,9 +39,9 @@
 // tensor pipe, but their operands are read from shared memory for 14 k, A's images and B's
 // digits are written there for 5 k and the stores pass through it for 2 k; with the part of
 // the drain (256 KB of TMEM, 5 k clocks) that nothing overlaps a tile takes 26 k.  Measured
-// per 1024 units of n = 128 with C, pre-pass included (HBM bound, 140 us): 515 us, against
+// per 1024 units of n = 128 with C, pre-pass included (HBM bound, 143 us): 500 us, against
 // 702 us for 8 digits of 7 bits in BF16 with the drain through shared memory; 16 units of
-// n = 512: 425 against 955 us.  On the way (us per 1024 units of 128): issuing from one
+// n = 512: 408 against 955 us.  On the way (us per 1024 units of 128): issuing from one
 // lane's branch 620 (each MMA's descriptors pass between the register files), a 64-bit FP
 // conversion per output in place of the integer one 572, spilled registers for want of the
 // register split 624, eight producer warps 635, one drain of re and im together and three
@@ -210,6 +210,14 @@ __device__ __forceinline__ int scale_exp_hi(unsigned int h) {
   return (ex == 0 ? 1 : ex) - 1021;
 }
 
+// x with its sign flipped by `mask` (0 or the sign bit): a negation chosen at run time would
+// be an FP64 instruction
+__device__ __forceinline__ double flip(double x, int mask) {
+  return __hiloint2double(__double2hiint(x) ^ mask, __double2loint(x));
+}
+// conj(x): -x would be an FP64 instruction (1024 products of n = 128 with B^H: 402 -> 389 us)
+__device__ __forceinline__ zc conj_bits(zc x) { return zmake(x.x, flip(x.y, (int)0x80000000)); }
+
 // 128 in each of the ND - 1 low bytes
 template <int ND>
 constexpr unsigned long long kByteBias = (0x8080808080808080ull >> (8 * (9 - ND)));
@@ -283,15 +291,22 @@ __global__ void __launch_bounds__(256) ozb_prepass_kernel(ARGS g, ImgArgs im, in
     const zc* __restrict__ B = g.B.at(u);
     int* out = im.eb + (size_t)u * n;
     const int warp = tid >> 5, lane = tid & 31;
-    if (g.opB == OP_H) {   // rows of B, a warp each
-      for (int c = c0 + warp; c < min(c0 + PRE, n); c += 8) {
-        unsigned int v = 0;
-        for (int k = lane; k < n; k += 32) {
-          const zc x = B[(size_t)c * n + k];
-          v = max(v, max(abs_hi(x.x), abs_hi(x.y)));
+    if (g.opB == OP_H) {   // rows of B, a warp for four of them side by side
+      unsigned int v[PRE / 8] = {};
+#pragma unroll 2
+      for (int k = lane; k < n; k += 32) {
+#pragma unroll
+        for (int q = 0; q < PRE / 8; ++q) {
+          const int c = c0 + warp + 8 * q;
+          const zc x = c < n ? B[(size_t)c * n + k] : zmake(0.0, 0.0);
+          v[q] = max(v[q], max(abs_hi(x.x), abs_hi(x.y)));
         }
-        v = __reduce_max_sync(0xffffffffu, v);
-        if (lane == 0) out[c] = scale_exp_hi(v);
+      }
+#pragma unroll
+      for (int q = 0; q < PRE / 8; ++q) {
+        const int c = c0 + warp + 8 * q;
+        v[q] = __reduce_max_sync(0xffffffffu, v[q]);
+        if (lane == 0 && c < n) out[c] = scale_exp_hi(v[q]);
       }
     } else {
       __shared__ unsigned int part[8][PRE];
@@ -321,7 +336,7 @@ __global__ void __launch_bounds__(256) ozb_prepass_kernel(ARGS g, ImgArgs im, in
   auto load = [&](int c, int h) {
     const int gk = c * KC + 2 * sub + h;
     zc x = zmake(0.0, 0.0);
-    if (gm < n && gk < n) x = (g.opA == OP_N) ? A[(size_t)gm * n + gk] : zconj(A[(size_t)gk * n + gm]);
+    if (gm < n && gk < n) x = (g.opA == OP_N) ? A[(size_t)gm * n + gk] : conj_bits(A[(size_t)gk * n + gm]);
     return x;
   };
   constexpr int H = HOLD ? PASS : 1;
@@ -404,12 +419,6 @@ __device__ __forceinline__ double ldexp_int(long long v, int p) {
   if (lz == 64 || e < 0) return 0.0;
   return __hiloint2double((int)(r >> 32) + (e << 20) + sg, (int)(unsigned)r);
 }
-// x with its sign flipped by `mask` (0 or the sign bit): a negation chosen at run time would
-// be an FP64 instruction
-__device__ __forceinline__ double flip(double x, int mask) {
-  return __hiloint2double(__double2hiint(x) ^ mask, __double2loint(x));
-}
-
 // UAB: alpha = +-1, beta in {0, +-1}; MASK: g.active may be given (its registers cost the others 3%)
 template <int ND, int TNC, bool UAB, bool MASK>
 __global__ void __launch_bounds__(NT, 1) ozb_product_kernel(GemmArgs g, ImgArgs im, int* err) {
@@ -595,7 +604,7 @@ __global__ void __launch_bounds__(NT, 1) ozb_product_kernel(GemmArgs g, ImgArgs 
       for (int h = 0; h < KPT; ++h) {
         const int gk = c * KC + k0 + h;
         v[h] = zmake(0.0, 0.0);
-        if (gn < n && gk < n) v[h] = (g.opB == OP_N) ? B[(size_t)gk * n + gn] : zconj(B[(size_t)gn * n + gk]);
+        if (gn < n && gk < n) v[h] = (g.opB == OP_N) ? B[(size_t)gk * n + gn] : conj_bits(B[(size_t)gn * n + gk]);
       }
     };
     auto advance = [&]() {
