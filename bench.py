@@ -28,7 +28,7 @@ sys.path.insert(0, ROOT)
 
 import workloads as W  # noqa: E402
 
-# BF16 slice-pair products per complex product in the sliced GEMM: NS (NS + 1) / 2 for NS
+# 16-bit slice products per complex product in the sliced GEMM: NS (NS + 1) / 2 for NS
 # digits per value (s + t <= NS + 1); set from the loaded library by run_gpu
 OZ_SLICE_PAIRS = 36.0
 
@@ -174,7 +174,7 @@ def roofline_for(cls, stats, peaks, peak_src, sustained=True):
               of a complex product on the tensor cores, TF32 dense peak / 3 (a complex
               product costs 24 n^3 TF32 flops as a 3-term split), the TF32 peak taken as
               the bf16 peak x (1.1 / 2.25) (nominal ratio).  For the sliced product the
-              executed BF16 work (OZ_SLICE_PAIRS x useful) against the bf16 peak is
+              executed 16-bit work (OZ_SLICE_PAIRS x useful) against the bf16 peak is
               reported beside it (tensor-pipe occupancy by the emulation).
     gemm_f64, inv_f64: FP64 pipe ("alu"), peak 1.25 TFLOP/s nominal.
     inv_f32 : FP32 CUDA cores ("alu"), peak 152 SM x 128 lanes x 2 x 2.07 GHz."""
@@ -191,7 +191,7 @@ def roofline_for(cls, stats, peaks, peak_src, sustained=True):
                 f"{'sustained' if sustained else 'burst'} {peak_src} x 1.1/2.25)")
         extra = {"executed_bf16_tflops": achieved * OZ_SLICE_PAIRS,
                  "executed_bf16_frac": achieved * OZ_SLICE_PAIRS / bf16,
-                 "executed_note": f"{OZ_SLICE_PAIRS:.0f} BF16 slice-pair products per complex product "
+                 "executed_note": f"{OZ_SLICE_PAIRS:.0f} 16-bit slice products per complex product "
                                   f"vs bf16 {'sustained' if sustained else 'burst'} {peak_src} peak"}
     elif cls == "gemm_tc":
         bound, peak, unit = "tensor", bf16 * (1.1 / 2.25) / 3.0, "TFLOP/s"

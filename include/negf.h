@@ -148,9 +148,9 @@ negf_status negf_worklist(const negf_system* sys, int32_t bs, int32_t* count, in
  * residual ||(a00 - a01 g a10) g - I||_F / sqrt(b) stays above 1e-10 gets
  * NEGF_ERR_NOCONV in status[e].  Sigma_L = a10 g_L a01, Sigma_R = a01 g_R a10.
  * prec: NEGF_FP64 runs every product in FP64; NEGF_MIXED runs the products of the
- * decimation, the residuals and the Newton steps on the digit-sliced BF16 tensor-core
- * path (FP64-class: exact FP32 accumulation of 8-bit slices, ~2^-54 of the row/column
- * scales) when 16 <= b <= 512, with the inverses in FP32 refined twice (twice
+ * decimation, the residuals and the Newton steps on the digit-sliced FP16 tensor-core
+ * path (FP64-class: FP32 accumulation of 8-bit slices, ~2^-54 of the row/column
+ * scales) when 16 <= b <= 512 (b <= 16 without a guess: one FP64 launch in every mode), with the inverses in FP32 refined twice (twice
  * more for units whose refinement residual stays above 1e-7) and redone in FP64 for any unit
  * still above it; NEGF_MIXED_TF32 is treated as NEGF_FP64 (a TF32 product is far too coarse
  * for the 1e-10 residual).
@@ -341,7 +341,7 @@ negf_status negf_observables(negf_ctx* ctx, const negf_system* sys, negf_precisi
  * complex128 blocks; X[u] lives at X + u * x_stride (elements; 0 = one block shared
  * by all units).  op: 0 = as stored, 2 = conjugate transpose.  alpha, beta: host
  * double[2] (re, im).  C may be NULL (beta ignored) or equal to D; D must not
- * overlap A or B.  NEGF_FP64: FP64 FMA; NEGF_MIXED: digit-sliced BF16 tensor-core
+ * overlap A or B.  NEGF_FP64: FP64 FMA; NEGF_MIXED: digit-sliced FP16 tensor-core
  * product for 16 <= n <= 512 (K in exact passes of 128); NEGF_MIXED_TF32: 3-term TF32 split for n >= 16
  * (FP64 FMA outside those ranges). */
 negf_status negf_block_gemm(negf_ctx* ctx, negf_precision prec, int32_t n, int32_t units, int32_t opA,

@@ -419,7 +419,7 @@ __global__ void one_minus_kernel(BMat R, int n, const int* act) {
 struct Engine {
   Ctx* ctx;
   cudaStream_t s;
-  int mixed;           // 0: FP64, 1: digit-sliced BF16 tensor-core products, 2: TF32 3-term split
+  int mixed;           // 0: FP64, 1: digit-sliced tensor-core products, 2: TF32 3-term split
   void* inv_scratch;   // for inverses too large for shared memory
   void* oz_scratch = nullptr;   // per-row/column scales of the sliced products (in-kernel digits)
   void* ozt_scratch = nullptr;  // scales and digit images of the digitize-once sliced products
