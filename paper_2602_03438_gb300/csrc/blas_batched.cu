@@ -273,11 +273,15 @@ static cudaError_t launch_inv(BMat X, BMat M, int n, int units, const int* activ
 }
 
 // FP64 inverses run as column tiles over several CTAs per block (inv_tiles.cu) where there is
-// scratch for it and one CTA per block would leave SMs idle or keep the matrix in global
-// memory.  Measured (us, tiles : one CTA): n = 64, 8 blocks 229 : 412, 64 blocks 378 : 413; n =
-// 100, 20 blocks 463 : 1249; n = 110, 152 blocks 2064 : 1589; n = 48, 300 blocks 507 : 449; n =
-// 128, 16 blocks 767 : 2504, 400 blocks 6121 : 7629; n = 200, 8 blocks 1565 : 8965.
-static bool f64_tiles(int n, int units) { return n >= 112 || (n >= 64 && units <= 76); }
+// scratch for it and one CTA per block (a flat time up to 152 units) would leave SMs idle or
+// keep the matrix in global memory.  Measured (us, tiles : one CTA): n = 32, 96 blocks 124 :
+// 111; n = 40, 96 blocks 154 : 163, 400 349 : 476; n = 48, 152 blocks 251 : 228, 300 348 : 451; n = 56, 96
+// blocks 260 : 347; n = 64, 152 blocks 393 : 413, 600 1137 : 1634; n = 72, 80 blocks 444 : 553, 152 765 :
+// 554; n = 96, 80 blocks 736 : 1098, 300 2447 : 2189; n = 128, 16 blocks 538 : 2504, 400 5745 : 7629.
+static bool f64_tiles(int n, int units) {
+  if (n > 64) return n >= 112 || units <= 76;
+  return n >= 56 || (n >= 40 && (units <= 96 || units > 152));
+}
 
 cudaError_t zinv(BMat X, BMat M, int n, int units, const int* active, int single, void* scratch,
                  int32_t* status, cudaStream_t s, void* lent, size_t lent_bytes, bool few) {

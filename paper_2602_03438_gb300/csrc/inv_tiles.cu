@@ -19,8 +19,8 @@
 // What bounds it: the n sequential pivot steps, each about 250 instructions (FP64: some 50 of
 // the FP64 pipe at 64 clocks) of every warp of one CTA and one barrier, plus a launch per
 // panel; the updates (W and C from L2) run beside them.  Measured (GB300) against one CTA
-// per block: FP32 n = 512, 16 blocks 27.9 -> 1.22 ms; n = 256, 8 blocks 4.01 -> 0.28 ms; FP64
-// n = 128, one block 2.50 -> 0.47 ms, 400 blocks 7.6 -> 6.1 ms; n = 512, 2 blocks 138 -> 5.5 ms.
+// per block: FP32 n = 512, 16 blocks 27.9 -> 0.88 ms; n = 256, 8 blocks 4.01 -> 0.27 ms; FP64
+// n = 128, one block 2.50 -> 0.41 ms, 400 blocks 7.6 -> 5.7 ms; n = 512, 2 blocks 138 -> 5.5 ms.
 // TW: a row's entries fit in 32 registers, and the update reads C once for TW columns.
 #include <algorithm>
 #include <type_traits>
@@ -310,26 +310,29 @@ __device__ __forceinline__ void tile_step(const TileInv<typename Tr<R>::C>& g, i
   }
 }
 
-// the CTA's units of a launch whose blockIdx.y starts at them: the next with its flag set, from u
-// on in steps of gridDim.y (g.units: none left).  Flags are read a warp at a time.
+// the next unit with its flag set, from u on in steps of `stride` (g.units: none left).  Flags are
+// read a warp at a time.
 template <typename C>
-__device__ __forceinline__ int next_unit(const TileInv<C>& g, int u) {
+__device__ __forceinline__ int next_unit(const TileInv<C>& g, int u, int stride) {
   if (!g.active) return min(u, g.units);
-  for (; u < g.units; u += 32 * gridDim.y) {
-    const long long x = u + (long long)(threadIdx.x & 31) * gridDim.y;
+  for (; u < g.units; u += 32 * stride) {
+    const long long x = u + (long long)(threadIdx.x & 31) * stride;
     const unsigned int m = __ballot_sync(0xffffffffu, x < g.units && g.active[x]);
-    if (m) return u + (__ffs(m) - 1) * (int)gridDim.y;
+    if (m) return u + (__ffs(m) - 1) * stride;
   }
   return g.units;
 }
 
+// The CTAs that factor the next panel come first (blockIdx.y = 0): where the launch takes more
+// than one round of the SMs, no pivot chain starts in the last.  FP32 n = 512, 16 blocks 1298 ->
+// 880 us; n = 200, 40 blocks 339 -> 276; FP64 n = 128, 64 blocks 1330 -> 1025.
 template <typename R, int NT>
 __global__ void __launch_bounds__(NT, (sizeof(R) == 4 ? 1024 : 512) / NT)
     inv_tile_kernel(TileInv<typename Tr<R>::C> g, int panel) {
   pdl_begin();
-  const int t = blockIdx.x;
+  const int t = (panel + 1 + (int)blockIdx.y) % (int)gridDim.y, stride = gridDim.x;
   if (t == panel) return;
-  for (int u = next_unit(g, blockIdx.y); u < g.units; u = next_unit(g, u + gridDim.y)) {
+  for (int u = next_unit(g, blockIdx.x, stride); u < g.units; u = next_unit(g, u + stride, stride)) {
     tile_step<R, NT>(g, panel, t, u);
     __syncthreads();   // the next unit of this CTA reuses the shared buffers
   }
@@ -362,19 +365,17 @@ __device__ __forceinline__ void gather_rows(const TileInv<C>& g, int last_panel,
 template <typename C>
 __global__ void __launch_bounds__(256) inv_gather_kernel(TileInv<C> g, int last_panel) {
   pdl_begin();
-  const int i0 = blockIdx.x * kOutRows;
-  for (int u = next_unit(g, blockIdx.y); u < g.units; u = next_unit(g, u + gridDim.y))
+  const int i0 = blockIdx.x * kOutRows, stride = gridDim.y;
+  for (int u = next_unit(g, blockIdx.y, stride); u < g.units; u = next_unit(g, u + stride, stride))
     gather_rows(g, last_panel, u, i0, min(kOutRows, g.n - i0));
 }
 
 // Up to 16 tiles and few units: one cluster per unit with a CTA per tile, cluster barriers in
 // place of the launches (the tiles still pass through L2).  No gaps between the panels, and
-// a mask without units costs one launch; but a waiting cluster holds its SMs, so many units
+// a mask without units costs one launch; but a waiting cluster holds its SMs, so more units
 // run better as launches.  Measured (GB300, us, launches : cluster): FP64 n = 128, no unit of
-// 384 set 110 : 6, 1 472 : 415, 8 472 : 598 (the CTAs of a cluster share SMs and their FP64
-// pipes), 32 1142 : 808, 48 1173 : 1329, 400 6103 : 8883; n = 72, 1 261 : 232, 24 327 : 460; n = 64,
-// 8 236 : 205.  FP32 n = 200, 1 254 : 196, 24 286 : 280, 40 371 : 452; n = 256, 32 537 : 361;
-// n = 140, 8 180 : 164, 40 218 : 310.
+// 384 set 110 : 6, 4 units 429 : 414, 16 538 : 680, 400 5745 : 8883; n = 64, 8 214 : 203.  FP32 n =
+// 140, 4 148 : 137, 8 148 : 165; n = 200, 4 209 : 198, 8 210 : 231; n = 256, 4 267 : 252, 16 291 : 322.
 constexpr int kMaxCluster = 16;   // more than 8 CTAs: opted in, every GPC has room for them
 __device__ __forceinline__ void cluster_barrier() {
   asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
@@ -383,9 +384,9 @@ template <typename R, int NT>
 __global__ void __launch_bounds__(NT, (sizeof(R) == 4 ? 1024 : 512) / NT)
     inv_cluster_kernel(TileInv<typename Tr<R>::C> g, int tiles) {
   pdl_begin();
-  const int t = blockIdx.x, per = (g.n + gridDim.x - 1) / gridDim.x, i0 = t * per;
+  const int t = blockIdx.x, per = (g.n + gridDim.x - 1) / gridDim.x, i0 = t * per, stride = gridDim.y;
   // (the CTAs of a cluster share blockIdx.y and so take the same units)
-  for (int u = next_unit(g, blockIdx.y); u < g.units; u = next_unit(g, u + gridDim.y)) {
+  for (int u = next_unit(g, blockIdx.y, stride); u < g.units; u = next_unit(g, u + stride, stride)) {
     for (int panel = -1; panel < tiles; ++panel) {
       if (t < tiles && t != panel) tile_step<R, NT>(g, panel, t, u);
       cluster_barrier();
@@ -397,7 +398,7 @@ __global__ void __launch_bounds__(NT, (sizeof(R) == 4 ? 1024 : 512) / NT)
 template <typename R, int NT>
 cudaError_t launch_tiles(const TileInv<typename Tr<R>::C>& g, int tiles, int rows, cudaStream_t s) {
   for (int panel = -1; panel < tiles; ++panel) {
-    cudaError_t e = launch_pdl(inv_tile_kernel<R, NT>, dim3(tiles, rows), NT, 0, s, g, panel);
+    cudaError_t e = launch_pdl(inv_tile_kernel<R, NT>, dim3(rows, tiles), NT, 0, s, g, panel);
     if (e != cudaSuccess) return e;
   }
   return launch_pdl(inv_gather_kernel<typename Tr<R>::C>, dim3((g.n + kOutRows - 1) / kOutRows, rows), 256, 0, s, g, tiles - 1);
@@ -443,7 +444,7 @@ cudaError_t run(BMat X, BMat M, int n, int units, const int* active, bool few, v
   g.status = status;
   const int tiles = (n + Tr<R>::TW - 1) / Tr<R>::TW;
   const int rows = std::min(units, active ? kMaskedUnits : 65535);
-  const bool cluster = active ? few : units * (tiles <= 8 ? 1 : 2) <= (sizeof(R) == 4 ? 48 : 8);
+  const bool cluster = active ? few : units * (tiles <= 8 ? 1 : 2) <= 8;
   if constexpr (sizeof(R) == 8) {   // (FP32 blocks up to 128: zinv_reg)
     if (n <= 64) return launch_inv<R, 64>(g, tiles, rows, cluster, INIT_INVC_D64, s);
     if (n <= 128) return launch_inv<R, 128>(g, tiles, rows, cluster, INIT_INVC_D128, s);

@@ -96,6 +96,11 @@ def test_zero_column_is_reported(P, n, col):
         assert float((eye - M[u] @ X[u]).norm()) <= bound
 
 
-@pytest.mark.parametrize("n,units", [(129, 24), (129, 25), (240, 26), (256, 24), (256, 25)])
-def test_tiles_of_few_and_many_blocks(P, n, units):   # one cluster per block up to 24 of them
+@pytest.mark.parametrize("n,units", [(129, 4), (240, 5), (129, 24), (129, 25), (240, 26), (256, 24), (256, 25)])
+def test_tiles_of_few_and_many_blocks(P, n, units):   # one cluster per block up to 4 of them
     test_tile_inverse(P, n, units)
+
+
+@pytest.mark.parametrize("n,units", [(39, 2), (40, 96), (40, 97), (41, 153), (55, 152), (56, 100), (64, 9), (64, 160)])
+def test_fp64_inverse_of_small_tiles(P, n, units):
+    test_fp64_inverse(P, n, units)
