@@ -283,15 +283,25 @@ static bool f64_tiles(int n, int units) {
   return n >= 56 || (n >= 40 && (units <= 96 || units > 152));
 }
 
+// FP32 blocks up to 128 are inverted in registers, one CTA per block and SM, in rounds of 120 us
+// at n = 128; tiles take about 100 us + 0.6 per block and win where the last round of the
+// registers is far from full (n = 128, us, tiles : registers: 152 blocks 187 : 125, 200 214 : 241,
+// 304 260 : 244, 400 324 : 359, 512 406 : 476, 1024 821 : 830; n = 100, 300 208 : 189; n = 96, 512 237 :
+// 246).  A mask may leave few of the units.
+bool f32_tiles(int n, int units, const int* active) {
+  if (n <= 96 || n > 128) return n > 128;
+  return !active && units > 152 && 500 + 3ll * units < 600ll * ((units + 151) / 152);
+}
+
 cudaError_t zinv(BMat X, BMat M, int n, int units, const int* active, int single, void* scratch,
                  int32_t* status, cudaStream_t s, void* lent, size_t lent_bytes, bool few) {
   if (units <= 0 || n <= 0) return cudaSuccess;
-  if (single && n <= 128) return zinv_reg(X, M, n, units, active, status, s);
-  if (n <= 512 && (single || f64_tiles(n, units))) {
+  if (n <= 512 && (single ? f32_tiles(n, units, active) : f64_tiles(n, units))) {
     const size_t need = zinv_tiles_bytes(n, units, single);
     void* t = lent_bytes >= need ? lent : (zinv_scratch_bytes(n, units, single) >= need ? scratch : nullptr);
     if (t) return zinv_tiles(X, M, n, units, active, single, t, status, s, few);
   }
+  if (single && n <= 128) return zinv_reg(X, M, n, units, active, status, s);
   if (single) return launch_inv<float>(X, M, n, units, active, scratch, status, s);
   return launch_inv<double>(X, M, n, units, active, scratch, status, s);
 }

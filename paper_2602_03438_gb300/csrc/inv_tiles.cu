@@ -445,9 +445,11 @@ cudaError_t run(BMat X, BMat M, int n, int units, const int* active, bool few, v
   const int tiles = (n + Tr<R>::TW - 1) / Tr<R>::TW;
   const int rows = std::min(units, active ? kMaskedUnits : 65535);
   const bool cluster = active ? few : units * (tiles <= 8 ? 1 : 2) <= 8;
-  if constexpr (sizeof(R) == 8) {   // (FP32 blocks up to 128: zinv_reg)
+  if constexpr (sizeof(R) == 8) {
     if (n <= 64) return launch_inv<R, 64>(g, tiles, rows, cluster, INIT_INVC_D64, s);
     if (n <= 128) return launch_inv<R, 128>(g, tiles, rows, cluster, INIT_INVC_D128, s);
+  } else if (n <= 128) {
+    return launch_tiles<R, 128>(g, tiles, rows, s);
   }
   return n <= 256 ? launch_inv<R, 256>(g, tiles, rows, cluster, INIT_INVC_F256, s)
                   : launch_inv<R, 512>(g, tiles, rows, false, 0, s);
@@ -464,9 +466,9 @@ cudaError_t run(BMat X, BMat M, int n, int units, const int* active, bool few, v
 // y_K of its own columns through shared memory.  No launch per panel and no pass over the
 // matrix: bound by the chain of n pivot steps, some 1000 clocks each (two barriers' worth of
 // exchange, one reciprocal, 15 column updates); the next step's search starts among them.
-// Measured (GB300, us, against column tiles): one block of 128 120 : 128, 152 blocks 125 : 285,
-// 400 360 : 396, 512 476 : 462, 1024 831 : 890; 512 of 96 247 : 291; 600 of 64 77 : 175; 1024 of
-// 32 36 : 86.  At 96 rows two CTAs per SM pay for a few spilled registers (344 with one).
+// Measured (GB300, us, against column tiles): one block of 128 120 : 114, 64 blocks 123 : 137, 152
+// 125 : 187, 200 241 : 213, 304 244 : 259, 512 476 : 406, 1024 830 : 818; 512 of 96 246 : 237; 600 of 64
+// 77 : 115; 1000 of 32 36 : 62.  At 96 rows two CTAs per SM pay for a few spilled registers (344 with one).
 // ---------------------------------------------------------------------------
 constexpr int RC = 32;        // columns per thread
 constexpr int RP = 16;        // columns per panel

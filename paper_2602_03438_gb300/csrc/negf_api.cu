@@ -524,9 +524,8 @@ struct Engine {
     const bool masked = active != nullptr && active_frac < 0.0;   // an unknown share of the work
     const double frac = (active && active_frac >= 0.0) ? active_frac : 1.0;
     begin(masked ? K_OTHER : (single ? K_INV_F32 : K_INV_F64));
-    // the FP32 inverse of large blocks may use the sliced products' scratch, whose images are
-    // then gone
-    void* lent = (single && n > 128 && mixed == 1 && oz_supported(n)) ? ozt_scratch : nullptr;
+    // the FP32 inverse as tiles may use the sliced products' scratch, whose images are then gone
+    void* lent = (single && f32_tiles(n, units, active) && mixed == 1 && oz_supported(n)) ? ozt_scratch : nullptr;
     size_t lent_bytes = lent ? ozt_scratch_bytes(n, units) : 0;
     if (lent) last_a = AKey();
     const long long nn = (long long)n * n;

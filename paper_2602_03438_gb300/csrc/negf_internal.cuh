@@ -190,6 +190,7 @@ cudaError_t zgemm_ozt_variant(const GemmArgs& g, void* scratch, int* err, cudaSt
 cudaError_t zinv(BMat X, BMat M, int n, int units, const int* active, int single, void* scratch,
                  int32_t* status, cudaStream_t s, void* lent = nullptr, size_t lent_bytes = 0, bool few = false);
 size_t zinv_scratch_bytes(int n, int units, int single);
+bool f32_tiles(int n, int units, const int* active);   // the FP32 inverse runs better with scratch for tiles
 // the inverse as column tiles, several CTAs per block (inv_tiles.cu; n <= 512); `scratch`
 // holds zinv_tiles_bytes(n, units, single) bytes, 16-byte aligned
 cudaError_t zinv_tiles(BMat X, BMat M, int n, int units, const int* active, int single, void* scratch, int32_t* status,

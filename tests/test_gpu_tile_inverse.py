@@ -104,3 +104,8 @@ def test_tiles_of_few_and_many_blocks(P, n, units):   # one cluster per block up
 @pytest.mark.parametrize("n,units", [(39, 2), (40, 96), (40, 97), (41, 153), (55, 152), (56, 100), (64, 9), (64, 160)])
 def test_fp64_inverse_of_small_tiles(P, n, units):
     test_fp64_inverse(P, n, units)
+
+
+@pytest.mark.parametrize("n,units", [(96, 153), (97, 152), (97, 153), (112, 160), (128, 153), (128, 304)])
+def test_fp32_inverse_past_one_round(P, n, units):   # tiles where the second round of 152 would be far from full
+    test_tile_inverse(P, n, units)
