@@ -574,7 +574,7 @@ def run_gpu(args):
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": ms / args.steps, "higher_is_better": True, "scaling": "weak",
         "vs_baseline": None,
-        "dtype": {P.MIXED: f"bf16 {ns}-digit slices (exact fp32 accumulate) + f32 inverse + f64",
+        "dtype": {P.MIXED: f"fp16 {ns}-digit slices (fp32 accumulate) + f32 inverse + f64",
                   P.MIXED_TF32: "tf32x3 + f32 inverse + f64", P.FP64: "f64"}[prec],
         "data": "synthetic",
         "config": {"workload": f"config 2: ballistic batched RGF, nb={nb}, b={b}, {ne} energies/GPU in [-3,3], "
