@@ -144,15 +144,18 @@ negf_status negf_worklist(const negf_system* sys, int32_t bs, int32_t* count, in
  * repeats block nb-1 with hop H_{nb-2,nb-1}.  Surface Green's functions by
  * Lopez Sancho-Rubio decimation in FP64 (stop when max|alpha|,|beta| < tol *
  * initial, at most max_iter steps), followed when needed by up to 3 FP64
- * Newton steps on the surface fixed-point equation; an energy whose surface
- * residual ||(a00 - a01 g a10) g - I||_F / sqrt(b) stays above 1e-10 gets
+ * Newton steps on the surface fixed-point equation.  A unit whose Newton steps
+ * diverge (the decimation passed a nearly singular block) starts again: decimation
+ * at 3, 5, 2, 8 and 16 times eta in turn, up to 6 Newton steps at eta from each, until
+ * a result's residual is <= 1e-10 and it passes the retarded-root test below; if
+ * none does, the first result stands.  An energy whose surface residual ||(a00 - a01 g a10) g - I||_F / sqrt(b) stays above 1e-10 gets
  * NEGF_ERR_NOCONV in status[e].  Sigma_L = a10 g_L a01, Sigma_R = a01 g_R a10.
  * prec: NEGF_FP64 runs every product in FP64; NEGF_MIXED runs the products of the
  * decimation, the residuals and the Newton steps on the digit-sliced FP16 tensor-core
  * path (FP64-class: FP32 accumulation of 8-bit slices, ~2^-54 of the row/column
- * scales) when 16 <= b <= 512 (b <= 16 without a guess: one FP64 launch in every mode), with the inverses in FP32 refined twice (twice
- * more for units whose refinement residual stays above 1e-7) and redone in FP64 for any unit
- * still above it; NEGF_MIXED_TF32 is treated as NEGF_FP64 (a TF32 product is far too coarse
+ * scales) when 16 <= b <= 512 (b <= 16 without a guess: one FP64 launch in every mode),
+ * with the inverses in FP32 refined twice (twice more for units whose refinement residual
+ * stays above 1e-7) and redone in FP64 for any unit still above it; NEGF_MIXED_TF32 is treated as NEGF_FP64 (a TF32 product is far too coarse
  * for the 1e-10 residual).
  *
  * Warm start (optional, per lead side): with g0_L and/or g0_R given, that side
@@ -168,10 +171,10 @@ negf_status negf_worklist(const negf_system* sys, int32_t bs, int32_t* count, in
  *   g0_L, g0_R : in, device [sum ne] blocks of surface-function guesses, or NULL.
  *   sigma_L/R  : out, device [sum ne] blocks.
  *   gs_L, gs_R : out, device [sum ne] blocks: the surface functions g_L, g_R, or NULL.
- *   iters      : out, device int32 [2*sum ne]: decimation steps (L, R) per energy
- *                (0 when the warm start was kept), or NULL.
- *   newton     : out, device int32 [2*sum ne]: Newton steps (L, R) per energy, warm
- *                and polishing steps together, or NULL.
+ *   iters      : out, device int32 [2*sum ne]: decimation steps (L, R) per energy of
+ *                the decimation at eta (0 when the warm start was kept), or NULL.
+ *   newton     : out, device int32 [2*sum ne]: Newton steps (L, R) per energy, warm,
+ *                polishing and restart steps together, or NULL.
  *   status     : out, device int32 [sum ne] (NEGF_OK or a negative code), or NULL.
  * Requires nb >= 2 for every device. */
 negf_status negf_obc(negf_ctx* ctx, const negf_system* sys, negf_precision prec, double tol, int32_t max_iter,

@@ -1228,12 +1228,17 @@ struct LeadArgs {
   const UnitDev* udev = nullptr;
   const int* unit_dev = nullptr;
   const int* unit_e = nullptr;
+  // a restart: the decimation's own slots of the units flagged in `only`, at `widen` times the
+  // broadening (a00, al0, be0 stay)
+  double widen = 1.0;
+  const int* only = nullptr;
 };
 
 // unit u < U: left lead of energy e0+u; u >= U: right lead of energy e0+u-U
 __global__ void lead_init_kernel(LeadArgs a) {
   pdl_begin();
   const int u = blockIdx.y;
+  if (a.only && !a.only[u]) return;
   const bool left = u < a.U;
   const int k = left ? u : u - a.U;   // the energy unit
   int e = a.e0 + k;
@@ -1243,7 +1248,7 @@ __global__ void lead_init_kernel(LeadArgs a) {
   }
   const int b = a.dv.b, nb = a.dv.nb;
   const long long bb = (long long)b * b;
-  const zc z = zmake(a.dv.E[e], a.dv.eta);
+  const zc z = zmake(a.dv.E[e], a.widen * a.dv.eta);
   const int cd = left ? 0 : nb - 1;   // lead cell copies this device block
   const int cu = left ? 0 : nb - 2;   // ... and this hop
   for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < bb;
@@ -1260,9 +1265,13 @@ __global__ void lead_init_kernel(LeadArgs a) {
     const zc al = left ? a10 : a01;
     const zc be = left ? a01 : a10;
     const long long o = u * bb + idx;
-    a.a00[o] = a00; a.eps[o] = a00; a.epss[o] = a00;
-    a.al0[o] = al; a.al[o] = al;
-    a.be0[o] = be; a.be[o] = be;
+    a.eps[o] = a00; a.epss[o] = a00;
+    a.al[o] = al;
+    a.be[o] = be;
+    if (a.only) continue;
+    a.a00[o] = a00;
+    a.al0[o] = al;
+    a.be0[o] = be;
   }
 }
 
@@ -1707,24 +1716,76 @@ __global__ void __launch_bounds__(1024) compact_kernel(const int* mask, int unit
   }
 }
 
+// the sum of v over the CTA, in thread 0
+__device__ __forceinline__ int cta_count(int v) {
+  __shared__ int red[32];
+  for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+  __syncthreads();
+  if (threadIdx.x == 0)
+    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) v += red[w];
+  return v;
+}
+
 __global__ void count_kernel(const int* flags, int units, int* out) {
   pdl_begin();
   int c = 0;
   for (int u = threadIdx.x; u < units; u += blockDim.x) c += flags[u] != 0;
-  for (int off = 16; off > 0; off >>= 1) c += __shfl_down_sync(0xffffffffu, c, off);
-  __shared__ int red[32];
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = c;
-  __syncthreads();
+  c = cta_count(c);
+  if (threadIdx.x == 0) *out = c;
+}
+
+// open[u] = 1 for the decimated units (cold, converged) whose residual is not accepted and whose
+// last Newton step (residual resn) diverged; out[0] = flags set, out[1] = open units
+__global__ void count_open_kernel(const int* flags, const int* cold, const int* done, const double* res,
+                                  const double* resn, double accept, int units, int* open, int* out) {
+  pdl_begin();
+  int c = 0, o = 0;
+  for (int u = threadIdx.x; u < units; u += blockDim.x) {
+    const int x = (cold[u] && done[u] == 1 && !(res[u] <= accept) && !(resn[u] <= kDiverged * res[u])) ? 1 : 0;
+    open[u] = x;
+    o += x;
+    c += flags[u] != 0;
+  }
+  c = cta_count(c);
+  o = cta_count(o);
   if (threadIdx.x == 0) {
-    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) c += red[w];
-    *out = c;
+    out[0] = c;
+    out[1] = o;
   }
 }
 
-__global__ void set_need_kernel(const double* res, int* need, int units, double target, const int* only) {
+// A restart's end.  open[u]: the unit was restarted; ok[u]: its result is accepted and retarded, and
+// the unit is open no more.  Otherwise g and res become what they were (kept in the
+// outputs' Sigma blocks and res0).  save: keep them instead
+__global__ void restart_settle_kernel(BMat g, BMat keep_L, BMat keep_R, int U, int n, double* res, double* res0, int* open,
+                                      const int* done, const int* ok, int save) {
+  pdl_begin();
+  const int u = blockIdx.x;
+  if (!open[u]) return;
+  const bool good = !save && done[u] == 1 && ok[u];
+  zc* x = g.at(u);
+  zc* y = u < U ? keep_L.at(u) : keep_R.at(u - U);
+  const int nn = n * n;
+  if (save) {
+    for (int i = threadIdx.x; i < nn; i += blockDim.x) y[i] = x[i];
+  } else if (!good) {
+    for (int i = threadIdx.x; i < nn; i += blockDim.x) x[i] = y[i];
+  }
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  if (save) res0[u] = res[u];
+  else if (good) open[u] = 0;
+  else res[u] = res0[u];
+}
+
+__global__ void set_need_kernel(const double* res, double* resn, int* need, int units, double target, const int* only) {
   pdl_begin();
   const int u = blockIdx.x * blockDim.x + threadIdx.x;
-  if (u < units) need[u] = (only[u] && res[u] > target) ? 1 : 0;
+  if (u >= units) return;
+  need[u] = (only[u] && res[u] > target) ? 1 : 0;
+  resn[u] = INFINITY;   // no Newton step yet
 }
 
 __global__ void obc_finish_kernel(const int* done, const double* res, const int* iters, const int* nsteps, int U,
@@ -2696,6 +2757,7 @@ negf_status negf_obc(negf_ctx* c, const negf_system* sys, negf_precision prec, d
       double* ref = (double*)p; p += sizeof(double) * NU;
       double* res = (double*)p; p += sizeof(double) * NU;
       double* resn = (double*)p; p += sizeof(double) * NU;
+      double* res0 = (double*)p; p += sizeof(double) * NU;            // a restarted unit's residual before
       long long* coff = (long long*)p; p += sizeof(long long) * NU;   // compact unit list (block offsets)
       int* done = (int*)p; p += sizeof(int) * NU;
       int* it_arr = (int*)p; p += sizeof(int) * NU;
@@ -2706,6 +2768,8 @@ negf_status negf_obc(negf_ctx* c, const negf_system* sys, negf_precision prec, d
       int* cold = (int*)p; p += sizeof(int) * NU;     // unit goes through the decimation
       int* nsteps = (int*)p; p += sizeof(int) * NU;   // Newton steps taken
       int* redo = (int*)p; p += sizeof(int) * NU;     // refined inverse redone in FP64
+      int* done2 = (int*)p; p += sizeof(int) * NU;    // done and iteration count of a restart
+      int* it2 = (int*)p; p += sizeof(int) * NU;
       int* n_active = (int*)p; p += 16;
       p = (char*)(((uintptr_t)p + 255) & ~(uintptr_t)255);
       eng.inv_scratch = zinv_scratch_bytes(b, NU, 0) ? (void*)p : nullptr;
@@ -2725,7 +2789,7 @@ negf_status negf_obc(negf_ctx* c, const negf_system* sys, negf_precision prec, d
         ObcSmall q;
         q.dv = dv; q.e0 = e0; q.U = U; q.b = b; q.max_iter = max_iter;
         q.udev = t_udev; q.unit_dev = t_dev; q.unit_e = t_e;
-        q.tol = tol; q.target = target;
+        q.tol = tol; q.target = target; q.accept = accept;
         q.sigma_L = lead_at(sigma_L); q.sigma_R = lead_at(sigma_R);
         q.gs_L = lead_at(gs_L); q.gs_R = lead_at(gs_R);
         q.done = done; q.iters = it_arr; q.nsteps = nsteps; q.res = res;
@@ -2877,26 +2941,28 @@ negf_status negf_obc(negf_ctx* c, const negf_system* sys, negf_precision prec, d
       const int n_cold = any_warm ? n_set(cold) : NU;
       if (n_cold < 0) return fail(ctx, NEGF_ERR_CUDA, "OBC: flag read-back failed");
 
-      launch_pdl(lead_norm_kernel, NU, book_threads(b), 0, s, al, be, b, 0, ref, done, act, it_arr, 0, tol, n_active,
-                 keep);
-      KCHECK();
-      if (n_cold > 0) {
-        // ---- decimation
+      // decimation of the units not in `skip`, the surface functions of those in `mask` (NULL: all)
+      // and their residuals
+      auto decimate = [&](const int* skip, const int* mask, int* dn, int* its, int count) -> negf_status {
+        launch_pdl(lead_norm_kernel, NU, book_threads(b), 0, s, al, be, b, 0, ref, dn, act, its, 0, tol, n_active, skip);
+        KCHECK();
+        if (count <= 0) return NEGF_OK;
+        negf_status sc;
         for (int it = 0; it <= max_iter; ++it) {
           // counts after the first step (most units end there) and every fourth
           const bool poll = it == 1 || (it & 3) == 3 || it == max_iter;
           if (poll) CU(cudaMemsetAsync(n_active, 0, sizeof(int), s));
-          launch_pdl(lead_norm_kernel, NU, book_threads(b), 0, s, al, be, b, 1, ref, done, act, it_arr, it,
+          launch_pdl(lead_norm_kernel, NU, book_threads(b), 0, s, al, be, b, 1, ref, dn, act, its, it,
                      tol, poll ? n_active : nullptr, nullptr);
           KCHECK();
           if (poll) {
             CU(cudaMemcpyAsync(ctx->h_pinned, n_active, sizeof(int), cudaMemcpyDeviceToHost, s));
             CU(cudaStreamSynchronize(s));
             if (ctx->h_pinned[0] == 0) break;
-            if ((st = compact(act, ctx->h_pinned[0])) != NEGF_OK) return st;
+            if ((sc = compact(act, ctx->h_pinned[0])) != NEGF_OK) return sc;
           }
           if (it == max_iter) break;
-          if ((st = lead_inverse(g, eps, act)) != NEGF_OK) return st;        // g = eps^{-1}
+          if ((sc = lead_inverse(g, eps, act)) != NEGF_OK) return sc;        // g = eps^{-1}
           // the two products of each left operand back to back (the sliced product keeps
           // its digit images for the second)
           CU(lgemm(T[0], al, OP_N, g, OP_N, ONE, NOMAT, ZERO, act));              // al g
@@ -2905,27 +2971,68 @@ negf_status negf_obc(negf_ctx* c, const negf_system* sys, negf_precision prec, d
           CU(lgemm(T[1], be, OP_N, g, OP_N, ONE, NOMAT, ZERO, act));              // be g
           CU(lgemm(T[3], T[1], OP_N, al, OP_N, ONE, NOMAT, ZERO, act));           // be g al
           CU(lgemm(T[5], T[1], OP_N, be, OP_N, MONE, NOMAT, ZERO, act, true));    // -be g be
-          launch_pdl(lead_update_kernel, eg, 256, 0, s, eps, epss, T[2], T[3], b, done);
+          launch_pdl(lead_update_kernel, eg, 256, 0, s, eps, epss, T[2], T[3], b, dn);
           KCHECK();
           std::swap(al, T[4]);
           std::swap(be, T[5]);
         }
         ncomp = 0;
-        // ---- surface function and its residual
-        if ((st = lead_inverse(g, epss, any_warm ? cold : nullptr)) != NEGF_OK) return st;
-        if ((st = residual(g, res, any_warm ? cold : nullptr)) != NEGF_OK) return st;
-        // ---- Newton polishing of the decimation result above the target
-        launch_pdl(set_need_kernel, (NU + 255) / 256, 256, 0, s, res, need, NU, target, cold);
+        if ((sc = lead_inverse(g, epss, mask)) != NEGF_OK) return sc;
+        return residual(g, res, mask);
+      };
+      // up to `most` Newton steps on the units in `only` above the target; n_open: how many
+      // decimated units it left outside its basin (flagged in `warm`, free by then)
+      auto polish = [&](const int* only, int most, int& n_open) -> negf_status {
+        negf_status sc;
+        launch_pdl(set_need_kernel, (NU + 255) / 256, 256, 0, s, res, resn, need, NU, target, only);
         KCHECK();
         BMat gn = eps;   // decimation slots are free now
-        for (int step = 0; step < 3; ++step) {
-          const int cnt = n_set(need);
-          if (cnt < 0) return fail(ctx, NEGF_ERR_CUDA, "OBC: flag read-back failed");
-          if (cnt == 0) break;
-          if ((st = newton_step(need, gn, cnt)) != NEGF_OK) return st;
+        for (int step = 0;; ++step) {
+          ++ctx->launches;
+          launch_pdl(count_open_kernel, 1, 256, 0, s, need, cold, done, res, resn, accept, NU,
+                     warm, n_active);
+          CU(cudaGetLastError());
+          CU(cudaMemcpyAsync(ctx->h_pinned, n_active, 2 * sizeof(int), cudaMemcpyDeviceToHost, s));
+          CU(cudaStreamSynchronize(s));
+          const int cnt = ctx->h_pinned[0];
+          n_open = ctx->h_pinned[1];
+          if (cnt == 0 || step == most) break;
+          if ((sc = newton_step(need, gn, cnt)) != NEGF_OK) return sc;
           launch_pdl(newton_accept_kernel, NU, 256, 0, s, g, gn, b, res, resn, need, target, nsteps);
           KCHECK();
           // units that took the step continue from T1/T2 (K, F of the accepted g)
+        }
+        return NEGF_OK;
+      };
+      const int* dec = any_warm ? cold : nullptr;   // the units to decimate (NULL: all)
+      if ((st = decimate(keep, dec, done, it_arr, n_cold)) != NEGF_OK) return st;
+      if (n_cold > 0) {
+        int n_open = 0;
+        if ((st = polish(cold, 3, n_open)) != NEGF_OK) return st;
+        // restarts of the units whose polishing diverged (restart_widen; the flags in `warm` are theirs)
+        const BMat kL = lead_at(sigma_L), kR = lead_at(sigma_R);
+        if (n_open > 0) {
+          launch_pdl(restart_settle_kernel, NU, 256, 0, s, g, kL, kR, U, b, res, res0, warm, done, keep, 1);
+          KCHECK();
+        }
+        for (int k = 0; k < kRestarts && n_open > 0; ++k) {
+          la.eps = eps.p; la.epss = epss.p; la.al = al.p; la.be = be.p;
+          la.widen = restart_widen(k);
+          la.only = warm;
+          launch_pdl(lead_init_kernel, eg, 256, 0, s, la);
+          KCHECK();
+          launch_pdl(not_kernel, (NU + 255) / 256, 256, 0, s, warm, keep, NU);
+          KCHECK();
+          if ((st = decimate(keep, warm, done2, it2, n_open)) != NEGF_OK) return st;
+          CU(cudaMemcpyAsync(keep, warm, sizeof(int) * NU, cudaMemcpyDeviceToDevice, s));   // the restarted units
+          int left = 0;
+          if ((st = polish(keep, kRestartSteps, left)) != NEGF_OK) return st;
+          launch_pdl(retarded_check_kernel, NU, 256, 0, s, g, T[0], b, keep, res, accept, 1e-12, act);
+          KCHECK();
+          CU(cudaMemcpyAsync(warm, keep, sizeof(int) * NU, cudaMemcpyDeviceToDevice, s));
+          launch_pdl(restart_settle_kernel, NU, 256, 0, s, g, kL, kR, U, b, res, res0, warm, done2, act, 0);
+          KCHECK();
+          if ((n_open = n_set(warm)) < 0) return fail(ctx, NEGF_ERR_CUDA, "OBC: flag read-back failed");
         }
       }
       // the lead blocks of the chunk's energies in the outputs: contiguous for one device,

@@ -240,12 +240,26 @@ struct UnitDev {
 // unit_e[k] of device udev[unit_dev[k]] when udev is given.  done, iters, nsteps, res
 // ([2U]) as the batched path leaves them; gs_L, gs_R nullable.
 constexpr int kObcSmallB = 16;
+// A lead unit whose Newton polishing diverges starts again: decimation at restart_widen times
+// the broadening, then up to kRestartSteps Newton steps at its own.  Where eps is nearly singular
+// on the way (condition 1e7 to 2e9 at eta = 1e-6), rounding leaves the surface function with a
+// residual of 1e-4 to 1e-2, outside Newton's basin: the result was then wrong by 1e-5 to 1e-3,
+// and which units it hit changed with every change of rounding (b = 128: 1 to 2 of 100 calls of
+// 192 energies).  A larger broadening lowers the condition, and up to several times the
+// lead's own (b = 128; wider for small blocks) its surface function lies inside the basin.  18
+// such units of b = 8 to 128, one restart at 2, 3, 4, 5, 6 times the broadening: 52, 68, 62, 62,
+// 60 of 72 trials solved; one of b = 16 wants 8 and more.
+// A step counts as divergence where it multiplies the residual by kDiverged and more or makes
+// it non-finite: a unit that ends at its rounding floor (|g| near 1 / eta) does not.
+constexpr int kRestarts = 5, kRestartSteps = 6;
+constexpr double kDiverged = 100.0;
+__host__ __device__ constexpr double restart_widen(int k) { return k == 0 ? 3.0 : k == 1 ? 5.0 : k == 2 ? 2.0 : k == 3 ? 8.0 : 16.0; }
 struct ObcSmall {
   DevView dv;
   int e0, U, b, max_iter;
   const UnitDev* udev;
   const int *unit_dev, *unit_e;
-  double tol, target;
+  double tol, target, accept;
   BMat sigma_L, sigma_R, gs_L, gs_R;
   int *done, *iters, *nsteps;
   double* res;

@@ -3,7 +3,8 @@
 // the surface function and its residual, up to three Newton steps on the surface
 // fixed-point equation (Smith doubling of the Stein equation) and Sigma, in shared memory
 // and FP64.  The steps, their order and the stop rules are those of the batched path
-// (negf_obc); a unit stops when it has converged instead of when the batch is polled.
+// (negf_obc), its restarts at a larger broadening included; a unit stops when it has converged
+// instead of when the batch is polled.
 //
 // What bounds it: the FP64 pipe (small_block.cuh) along one unit's serial chain of six
 // products and an inverse per decimation step and four products per Smith level.
@@ -55,28 +56,27 @@ __global__ void __launch_bounds__(small_threads(kObcSmallB)) obc_small_kernel(Ob
   __shared__ double red[4][kMaxWarps];
   __shared__ int piv[kSmallB];
   const SmallElem t(b);
-  const zc z = zmake(a.dv.E[e], a.dv.eta);
   const int cd = left ? 0 : a.dv.nb - 1, cu = left ? 0 : a.dv.nb - 2;
   const long long idx = (long long)t.r * b + t.c, cr = (long long)t.c * b + t.r;
   zc *al = buf(0), *be = buf(1), *g = buf(2), *V = buf(3), *T0 = buf(4), *T1 = buf(5);
   zc *S = buf(6), *F = buf(7), *X = buf(8), *Y = buf(9);
 
-  // this thread's component of the lead's A blocks: the onsite block, the coupling alpha away
-  // from the surface and beta back (right lead: a01, a10; left lead: swapped)
-  auto a01 = [&]() {
-    const zc s = a.dv.Su ? a.dv.Su[cu * bb + idx] : zmake(0.0, 0.0);
-    return t.of(zsub(zmul(z, s), a.dv.Hu[cu * bb + idx]));
+  // this thread's component of the lead's A blocks at broadening eta: the onsite block, the
+  // coupling alpha away from the surface and beta back (right lead: a01, a10; left lead: swapped)
+  auto onsite = [&](double eta) {
+    const zc s = a.dv.Sd ? a.dv.Sd[cd * bb + idx] : zmake(t.r == t.c ? 1.0 : 0.0, 0.0);
+    return t.of(zsub(zmul(zmake(a.dv.E[e], eta), s), a.dv.Hd[cd * bb + idx]));
   };
-  auto a10 = [&]() {
-    const zc s = a.dv.Su ? zconj(a.dv.Su[cu * bb + cr]) : zmake(0.0, 0.0);
-    return t.of(zsub(zmul(z, s), zconj(a.dv.Hu[cu * bb + cr])));
+  auto load_hops = [&](double eta) {
+    const zc z = zmake(a.dv.E[e], eta);
+    const zc s01 = a.dv.Su ? a.dv.Su[cu * bb + idx] : zmake(0.0, 0.0);
+    const zc s10 = a.dv.Su ? zconj(a.dv.Su[cu * bb + cr]) : zmake(0.0, 0.0);
+    const double a01 = t.of(zsub(zmul(z, s01), a.dv.Hu[cu * bb + idx]));
+    const double a10 = t.of(zsub(zmul(z, s10), zconj(a.dv.Hu[cu * bb + cr])));
+    t.put(al, left ? a10 : a01);
+    t.put(be, left ? a01 : a10);
   };
-  const zc s00 = a.dv.Sd ? a.dv.Sd[cd * bb + idx] : zmake(t.r == t.c ? 1.0 : 0.0, 0.0);
-  const double a00 = t.of(zsub(zmul(z, s00), a.dv.Hd[cd * bb + idx]));
-  auto load_hops = [&]() {
-    t.put(al, left ? a10() : a01());
-    t.put(be, left ? a01() : a10());
-  };
+  const double a00 = onsite(a.dv.eta);
   // the largest |entry| of the two hops
   int turn = 0;
   auto abs2 = [&](double v) {   // |element|^2 from the two components of the thread pair
@@ -104,92 +104,140 @@ __global__ void __launch_bounds__(small_threads(kObcSmallB)) obc_small_kernel(Ob
     return sqrt(sum / b);
   };
 
-  // ---------------- decimation
-  load_hops();
-  double eps = a00, epss = a00;
-  __syncthreads();
-  const double ref = fmax(sqrt(hop_norm2()), 1e-300);
-  const double lim = a.tol * ref, lim2 = lim * lim;
-  int done = 0, iters = 0;
-  for (int it = 0; it <= a.max_iter; ++it) {
-    const double m2 = hop_norm2();
-    const bool fin = isfinite(m2);
-    if (!fin || (lim2 > 1e-280 ? m2 < lim2 : sqrt(m2) < lim)) {
-      done = fin ? 1 : 2;
-      iters = it;
-      break;
+  // the retarded root: every LDL^H pivot of i (g - g^H) is above -1e-12 times its largest
+  // diagonal entry (a pivot within that of zero is skipped), as retarded_check_kernel has it
+  auto retarded = [&]() {
+    const zc x = g[t.r * t.ld + t.c], y = g[t.c * t.ld + t.r];
+    double v = t.comp ? x.x - y.x : -(x.y + y.y);
+    const double top = cta_reduce<true>(t.on && t.r == t.c && t.comp == 0 ? fmax(v, 0.0) : 0.0, red[turn ^= 1]);
+    const double lim = 1e-12 * fmax(top, 1e-300);
+    t.put(V, v);
+    for (int p = 0; p < b; ++p) {
+      __syncthreads();
+      const double d = V[p * t.ld + p].x;
+      if (d < -lim || !isfinite(d)) return false;   // (the same in every thread)
+      if (d > lim && t.r > p && t.c > p) {          // rows and columns up to p are read only
+        const zc l = V[t.r * t.ld + p], q = V[p * t.ld + t.c];
+        v -= (t.comp ? l.x * q.y + l.y * q.x : l.x * q.x - l.y * q.y) / d;
+        t.put(V, v);
+      }
     }
-    if (it == a.max_iter) break;
-    t.put(g, eps);
+    return true;
+  };
+
+  // One pass, and where its polishing diverges further ones that decimate at a larger broadening
+  // and polish at the lead's own (restart_widen in negf_internal.cuh)
+  int done = 0, iters = 0, steps = 0;
+  double res = 0.0, kept = 0.0, kept_res = 0.0;   // (kept: of the pass before)
+#pragma unroll 1
+  for (int pass = 0;; ++pass) {
+    const double eta = pass ? restart_widen(pass - 1) * a.dv.eta : a.dv.eta;
+    const int most = pass ? kRestartSteps : 3;
+    int conv = 0, its = 0;
+    // ---------------- decimation
+    __syncthreads();
+    load_hops(eta);
+    double eps = onsite(eta), epss = eps;
+    __syncthreads();
+    const double ref = fmax(sqrt(hop_norm2()), 1e-300);
+    const double lim = a.tol * ref, lim2 = lim * lim;
+    for (int it = 0; it <= a.max_iter; ++it) {
+      const double m2 = hop_norm2();
+      const bool fin = isfinite(m2);
+      if (!fin || (lim2 > 1e-280 ? m2 < lim2 : sqrt(m2) < lim)) {
+        conv = fin ? 1 : 2;
+        its = it;
+        break;
+      }
+      if (it == a.max_iter) break;
+      t.put(g, eps);
+      __syncthreads();
+      small_inverse(g, V, t, piv);
+      t.put(T0, t.mul(al, g));          // al g
+      t.put(T1, t.mul(be, g));          // be g
+      __syncthreads();
+      const double agb = t.mul(T0, be), bga = t.mul(T1, al);
+      const double na = -t.mul(T0, al), nb = -t.mul(T1, be);
+      epss -= agb;
+      eps = (eps - agb) - bga;
+      __syncthreads();
+      t.put(al, na);
+      t.put(be, nb);
+      __syncthreads();
+    }
+    // ---------------- surface function and its residual
+    __syncthreads();
+    load_hops(a.dv.eta);
+    t.put(g, epss);
     __syncthreads();
     small_inverse(g, V, t, piv);
-    t.put(T0, t.mul(al, g));          // al g
-    t.put(T1, t.mul(be, g));          // be g
-    __syncthreads();
-    const double agb = t.mul(T0, be), bga = t.mul(T1, al);
-    const double na = -t.mul(T0, al), nb = -t.mul(T1, be);
-    epss -= agb;
-    eps = (eps - agb) - bga;
-    __syncthreads();
-    t.put(al, na);
-    t.put(be, nb);
-    __syncthreads();
-  }
-  // ---------------- surface function and its residual
-  __syncthreads();
-  load_hops();
-  t.put(g, epss);
-  __syncthreads();
-  small_inverse(g, V, t, piv);
-  double res = residual(g);
-  // ---------------- Newton polishing: D = -K^{-1} F + (K^{-1} al) D (be g)
-  int steps = 0;
-  bool need = res > a.target;
-  while (need && steps < 3) {
-    __syncthreads();
-    t.put(X, t.get(T1));
-    __syncthreads();
-    small_inverse(X, V, t, piv);                          // K^{-1}
-    const double p0 = t.mul(X, al), q0 = t.mul(be, g), s0 = -t.mul(X, F);
-    __syncthreads();
-    zc *Pm = X, *Qm = Y;
-    t.put(Pm, p0);
-    t.put(Qm, q0);
-    t.put(S, s0);
-    double sv = s0;
-    __syncthreads();
-    for (int j = 0; j < 96; ++j) {
-      t.put(T0, t.mul(Pm, S));                            // P S
-      const double pp = t.mul(Pm, Pm), qq = t.mul(Qm, Qm);   // P^2, Q^2 (of a level that may be the last)
+    res = residual(g);
+    // ---------------- Newton polishing: D = -K^{-1} F + (K^{-1} al) D (be g)
+    bool need = res > a.target;
+    bool diverged = isnan(res);
+    for (int step = 0; need && step < most; ++step) {
       __syncthreads();
-      const double inc = t.mul(T0, Qm);                   // P S Q
-      sv += inc;
-      const double mi = largest(inc), ms = largest(sv);
-      if (mi <= 1e-30 * ms || !isfinite(ms)) break;   // |increment| <= 1e-15 |S|
-      // balance P^2 against Q^2 by the power of two nearest to the square root of the ratio
-      // of their largest entries (from the exponent fields of the squared moduli)
-      const int ep = (int)(__double_as_longlong(largest(pp)) >> 52), eq = (int)(__double_as_longlong(largest(qq)) >> 52);
-      const int sh = (ep > 0 && eq > 0 && ep < 2047 && eq < 2047) ? (eq - ep) / 4 : 0;
-      const double sc = __longlong_as_double((long long)(1023 + sh) << 52);
-      const double si = __longlong_as_double((long long)(1023 - sh) << 52);
-      t.put(S, sv);
-      t.put(Pm, pp * sc);
-      t.put(Qm, qq * si);
+      t.put(X, t.get(T1));
+      __syncthreads();
+      small_inverse(X, V, t, piv);                          // K^{-1}
+      const double p0 = t.mul(X, al), q0 = t.mul(be, g), s0 = -t.mul(X, F);
+      __syncthreads();
+      zc *Pm = X, *Qm = Y;
+      t.put(Pm, p0);
+      t.put(Qm, q0);
+      t.put(S, s0);
+      double sv = s0;
+      __syncthreads();
+      for (int j = 0; j < 96; ++j) {
+        t.put(T0, t.mul(Pm, S));                            // P S
+        const double pp = t.mul(Pm, Pm), qq = t.mul(Qm, Qm);   // P^2, Q^2 (of a level that may be the last)
+        __syncthreads();
+        const double inc = t.mul(T0, Qm);                   // P S Q
+        sv += inc;
+        const double mi = largest(inc), ms = largest(sv);
+        if (mi <= 1e-30 * ms || !isfinite(ms)) break;   // |increment| <= 1e-15 |S|
+        // balance P^2 against Q^2 by the power of two nearest to the square root of the ratio
+        // of their largest entries (from the exponent fields of the squared moduli)
+        const int ep = (int)(__double_as_longlong(largest(pp)) >> 52), eq = (int)(__double_as_longlong(largest(qq)) >> 52);
+        const int sh = (ep > 0 && eq > 0 && ep < 2047 && eq < 2047) ? (eq - ep) / 4 : 0;
+        const double sc = __longlong_as_double((long long)(1023 + sh) << 52);
+        const double si = __longlong_as_double((long long)(1023 - sh) << 52);
+        t.put(S, sv);
+        t.put(Pm, pp * sc);
+        t.put(Qm, qq * si);
+        __syncthreads();
+      }
+      const double gv = t.get(g), gn = gv + sv;
+      t.put(V, gn);
+      __syncthreads();
+      const double resn = residual(V);
+      ++steps;
+      const bool take = resn < res;
+      if (take) {
+        res = resn;
+        t.put(g, gn);
+      }
+      diverged = !(resn <= kDiverged * res);
+      need = take && res > a.target;
       __syncthreads();
     }
-    const double gv = t.get(g), gn = gv + sv;
-    t.put(V, gn);
-    __syncthreads();
-    const double resn = residual(V);
-    ++steps;
-    const bool take = resn < res;
-    if (take) {
-      res = resn;
-      t.put(g, gn);
+    if (pass == 0) {
+      done = conv;
+      iters = its;
+      if (done != 1 || res <= a.accept || !diverged) break;
+      kept = t.get(g);
+      kept_res = res;
+    } else {
+      if (conv == 1 && res <= a.accept && retarded()) break;
+      if (pass == kRestarts) {
+        __syncthreads();
+        t.put(g, kept);
+        res = kept_res;
+        break;
+      }
     }
-    need = take && res > a.target;
-    __syncthreads();
   }
+  __syncthreads();
   // ---------------- outputs: g, Sigma = al g be
   const BMat& gs = left ? a.gs_L : a.gs_R;
   const BMat& sg = left ? a.sigma_L : a.sigma_R;

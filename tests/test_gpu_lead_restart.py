@@ -1,0 +1,92 @@
+"""Lead units whose Newton polishing diverges from the decimation's result are decimated again at a
+larger broadening.
+
+At eta = 1e-6 the decimation passes nearly singular blocks at a few energies, and its surface
+function then has a residual of 1e-4 and more: the seeds below hold such units (in one of the
+precisions or both; all others of their energies are ordinary ones).  Every energy has to end
+solved, by the definition: the fixed point's residual is within the accepted 1e-10 (formed here in
+complex128), and the root is the retarded one, i (g - g^H) >= 0 up to rounding.  The two precisions
+meet within 1e-6 of the largest entry: residuals of 1e-13, amplified by at most |g| / eta with
+|g| up to about 10.
+"""
+import numpy as np
+import pytest
+import torch
+
+import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def P():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2602_03438_gb300 as P
+    P.negf.load_library()
+    return P
+
+
+def device(b, ne, seed):
+    dev = W.banded_device(2, b, ne, seed, overlap=True)
+    rng = np.random.default_rng(seed)
+    dev.H_up = dev.H_up + 0.3 / np.sqrt(b) * (rng.normal(size=dev.H_up.shape) + 1j * rng.normal(size=dev.H_up.shape))
+    dev.eta = 1e-6
+    return dev
+
+
+def solve(P, ctx, devs, prec):
+    """Per device and side: (g, residual per energy, the smallest eigenvalue of i (g - g^H) over the
+    largest), and the statuses."""
+    sys_ = P.upload(devs)
+    ne, b = sum(len(d.energy) for d in devs), devs[0].H_up.shape[-1]
+    z = lambda: torch.empty(ne * b * b, dtype=torch.complex128, device="cuda")
+    sL, sR, gL, gR = z(), z(), z(), z()
+    status = torch.full((ne,), 9, dtype=torch.int32, device="cuda")
+    P.negf_obc(ctx, sys_, sL, sR, None, status, gs_L=gL, gs_R=gR, prec=prec)
+    assert ctx.sync() == 0
+    out, at = [], 0
+    for d in devs:
+        n = len(d.energy)
+        t = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+        Z = (t(d.energy) + 1j * d.eta)[:, None, None]
+        for left, gs, sg in ((True, gL, sL), (False, gR, sR)):
+            cd, cu = (0, 0) if left else (-1, -1)
+            a00 = Z * t(d.S_diag[cd]) - t(d.H_diag[cd])
+            a01, a10 = Z * t(d.S_up[cu]) - t(d.H_up[cu]), Z * t(d.S_up[cu]).mH - t(d.H_up[cu]).mH
+            al, be = (a10, a01) if left else (a01, a10)
+            g = gs.view(-1, b, b)[at:at + n]
+            r = (a00 - al @ g @ be) @ g - torch.eye(b, dtype=g.dtype, device="cuda")
+            ev = torch.linalg.eigvalsh(1j * (g - g.mH))
+            assert float((sg.view(-1, b, b)[at:at + n] - al @ g @ be).abs().max()) <= 1e-9 * float(g.abs().max())
+            out.append((g, r.flatten(1).norm(dim=1) / b ** 0.5, ev[:, 0] / ev[:, -1]))
+        at += n
+    return out, status.tolist()
+
+
+CASES = [(8, 128, 230), (32, 128, 17), (32, 128, 33), (32, 128, 41), (64, 128, 62), (128, 192, 151)]
+
+
+@pytest.mark.parametrize("b,ne,seed", CASES)
+def test_diverging_units_are_solved(P, b, ne, seed):
+    _check(P, [device(b, ne, seed)])
+
+
+@pytest.mark.parametrize("b,seeds", [(8, (3, 230)), (32, (17, 41))])
+def test_diverging_units_of_a_batch(P, b, seeds):   # devices of one block size: one work list of units
+    _check(P, [device(b, 128, s) for s in seeds])
+
+
+def _check(P, devs):
+    ctx = P.Context(0, 1 << 30)
+    try:
+        got = [solve(P, ctx, devs, prec) for prec in (P.FP64, P.MIXED)]
+        for sides, status in got:
+            assert not any(status)
+            for g, res, low in sides:
+                assert float(res.max()) <= 1e-10
+                assert float(low.min()) >= -1e-9
+        for (x, _, _), (y, _, _) in zip(got[0][0], got[1][0]):
+            assert float(((x - y).abs().amax(dim=(1, 2)) / x.abs().amax(dim=(1, 2))).max()) <= 1e-6
+    finally:
+        ctx.close()
