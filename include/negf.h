@@ -346,7 +346,10 @@ negf_status negf_observables(negf_ctx* ctx, const negf_system* sys, negf_precisi
  * double[2] (re, im).  C may be NULL (beta ignored) or equal to D; D must not
  * overlap A or B.  NEGF_FP64: FP64 FMA; NEGF_MIXED: digit-sliced FP16 tensor-core
  * product for 16 <= n <= 512 (K in exact passes of 128); NEGF_MIXED_TF32: 3-term TF32 split for n >= 16
- * (FP64 FMA outside those ranges). */
+ * (FP64 FMA outside those ranges).  In the digit-sliced product a row of op(A) or a
+ * column of op(B) that holds an infinity or a NaN makes its whole row or column of the
+ * product NaN, results past the range of a double are infinite, and results below the
+ * normal range are zero. */
 negf_status negf_block_gemm(negf_ctx* ctx, negf_precision prec, int32_t n, int32_t units, int32_t opA,
                             int32_t opB, const double* alpha, const void* A, int64_t a_stride, const void* B,
                             int64_t b_stride, const double* beta, const void* C, int64_t c_stride, void* D,

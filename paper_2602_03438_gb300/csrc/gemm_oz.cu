@@ -177,9 +177,11 @@ __device__ __forceinline__ void mma_commit(uint64_t* bar) {
 __device__ __forceinline__ unsigned int abs_hi(double x) { return (unsigned int)__double2hiint(x) & 0x7FFFFFFFu; }
 // scale exponent e with |x| < 2^(e-1) for the largest |entry|, from its abs_hi word, so that
 // the top digit stays within 64: exponent field - 1021 for a normal maximum, 0 for an
-// all-zero vector, -1021 for a subnormal maximum
+// all-zero vector, -1021 for a subnormal maximum, kNonFiniteScale for an infinity or a NaN (whose
+// digits come out as zeros)
 __device__ __forceinline__ int scale_exp_hi(unsigned int h) {
   if (h == 0) return 0;
+  if (h >= 0x7FF00000u) return kNonFiniteScale;
   const int ex = (int)(h >> 20);
   return (ex == 0 ? 1 : ex) - 1021;
 }
@@ -235,12 +237,15 @@ static_assert(HSPLIT == 4, "the halves split the groups as [0, 4) and [4, NG)");
 
 // int64 v (|v| < 2^62) times 2^p as an IEEE double: the conversion to nearest, then p added
 // to the exponent field with one integer addition (0 when v = 0 or the result would
-// fall below the normal range, far below the tile's FP64-class accuracy)
+// fall below the normal range, far below the tile's FP64-class accuracy; infinity above
+// the range; NaN where p holds a kNonFiniteScale)
 __device__ __forceinline__ double ldexp_int(long long v, int p) {
   const double x = __ll2double_rn(v);
   const int hi = __double2hiint(x);
   const int e = ((hi >> 20) & 0x7FF) + p;
+  if (p > kNonFiniteScale / 2) return __hiloint2double(0x7FF80000, 0);
   if (v == 0 || e <= 0) return 0.0;
+  if (e >= 0x7FF) return __hiloint2double((hi & (int)0x80000000) | 0x7FF00000, 0);
   return __hiloint2double(hi + (int)((unsigned)p << 20), __double2loint(x));
 }
 

@@ -202,10 +202,12 @@ __device__ __forceinline__ void part_mmas(uint32_t c, uint32_t sp, uint64_t a, u
 // digits
 // ---------------------------------------------------------------------------
 // the high word of |x| orders like the value and carries its exponent: scales from integer
-// maxima.  e with |x| < 2^(e - 1) for the largest word (0 for an all-zero vector)
+// maxima.  e with |x| < 2^(e - 1) for the largest word (0 for an all-zero vector;
+// kNonFiniteScale where it is an infinity's or a NaN's, whose digits come out as zeros)
 __device__ __forceinline__ unsigned int abs_hi(double x) { return (unsigned int)__double2hiint(x) & 0x7FFFFFFFu; }
 __device__ __forceinline__ int scale_exp_hi(unsigned int h) {
   if (h == 0) return 0;
+  if (h >= 0x7FF00000u) return kNonFiniteScale;
   const int ex = (int)(h >> 20);
   return (ex == 0 ? 1 : ex) - 1021;
 }
@@ -406,9 +408,10 @@ __device__ __forceinline__ long long combine(const uint32_t (&g)[8][4], int j) {
   return w + (long long)top * (1 << 24);
 }
 
-// v 2^p as a double (0 for v = 0 or below the normal range), |v| < 2^62, built in integers:
-// a 64-bit conversion is an FP64-pipe instruction, and a tile's 8192 of them held that
-// pipe for a third of the tile's time
+// v 2^p as a double (0 for v = 0 or below the normal range), |v| < 2^62 and p <= kMaxExp, built in
+// integers: a 64-bit conversion is an FP64-pipe instruction, and a tile's 8192 of them held
+// that pipe for a third of the tile's time
+constexpr int kMaxExp = 960;   // no result is past the range of a double up to here
 __device__ __forceinline__ double ldexp_int(long long v, int p) {
   const int sg = (int)(v >> 32) & (int)0x80000000;
   const unsigned long long a = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
@@ -418,6 +421,14 @@ __device__ __forceinline__ double ldexp_int(long long v, int p) {
   const int e = 1085 - lz + p;                                     // exponent field - 1: the leading bit adds 1
   if (lz == 64 || e < 0) return 0.0;
   return __hiloint2double((int)(r >> 32) + (e << 20) + sg, (int)(unsigned)r);
+}
+// the same for any p: infinity past the range, NaN where p holds a kNonFiniteScale
+__device__ __forceinline__ double ldexp_any(long long v, int p) {
+  if (p > kNonFiniteScale / 2) return NAN;
+  const int down = p > kMaxExp ? p - kMaxExp : 0;   // (up to 1200)
+  double x = ldexp_int(v, p - down);
+  for (int d = down; d > 0; d -= 600) x *= __hiloint2double((1023 + min(d, 600)) << 20, 0);
+  return x;
 }
 // UAB: alpha = +-1, beta in {0, +-1}; MASK: g.active may be given (its registers cost the others 3%)
 template <int ND, int TNC, bool UAB, bool MASK>
@@ -720,6 +731,36 @@ __global__ void __launch_bounds__(NT, 1) ozb_product_kernel(GemmArgs g, ImgArgs 
       const zc* Cm = (g.C.p && !(UAB && g.beta.x == 0.0)) ? g.C.at(u) : nullptr;
       const int j = lane & 7, r4 = lane >> 3;
       const int neg_a = g.alpha.x < 0.0 ? (int)0x80000000 : 0, neg_b = g.beta.x < 0.0 ? (int)0x80000000 : 0;
+      int eb_max = ebj[0];
+#pragma unroll
+      for (int h = 1; h < CW / 8; ++h) eb_max = max(eb_max, ebj[h]);
+      if (__reduce_max_sync(0xffffffffu, er) + __reduce_max_sync(0xffffffffu, eb_max) > kMaxExp) {
+        // results near the end of the range or past it: the integers through shared memory, each
+        // converted with its own check (in the path below that check cost 2% of the product)
+#pragma unroll
+        for (int h = 0; h < CW / 8; ++h) {
+#pragma unroll
+          for (int q = 0; q < 8; ++q)
+            *reinterpret_cast<longlong2*>(stg + lane * 128 + ((q ^ (lane & 7)) << 4)) = make_longlong2(vr[8 * h + q], vi[8 * h + q]);
+          __syncwarp();
+          const int gcol = n0 + 8 * h + j;
+#pragma unroll 1
+          for (int k = 0; k < 8; ++k) {
+            const int rl = 4 * k + r4, row = m0 + rl;
+            const int p = __shfl_sync(0xffffffffu, er, rl) + __shfl_sync(0xffffffffu, ebj[h], j);
+            const longlong2 x = *reinterpret_cast<const longlong2*>(stg + rl * 128 + ((j ^ (rl & 7)) << 4));
+            if (row >= n || gcol >= n) continue;
+            const zc acc = zmake(ldexp_any(x.x, p), ldexp_any(x.y, p));
+            const zc c = Cm ? Cm[(size_t)row * n + gcol] : zmake(0.0, 0.0);
+            zc v = UAB ? zmake(flip(acc.x, neg_a), flip(acc.y, neg_a)) : zmul(g.alpha, acc);
+            if (Cm) v = zadd(v, UAB ? zmake(flip(c.x, neg_b), flip(c.y, neg_b)) : zmul(g.beta, c));
+            if (g.plus_identity && row == gcol) v.x += 1.0;
+            D[(size_t)row * n + gcol] = v;
+          }
+          __syncwarp();
+        }
+        continue;
+      }
 #pragma unroll
       for (int h = 0; h < CW / 8; ++h) {
         if (n0 + 8 * h >= n) break;

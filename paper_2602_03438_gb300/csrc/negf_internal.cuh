@@ -164,6 +164,9 @@ cudaError_t zgemm_ozt_lo(const GemmArgs& g, void* scratch, int* err, cudaStream_
 // one bounded device wait that runs out after limit_ns and raises NEGF_ERR_TIMEOUT on err
 cudaError_t wait_selftest(int* err, unsigned long long limit_ns, cudaStream_t s);
 bool tc_supported(int n);
+// The scale exponent of a row or column with a NaN or an infinity in it (the others are below 1100):
+// the sliced products' results of that row or column are NaN
+constexpr int kNonFiniteScale = 1 << 20;
 // FP64-class complex GEMM on the tensor cores by exact accumulation of digit slices, all
 // digits made in the kernel (BF16, 16 <= n <= 256); `scratch` holds oz_scratch_bytes(n,
 // units) bytes of per-row/column scales
