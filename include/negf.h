@@ -144,8 +144,9 @@ negf_status negf_worklist(const negf_system* sys, int32_t bs, int32_t* count, in
  * repeats block nb-1 with hop H_{nb-2,nb-1}.  Surface Green's functions by
  * Lopez Sancho-Rubio decimation in FP64 (stop when max|alpha|,|beta| < tol *
  * initial, at most max_iter steps), followed when needed by up to 3 FP64
- * Newton steps on the surface fixed-point equation.  A unit whose Newton steps
- * diverge (the decimation passed a nearly singular block) starts again: decimation
+ * Newton steps on the surface fixed-point equation.  A unit whose decimation ends in
+ * infinities or NaN or whose Newton steps diverge (the decimation passed a nearly
+ * singular block) starts again: decimation
  * at 3, 5, 2, 8 and 16 times eta in turn, up to 6 Newton steps at eta from each, until
  * a result's residual is <= 1e-10 and it passes the retarded-root test below; if
  * none does, the first result stands.  An energy whose surface residual ||(a00 - a01 g a10) g - I||_F / sqrt(b) stays above 1e-10 gets

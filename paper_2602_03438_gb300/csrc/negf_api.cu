@@ -1736,14 +1736,16 @@ __global__ void count_kernel(const int* flags, int units, int* out) {
   if (threadIdx.x == 0) *out = c;
 }
 
-// open[u] = 1 for the decimated units (cold, converged) whose residual is not accepted and whose
-// last Newton step (residual resn) diverged; out[0] = flags set, out[1] = open units
+// open[u] = 1 for the decimated units (cold) that start again: those whose decimation ended in
+// infinities or NaN, and the converged ones whose residual is not accepted and whose last
+// Newton step (residual resn) diverged; out[0] = flags set, out[1] = open units
 __global__ void count_open_kernel(const int* flags, const int* cold, const int* done, const double* res,
                                   const double* resn, double accept, int units, int* open, int* out) {
   pdl_begin();
   int c = 0, o = 0;
   for (int u = threadIdx.x; u < units; u += blockDim.x) {
-    const int x = (cold[u] && done[u] == 1 && !(res[u] <= accept) && !(resn[u] <= kDiverged * res[u])) ? 1 : 0;
+    const bool lost = done[u] == 1 && !(res[u] <= accept) && !(resn[u] <= kDiverged * res[u]);
+    const int x = (cold[u] && (done[u] == 2 || lost)) ? 1 : 0;
     open[u] = x;
     o += x;
     c += flags[u] != 0;
@@ -1756,15 +1758,15 @@ __global__ void count_open_kernel(const int* flags, const int* cold, const int* 
   }
 }
 
-// A restart's end.  open[u]: the unit was restarted; ok[u]: its result is accepted and retarded, and
-// the unit is open no more.  Otherwise g and res become what they were (kept in the
-// outputs' Sigma blocks and res0).  save: keep them instead
+// A restart's end.  open[u]: the unit was restarted; done2[u], ok[u]: its decimation converged, and its
+// result is accepted and retarded: the unit is done and open no more.  Otherwise g and
+// res become what they were (kept in the outputs' Sigma blocks and res0).  save: keep them instead
 __global__ void restart_settle_kernel(BMat g, BMat keep_L, BMat keep_R, int U, int n, double* res, double* res0, int* open,
-                                      const int* done, const int* ok, int save) {
+                                      int* done, const int* done2, const int* ok, int save) {
   pdl_begin();
   const int u = blockIdx.x;
   if (!open[u]) return;
-  const bool good = !save && done[u] == 1 && ok[u];
+  const bool good = !save && done2[u] == 1 && ok[u];
   zc* x = g.at(u);
   zc* y = u < U ? keep_L.at(u) : keep_R.at(u - U);
   const int nn = n * n;
@@ -1776,8 +1778,8 @@ __global__ void restart_settle_kernel(BMat g, BMat keep_L, BMat keep_R, int U, i
   __syncthreads();
   if (threadIdx.x != 0) return;
   if (save) res0[u] = res[u];
-  else if (good) open[u] = 0;
-  else res[u] = res0[u];
+  else if (!good) res[u] = res0[u];
+  else open[u] = 0, done[u] = 1;
 }
 
 __global__ void set_need_kernel(const double* res, double* resn, int* need, int units, double target, const int* only) {
@@ -2792,8 +2794,8 @@ negf_status negf_obc(negf_ctx* c, const negf_system* sys, negf_precision prec, d
         q.tol = tol; q.target = target; q.accept = accept;
         q.sigma_L = lead_at(sigma_L); q.sigma_R = lead_at(sigma_R);
         q.gs_L = lead_at(gs_L); q.gs_R = lead_at(gs_R);
-        q.done = done; q.iters = it_arr; q.nsteps = nsteps; q.res = res;
-        ctx->launches += 2;
+        q.done = done; q.iters = it_arr; q.nsteps = nsteps; q.res = res; q.open = need;
+        ctx->launches += 3;
         CU(obc_small(q, s));
         const long long ob = batched ? 0 : o[2] + e0;
         launch_pdl(obc_finish_kernel, (U + 127) / 128, 128, 0, s, 
@@ -2981,7 +2983,7 @@ negf_status negf_obc(negf_ctx* c, const negf_system* sys, negf_precision prec, d
         return residual(g, res, mask);
       };
       // up to `most` Newton steps on the units in `only` above the target; n_open: how many
-      // decimated units it left outside its basin (flagged in `warm`, free by then)
+      // decimated units start again (flagged in `warm`, free by then)
       auto polish = [&](const int* only, int most, int& n_open) -> negf_status {
         negf_status sc;
         launch_pdl(set_need_kernel, (NU + 255) / 256, 256, 0, s, res, resn, need, NU, target, only);
@@ -3012,7 +3014,7 @@ negf_status negf_obc(negf_ctx* c, const negf_system* sys, negf_precision prec, d
         // restarts of the units whose polishing diverged (restart_widen; the flags in `warm` are theirs)
         const BMat kL = lead_at(sigma_L), kR = lead_at(sigma_R);
         if (n_open > 0) {
-          launch_pdl(restart_settle_kernel, NU, 256, 0, s, g, kL, kR, U, b, res, res0, warm, done, keep, 1);
+          launch_pdl(restart_settle_kernel, NU, 256, 0, s, g, kL, kR, U, b, res, res0, warm, done, done2, keep, 1);
           KCHECK();
         }
         for (int k = 0; k < kRestarts && n_open > 0; ++k) {
@@ -3030,7 +3032,7 @@ negf_status negf_obc(negf_ctx* c, const negf_system* sys, negf_precision prec, d
           launch_pdl(retarded_check_kernel, NU, 256, 0, s, g, T[0], b, keep, res, accept, 1e-12, act);
           KCHECK();
           CU(cudaMemcpyAsync(warm, keep, sizeof(int) * NU, cudaMemcpyDeviceToDevice, s));
-          launch_pdl(restart_settle_kernel, NU, 256, 0, s, g, kL, kR, U, b, res, res0, warm, done2, act, 0);
+          launch_pdl(restart_settle_kernel, NU, 256, 0, s, g, kL, kR, U, b, res, res0, warm, done, done2, act, 0);
           KCHECK();
           if ((n_open = n_set(warm)) < 0) return fail(ctx, NEGF_ERR_CUDA, "OBC: flag read-back failed");
         }

@@ -243,7 +243,7 @@ struct UnitDev {
 // unit_e[k] of device udev[unit_dev[k]] when udev is given.  done, iters, nsteps, res
 // ([2U]) as the batched path leaves them; gs_L, gs_R nullable.
 constexpr int kObcSmallB = 16;
-// A lead unit whose Newton polishing diverges starts again: decimation at restart_widen times
+// A lead unit whose decimation blows up or whose Newton polishing diverges starts again: decimation at restart_widen times
 // the broadening, then up to kRestartSteps Newton steps at its own.  Where eps is nearly singular
 // on the way (condition 1e7 to 2e9 at eta = 1e-6), rounding leaves the surface function with a
 // residual of 1e-4 to 1e-2, outside Newton's basin: the result was then wrong by 1e-5 to 1e-3,
@@ -264,7 +264,7 @@ struct ObcSmall {
   const int *unit_dev, *unit_e;
   double tol, target, accept;
   BMat sigma_L, sigma_R, gs_L, gs_R;
-  int *done, *iters, *nsteps;
+  int *done, *iters, *nsteps, *open;   // open: scratch of 2U
   double* res;
 };
 cudaError_t obc_small(const ObcSmall& a, cudaStream_t s);

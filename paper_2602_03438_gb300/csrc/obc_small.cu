@@ -3,8 +3,8 @@
 // the surface function and its residual, up to three Newton steps on the surface
 // fixed-point equation (Smith doubling of the Stein equation) and Sigma, in shared memory
 // and FP64.  The steps, their order and the stop rules are those of the batched path
-// (negf_obc), its restarts at a larger broadening included; a unit stops when it has converged
-// instead of when the batch is polled.
+// (negf_obc); a unit stops when it has converged instead of when the batch is polled.  (A second
+// launch holds the rare units that start again.)
 //
 // What bounds it: the FP64 pipe (small_block.cuh) along one unit's serial chain of six
 // products and an inverse per decimation step and four products per Smith level.
@@ -40,9 +40,13 @@ __device__ __forceinline__ double cta_reduce(double v, double* red) {
   return v;
 }
 
+// AGAIN: the restarts (restart_widen) of the units that the launch before left open, in a launch of
+// its own, which costs the others 1 us (as a loop around the one pass it cost 5 to 17)
+template <bool AGAIN>
 __global__ void __launch_bounds__(small_threads(kObcSmallB)) obc_small_kernel(ObcSmall a) {
   pdl_begin();
   const int u = blockIdx.x, b = a.b;
+  if (AGAIN && !a.open[u]) return;
   const bool left = u < a.U;
   const int k = left ? u : u - a.U;   // the energy unit
   int e = a.e0 + k;
@@ -125,19 +129,16 @@ __global__ void __launch_bounds__(small_threads(kObcSmallB)) obc_small_kernel(Ob
     return true;
   };
 
-  // One pass, and where its polishing diverges further ones that decimate at a larger broadening
-  // and polish at the lead's own (restart_widen in negf_internal.cuh)
   int done = 0, iters = 0, steps = 0;
-  double res = 0.0, kept = 0.0, kept_res = 0.0;   // (kept: of the pass before)
+  double res = 0.0;
 #pragma unroll 1
-  for (int pass = 0;; ++pass) {
-    const double eta = pass ? restart_widen(pass - 1) * a.dv.eta : a.dv.eta;
-    const int most = pass ? kRestartSteps : 3;
-    int conv = 0, its = 0;
+  for (int again = 0; again < (AGAIN ? kRestarts : 1); ++again) {
+    const double eta = AGAIN ? restart_widen(again) * a.dv.eta : a.dv.eta;
+    done = 0;
     // ---------------- decimation
     __syncthreads();
     load_hops(eta);
-    double eps = onsite(eta), epss = eps;
+    double eps = AGAIN ? onsite(eta) : a00, epss = eps;
     __syncthreads();
     const double ref = fmax(sqrt(hop_norm2()), 1e-300);
     const double lim = a.tol * ref, lim2 = lim * lim;
@@ -145,8 +146,8 @@ __global__ void __launch_bounds__(small_threads(kObcSmallB)) obc_small_kernel(Ob
       const double m2 = hop_norm2();
       const bool fin = isfinite(m2);
       if (!fin || (lim2 > 1e-280 ? m2 < lim2 : sqrt(m2) < lim)) {
-        conv = fin ? 1 : 2;
-        its = it;
+        done = fin ? 1 : 2;
+        iters = it;
         break;
       }
       if (it == a.max_iter) break;
@@ -175,7 +176,7 @@ __global__ void __launch_bounds__(small_threads(kObcSmallB)) obc_small_kernel(Ob
     // ---------------- Newton polishing: D = -K^{-1} F + (K^{-1} al) D (be g)
     bool need = res > a.target;
     bool diverged = isnan(res);
-    for (int step = 0; need && step < most; ++step) {
+    for (int step = 0; need && step < (AGAIN ? kRestartSteps : 3); ++step) {
       __syncthreads();
       t.put(X, t.get(T1));
       __syncthreads();
@@ -221,20 +222,11 @@ __global__ void __launch_bounds__(small_threads(kObcSmallB)) obc_small_kernel(Ob
       need = take && res > a.target;
       __syncthreads();
     }
-    if (pass == 0) {
-      done = conv;
-      iters = its;
-      if (done != 1 || res <= a.accept || !diverged) break;
-      kept = t.get(g);
-      kept_res = res;
+    if (!AGAIN) {
+      if (threadIdx.x == 0) a.open[u] = done == 2 || (done == 1 && !(res <= a.accept) && diverged);
     } else {
-      if (conv == 1 && res <= a.accept && retarded()) break;
-      if (pass == kRestarts) {
-        __syncthreads();
-        t.put(g, kept);
-        res = kept_res;
-        break;
-      }
+      if (done == 1 && res <= a.accept && retarded()) break;
+      if (again + 1 == kRestarts) return;   // the first result stands
     }
   }
   __syncthreads();
@@ -247,8 +239,8 @@ __global__ void __launch_bounds__(small_threads(kObcSmallB)) obc_small_kernel(Ob
   t.put_g(sg.at(k), t.mul(T0, be));
   if (threadIdx.x == 0) {
     a.done[u] = done;
-    a.iters[u] = iters;
-    a.nsteps[u] = steps;
+    if (!AGAIN) a.iters[u] = iters;
+    a.nsteps[u] = steps + (AGAIN ? a.nsteps[u] : 0);
     a.res[u] = res;
   }
 }
@@ -261,12 +253,14 @@ cudaError_t obc_small(const ObcSmall& a, cudaStream_t s) {
   if (a.U <= 0) return cudaSuccess;
   if (a.b < 1 || a.b > kObcSmallB) return cudaErrorInvalidValue;
   cudaError_t e = once_per_device(INIT_OBC_SMALL, [](int) {
-    return cudaFuncSetAttribute(obc_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)obc_small_smem(kObcSmallB));
+    const cudaFuncAttribute smem = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    const cudaError_t r = cudaFuncSetAttribute(obc_small_kernel<false>, smem, (int)obc_small_smem(kObcSmallB));
+    return r != cudaSuccess ? r : cudaFuncSetAttribute(obc_small_kernel<true>, smem, (int)obc_small_smem(kObcSmallB));
   });
   if (e != cudaSuccess) return e;
-  launch_pdl(obc_small_kernel, 2 * a.U, small_threads(a.b), obc_small_smem(a.b), s, a);
-  return cudaGetLastError();
+  e = launch_pdl(obc_small_kernel<false>, 2 * a.U, small_threads(a.b), obc_small_smem(a.b), s, a);
+  if (e != cudaSuccess) return e;
+  return launch_pdl(obc_small_kernel<true>, 2 * a.U, small_threads(a.b), obc_small_smem(a.b), s, a);
 }
 
 }  // namespace negf

@@ -52,8 +52,10 @@ def solve(P, ctx, devs, prec):
         Z = (t(d.energy) + 1j * d.eta)[:, None, None]
         for left, gs, sg in ((True, gL, sL), (False, gR, sR)):
             cd, cu = (0, 0) if left else (-1, -1)
-            a00 = Z * t(d.S_diag[cd]) - t(d.H_diag[cd])
-            a01, a10 = Z * t(d.S_up[cu]) - t(d.H_up[cu]), Z * t(d.S_up[cu]).mH - t(d.H_up[cu]).mH
+            S = torch.eye(b, dtype=torch.complex128, device="cuda") if d.S_diag is None else t(d.S_diag[cd])
+            Su = 0.0 * S if d.S_up is None else t(d.S_up[cu])
+            a00 = Z * S - t(d.H_diag[cd])
+            a01, a10 = Z * Su - t(d.H_up[cu]), Z * Su.mH - t(d.H_up[cu]).mH
             al, be = (a10, a01) if left else (a01, a10)
             g = gs.view(-1, b, b)[at:at + n]
             r = (a00 - al @ g @ be) @ g - torch.eye(b, dtype=g.dtype, device="cuda")
@@ -75,6 +77,26 @@ def test_diverging_units_are_solved(P, b, ne, seed):
 @pytest.mark.parametrize("b,seeds", [(8, (3, 230)), (32, (17, 41))])
 def test_diverging_units_of_a_batch(P, b, seeds):   # devices of one block size: one work list of units
     _check(P, [device(b, 128, s) for s in seeds])
+
+
+def test_decimation_that_blows_up_starts_again(P):
+    """Inputs drawn on the GPU: at one energy the decimation's hops end in infinities, which counted as
+    not converged whatever the surface function's residual was."""
+    b, ne = 30, 200
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(261)
+    cn = lambda n: torch.randn(n, b, b, dtype=torch.complex128, device="cuda", generator=gen)
+    r = torch.arange(b, device="cuda", dtype=torch.float64)
+    d0 = torch.exp(-(r[:, None] - r[None]).abs() / 4.0) / b ** 0.5
+    d1 = torch.exp(-(b + r[None] - r[:, None]) / 4.0) / b ** 0.5
+    x = cn(2)
+    H = 0.5 * (x + x.mH) * d0 + torch.tensor([0.1, -0.1], dtype=x.dtype, device="cuda")[:, None, None] * torch.eye(
+        b, dtype=x.dtype, device="cuda")
+    Hu = cn(1) * d1 + 0.3 / b ** 0.5 * cn(1)
+    dev = device(b, ne, 0)
+    dev.H_diag, dev.H_up, dev.S_diag, dev.S_up = H.cpu().numpy(), Hu.cpu().numpy(), None, None
+    dev.energy = torch.linspace(-3.0, 3.0, ne, dtype=torch.float64, device="cuda").cpu().numpy()
+    _check(P, [dev])
 
 
 def _check(P, devs):
