@@ -17,7 +17,11 @@
 // 2 128 2^14 = 2^22, so an accumulator is exact (2^24) for up to 4 of them.  Groups of 5
 // and more: g = 4 of ND = 7 puts one of its five into a spare accumulator; the last two
 // groups may round above 2^24, at 2^-56 and 2^-64 of the scales, far below what the dropped
-// products leave out.  Larger n runs in passes, each drained into 64-bit integers.
+// products leave out.  Larger n runs in passes, each drained into 64-bit integers that keep
+// every bit (they may wrap once: the sign that a sum had is kept beside it).  Error against 128-bit
+// sums, rms of the row x column norms, 8 digits of 7 bits before and now: normal entries n =
+// 128 2.71e-17 2.55e-17, 512 1.77e-17 1.63e-17; entries decaying from the diagonal 128
+// 1.26e-16 1.18e-16, 512 8.3e-17 8.0e-17; smaller at every size measured from 16 to 512.
 //
 // Layout: digits of op(A) are made by a pre-pass as shared-memory images in global memory,
 // [unit][row tile][chunk of 16 k][real, imaginary][digit], each plane 128 rows of 16 FP16
@@ -47,6 +51,8 @@
 // register split 624, eight producer warps 635, one drain of re and im together and three
 // waits per chunk 535.  A planes kept in the collector for two instructions each: no faster.
 #include <cuda_fp16.h>
+
+#include <type_traits>
 
 #include "negf_internal.cuh"
 
@@ -389,9 +395,9 @@ __global__ void __launch_bounds__(256) ozb_prepass_kernel(ARGS g, ImgArgs im, in
 // ---------------------------------------------------------------------------
 // the product
 // ---------------------------------------------------------------------------
-// one output's exact group sums (column j of the loaded registers) as a 64-bit integer in
-// units of 2^-56 (ND = 7; the last group's low byte rounded off, 2^-57 where the dropped
-// products leave out some 2^-54) or 2^-48 (ND = 5) of the scales: below 2^62
+// one output's group sums of a pass (column j of the loaded registers) as a 64-bit integer in units
+// of 2^-56 (ND = 7; the last group's low byte rounded off, 2^-57 where the dropped products
+// leave out some 2^-54) or 2^-48 (ND = 5) of the scales: below 2^62
 template <int ND>
 __device__ __forceinline__ long long combine(const uint32_t (&g)[8][4], int j) {
   auto G = [&](int d) { return __float2int_rn(__uint_as_float(g[d][j])); };
@@ -408,7 +414,7 @@ __device__ __forceinline__ long long combine(const uint32_t (&g)[8][4], int j) {
   return w + (long long)top * (1 << 24);
 }
 
-// v 2^p as a double (0 for v = 0 or below the normal range), |v| < 2^62 and p <= kMaxExp, built in
+// v 2^p as a double (0 for v = 0 or below the normal range), |v| < 2^63 and p <= kMaxExp, built in
 // integers: a 64-bit conversion is an FP64-pipe instruction, and a tile's 8192 of them held
 // that pipe for a third of the tile's time
 constexpr int kMaxExp = 960;   // no result is past the range of a double up to here
@@ -423,10 +429,18 @@ __device__ __forceinline__ double ldexp_int(long long v, int p) {
   return __hiloint2double((int)(r >> 32) + (e << 20) + sg, (int)(unsigned)r);
 }
 // the same for any p: infinity past the range, NaN where p holds a kNonFiniteScale
-__device__ __forceinline__ double ldexp_any(long long v, int p) {
+// other_sign: v stands 2^64 off, to the side of its sign
+__device__ __forceinline__ double ldexp_any(long long v, bool other_sign, int p) {
   if (p > kNonFiniteScale / 2) return NAN;
   const int down = p > kMaxExp ? p - kMaxExp : 0;   // (up to 1200)
-  double x = ldexp_int(v, p - down);
+  double x;
+  if (other_sign) {   // 2^63 <= |value| < 2^64
+    const bool neg = v >= 0;
+    const unsigned long long a = neg ? 0ull - (unsigned long long)v : (unsigned long long)v;
+    x = flip(ldexp_int((long long)((a >> 1) | (a & 1)), p - down + 1), neg ? (int)0x80000000 : 0);
+  } else {
+    x = ldexp_int(v, p - down);
+  }
   for (int d = down; d > 0; d -= 600) x *= __hiloint2double((1023 + min(d, 600)) << 20, 0);
   return x;
 }
@@ -676,21 +690,25 @@ __global__ void __launch_bounds__(NT, 1) ozb_product_kernel(GemmArgs g, ImgArgs 
     const uint32_t lane_base = tmem + ((uint32_t)(32 * quad) << 16);
     unsigned char* stg = base + T::OFF_ST + warp * 4096;
     uint32_t passes = 0;
-    const int xs = ND == 7 ? (chunks > 2 * PASS ? 2 : chunks > PASS ? 1 : 0) : 0;   // headroom of several passes
     for (long long i = blockIdx.x; i < ntiles && !s_fail; i += gridDim.x) {
       int u, tm, tn;
       if (!tile_at(i, u, tm, tn)) continue;
       const int m0 = tm * TM + 32 * quad, n0 = tn * TNC + cb;
       // the scales, long before they are used
-      const int er = (m0 + lane < n) ? im.ea[(size_t)u * n + m0 + lane] - (ND == 7 ? 56 : 48) + xs : 0;
+      const int er = (m0 + lane < n) ? im.ea[(size_t)u * n + m0 + lane] - (ND == 7 ? 56 : 48) : 0;
       int ebj[CW / 8];   // lane j holds column j's
 #pragma unroll
       for (int h = 0; h < CW / 8; ++h) {
         const int gcol = n0 + 8 * h + (lane & 7);
         ebj[h] = gcol < n ? im.eb[(size_t)u * n + gcol] : 0;
       }
+      // The passes' sums wrap: each is below 2^62 and four below 2^64.  Bit j of wrapped (CW + j for the
+      // imaginary part) says that column j's stands 2^64 off, to the side of its sign.
       long long vr[CW], vi[CW];
-      for (int c0 = 0; c0 < chunks; c0 += PASS) {
+      uint32_t wrapped = 0;
+      // one pass: the first, or a later one, whose sums may wrap (each in code of its own: the check's
+      // instructions in every pass cost 2% of a product of one)
+      auto drain = [&](auto first) {
         bool ok = true;
 #pragma unroll
         for (int part = 0; part < 2; ++part) {
@@ -712,20 +730,30 @@ __global__ void __launch_bounds__(NT, 1) ozb_product_kernel(GemmArgs g, ImgArgs 
             if (cc + 1 < CW / 4) fetch(cc + 1, w[(cc + 1) & 1]);
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-              long long v = combine<ND>(w[cc & 1], j);
-              if (ND == 7 && xs > 0) v = (v + (1ll << (xs - 1))) >> xs;
+              const long long v = combine<ND>(w[cc & 1], j);
               long long& o = part ? vi[4 * cc + j] : vr[4 * cc + j];
-              o = (c0 == 0) ? v : o + v;
+              if (decltype(first)::value) {
+                o = v;
+              } else if (ND < 7) {
+                o += v;
+              } else {
+                const long long t = (long long)((unsigned long long)o + (unsigned long long)v);
+                wrapped ^= ((uint32_t)(((o ^ t) & (v ^ t)) >> 32) >> 31) << (part * CW + 4 * cc + j);
+                o = t;
+              }
             }
           }
           asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
           __syncwarp();
           if (lane == 0) mbar_arrive(part ? freeI : freeR);
         }
-        if (!ok) { s_fail = 1; break; }
+        if (!ok) s_fail = 1;
         ++passes;
-      }
-      if (s_fail) break;
+        return ok;
+      };
+      bool ok = drain(std::true_type());
+      for (int c0 = PASS; ok && c0 < chunks; c0 += PASS) ok = drain(std::false_type());
+      if (!ok) break;
       // rows of this lane -> doubles -> shared memory, then 8 lanes per row: whole lines
       zc* D = g.D.at(u);
       const zc* Cm = (g.C.p && !(UAB && g.beta.x == 0.0)) ? g.C.at(u) : nullptr;
@@ -734,8 +762,9 @@ __global__ void __launch_bounds__(NT, 1) ozb_product_kernel(GemmArgs g, ImgArgs 
       int eb_max = ebj[0];
 #pragma unroll
       for (int h = 1; h < CW / 8; ++h) eb_max = max(eb_max, ebj[h]);
-      if (__reduce_max_sync(0xffffffffu, er) + __reduce_max_sync(0xffffffffu, eb_max) > kMaxExp) {
-        // results near the end of the range or past it: the integers through shared memory, each
+      if (__reduce_max_sync(0xffffffffu, er) + __reduce_max_sync(0xffffffffu, eb_max) > kMaxExp ||
+          __any_sync(0xffffffffu, wrapped != 0)) {
+        // results near the end of the range or past it, or past 64 bits: the integers through shared memory, each
         // converted with its own check (in the path below that check cost 2% of the product)
 #pragma unroll
         for (int h = 0; h < CW / 8; ++h) {
@@ -749,8 +778,9 @@ __global__ void __launch_bounds__(NT, 1) ozb_product_kernel(GemmArgs g, ImgArgs 
             const int rl = 4 * k + r4, row = m0 + rl;
             const int p = __shfl_sync(0xffffffffu, er, rl) + __shfl_sync(0xffffffffu, ebj[h], j);
             const longlong2 x = *reinterpret_cast<const longlong2*>(stg + rl * 128 + ((j ^ (rl & 7)) << 4));
+            const uint32_t off = __shfl_sync(0xffffffffu, wrapped, rl) >> (8 * h + j);
             if (row >= n || gcol >= n) continue;
-            const zc acc = zmake(ldexp_any(x.x, p), ldexp_any(x.y, p));
+            const zc acc = zmake(ldexp_any(x.x, off & 1, p), ldexp_any(x.y, (off >> CW) & 1, p));
             const zc c = Cm ? Cm[(size_t)row * n + gcol] : zmake(0.0, 0.0);
             zc v = UAB ? zmake(flip(acc.x, neg_a), flip(acc.y, neg_a)) : zmul(g.alpha, acc);
             if (Cm) v = zadd(v, UAB ? zmake(flip(c.x, neg_b), flip(c.y, neg_b)) : zmul(g.beta, c));
