@@ -652,8 +652,8 @@ struct BatchPlan {
 
 negf_status rgf_chunk(Ctx* ctx, Engine& eng, const DevView& dv, const ScatView& sc, const RgfIO& io, int e0,
                       int U, char* ws, const BatchPlan* bp = nullptr, int out_e0 = -1) {
-  // the output buffers' first block is energy eo's (e0: the caller's full arrays)
-  const int eo = out_e0 < 0 ? e0 : out_e0;
+  // the output buffers' first block is energy eo's (out_e0 < 0: the caller's full arrays)
+  const int eo = out_e0 < 0 ? 0 : out_e0;
   const int nb = bp ? bp->nb : dv.nb, b = dv.b;
   const long long bb = (long long)b * b;
   const size_t blk = sizeof(zc) * bb;
