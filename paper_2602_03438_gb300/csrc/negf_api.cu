@@ -2374,7 +2374,7 @@ static negf_status rgf_common(Ctx* ctx, const negf_system* sys, negf_precision p
     io.status = status ? status + o[2] : nullptr;
     io.lesser = lesser;
     size_t per = rgf_bytes_per_energy(dv.nb, dv.b, io, eng.mixed);
-    if (per > ctx->ws_bytes) {   // no room for every index's blocks of one energy: step by step
+    if (per > ctx->ws_bytes && rgf_small_optional(dv.b, eng.mixed)) {   // no room for every index's blocks of one energy
       io.allow_small = false;
       per = std::min(per, rgf_bytes_per_energy(dv.nb, dv.b, io, eng.mixed));
     }
@@ -3163,7 +3163,7 @@ negf_status negf_rgf_observables(negf_ctx* c, const negf_system* sys, negf_preci
       return gblocks * blk + rgf_bytes_per_energy(nb, b, io, eng.mixed) + observables_bytes_per_energy(dv, sl) + 3072;
     };
     size_t per = bytes();
-    if (per > ctx->ws_bytes) {   // as in rgf_common
+    if (per > ctx->ws_bytes && rgf_small_optional(b, eng.mixed)) {   // as in rgf_common
       io.allow_small = false;
       per = std::min(per, bytes());
     }

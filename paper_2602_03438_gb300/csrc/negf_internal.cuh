@@ -284,6 +284,7 @@ struct SmallSweep {
   int32_t* status;
 };
 bool rgf_small_supported(int b, int mixed);
+bool rgf_small_optional(int b, int mixed);   // runs step by step where the workspace is too small for the one launch
 cudaError_t rgf_small_sweep(const SmallSweep& a, cudaStream_t s);
 
 // Eq. (3) on a uniform grid: Y[e][i] = sum_{m=-M..M} w_m X[e-m][i] for i < nelem (element i

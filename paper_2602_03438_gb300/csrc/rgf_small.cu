@@ -138,6 +138,8 @@ __global__ void __launch_bounds__(small_threads(kSmallB)) rgf_small_kernel(Small
 // took 8.5 ms step by step and takes 2.0 ms in one launch
 bool rgf_small_supported(int b, int mixed) { return b >= 1 && (b < 16 || (b == 16 && mixed != 2)); }
 
+bool rgf_small_optional(int b, int mixed) { return b == 16 && mixed == 1; }
+
 size_t rgf_small_smem(int b) { return sizeof(zc) * (size_t)kBufs * small_block_elems(b); }
 
 cudaError_t rgf_small_sweep(const SmallSweep& a, cudaStream_t s) {
