@@ -144,13 +144,14 @@ negf_status negf_worklist(const negf_system* sys, int32_t bs, int32_t* count, in
  * repeats block nb-1 with hop H_{nb-2,nb-1}.  Surface Green's functions by
  * Lopez Sancho-Rubio decimation in FP64 (stop when max|alpha|,|beta| < tol *
  * initial, at most max_iter steps), followed when needed by up to 3 FP64
- * Newton steps on the surface fixed-point equation.  A unit whose decimation ends in
- * infinities or NaN or whose Newton steps diverge (the decimation passed a nearly
- * singular block) starts again: decimation
- * at 3, 5, 2, 8 and 16 times eta in turn, up to 6 Newton steps at eta from each, until
- * a result's residual is <= 1e-10 and it passes the retarded-root test below; if
- * none does, the first result stands.  An energy whose surface residual ||(a00 - a01 g a10) g - I||_F / sqrt(b) stays above 1e-10 gets
- * NEGF_ERR_NOCONV in status[e].  Sigma_L = a10 g_L a01, Sigma_R = a01 g_R a10.
+ * Newton steps on the surface fixed-point equation.  A unit whose decimation ends
+ * in infinities or NaN or whose Newton steps diverge (the decimation passed a
+ * nearly singular block) starts again: decimation at 3, 5, 2, 8 and 16 times eta
+ * in turn (at 3 only where more than 4 and than 1/16 of the units need it), up to
+ * 6 Newton steps at eta from each, until a result's residual is <= 1e-10 and it
+ * passes the retarded-root test below; if none does, the first result stands.  An
+ * energy whose surface residual ||(a00 - a01 g a10) g - I||_F / sqrt(b) stays above
+ * 1e-10 gets NEGF_ERR_NOCONV in status[e].  Sigma_L = a10 g_L a01, Sigma_R = a01 g_R a10.
  * prec: NEGF_FP64 runs every product in FP64; NEGF_MIXED runs the products of the
  * decimation, the residuals and the Newton steps on the digit-sliced FP16 tensor-core
  * path (FP64-class: FP32 accumulation of 8-bit slices, ~2^-54 of the row/column

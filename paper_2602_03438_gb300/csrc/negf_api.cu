@@ -3017,7 +3017,7 @@ negf_status negf_obc(negf_ctx* c, const negf_system* sys, negf_precision prec, d
           launch_pdl(restart_settle_kernel, NU, 256, 0, s, g, kL, kR, U, b, res, res0, warm, done, done2, keep, 1);
           KCHECK();
         }
-        for (int k = 0; k < kRestarts && n_open > 0; ++k) {
+        for (int k = 0; k < kRestarts && n_open > 0 && (k == 0 || n_open <= restart_many(NU)); ++k) {
           la.eps = eps.p; la.epss = epss.p; la.al = al.p; la.be = be.p;
           la.widen = restart_widen(k);
           la.only = warm;

@@ -257,6 +257,9 @@ constexpr int kObcSmallB = 16;
 constexpr int kRestarts = 5, kRestartSteps = 6;
 constexpr double kDiverged = 100.0;
 __host__ __device__ constexpr double restart_widen(int k) { return k == 0 ? 3.0 : k == 1 ? 5.0 : k == 2 ? 2.0 : k == 3 ? 8.0 : 16.0; }
+// Where more units are open than this, the cause is not a chance one (a broadening below what the
+// decimation can resolve): one restart is tried, not all
+__host__ __device__ constexpr int restart_many(int units) { return units / 16 > 4 ? units / 16 : 4; }
 struct ObcSmall {
   DevView dv;
   int e0, U, b, max_iter;

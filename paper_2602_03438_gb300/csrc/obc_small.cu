@@ -46,7 +46,13 @@ template <bool AGAIN>
 __global__ void __launch_bounds__(small_threads(kObcSmallB)) obc_small_kernel(ObcSmall a) {
   pdl_begin();
   const int u = blockIdx.x, b = a.b;
-  if (AGAIN && !a.open[u]) return;
+  int passes = 1;
+  if (AGAIN) {
+    if (!a.open[u]) return;
+    int open = 0;
+    for (int i = 0; i < 2 * a.U; i += blockDim.x) open += __syncthreads_count(i + threadIdx.x < 2 * a.U && a.open[i + threadIdx.x]);
+    passes = open <= restart_many(2 * a.U) ? kRestarts : 1;
+  }
   const bool left = u < a.U;
   const int k = left ? u : u - a.U;   // the energy unit
   int e = a.e0 + k;
@@ -132,7 +138,7 @@ __global__ void __launch_bounds__(small_threads(kObcSmallB)) obc_small_kernel(Ob
   int done = 0, iters = 0, steps = 0;
   double res = 0.0;
 #pragma unroll 1
-  for (int again = 0; again < (AGAIN ? kRestarts : 1); ++again) {
+  for (int again = 0; again < passes; ++again) {
     const double eta = AGAIN ? restart_widen(again) * a.dv.eta : a.dv.eta;
     done = 0;
     // ---------------- decimation
@@ -226,7 +232,7 @@ __global__ void __launch_bounds__(small_threads(kObcSmallB)) obc_small_kernel(Ob
       if (threadIdx.x == 0) a.open[u] = done == 2 || (done == 1 && !(res <= a.accept) && diverged);
     } else {
       if (done == 1 && res <= a.accept && retarded()) break;
-      if (again + 1 == kRestarts) return;   // the first result stands
+      if (again + 1 == passes) return;   // the first result stands
     }
   }
   __syncthreads();

@@ -99,6 +99,32 @@ def test_decimation_that_blows_up_starts_again(P):
     _check(P, [dev])
 
 
+@pytest.mark.parametrize("b", [8, 48])
+def test_one_restart_where_most_units_diverge(P, b):
+    """Energies within 1e-9 of a level of the onsite block at eta = 1e-9: beyond what the decimation can
+    resolve.  Unsolved energies are reported; more than a sixteenth of the units take one restart (3
+    and 6 Newton steps at most), not all."""
+    ne = 40
+    dev = device(b, ne, b)
+    dev.S_diag = dev.S_up = None
+    dev.eta = 1e-9
+    dev.energy = np.linalg.eigvalsh(dev.H_diag[0])[b // 2] + np.linspace(-1e-9, 1e-9, ne)
+    sys_ = P.upload(dev)
+    z = lambda: torch.empty(ne * b * b, dtype=torch.complex128, device="cuda")
+    ctx = P.Context(0, 1 << 29)
+    try:
+        for prec in (P.FP64, P.MIXED):
+            status = torch.full((ne,), 9, dtype=torch.int32, device="cuda")
+            newton = torch.zeros(2 * ne, dtype=torch.int32, device="cuda")
+            P.negf_obc(ctx, sys_, z(), z(), None, status, newton=newton, prec=prec)
+            assert ctx.sync() == 0
+            assert set(status.tolist()) <= {0, P.negf.NEGF_ERR_NOCONV}
+            if int((status != 0).sum()) > 2 * ne // 16:
+                assert int(newton.max()) <= 9
+    finally:
+        ctx.close()
+
+
 def _check(P, devs):
     ctx = P.Context(0, 1 << 30)
     try:
