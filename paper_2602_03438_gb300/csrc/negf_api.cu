@@ -518,7 +518,7 @@ struct Engine {
     return e;
   }
   // l1, l2: two adjacent blocks per unit that are free meanwhile (nullable), lent to the FP64
-  // inverse as scratch; few: some tens of the mask's units at most
+  // inverse as scratch; few: see zinv
   cudaError_t inv(BMat X, BMat M, int n, int units, const int* active, int single, int32_t* status, BMat l1 = BMat{nullptr, 0},
                   BMat l2 = BMat{nullptr, 0}, bool few = false) {
     const bool masked = active != nullptr && active_frac < 0.0;   // an unknown share of the work
@@ -2829,7 +2829,9 @@ negf_status negf_obc(negf_ctx* c, const negf_system* sys, negf_precision prec, d
         launch_pdl(refine_check_kernel, NU, book_threads(b), 0, s, T[0], b, mask, 1e-7, redo);
         KCHECK();
         // units whose refinement converges slowly (kappa(eps) up to ~1e7) take two more
-        // steps; FP64 Gauss-Jordan for what is left
+        // steps; FP64 Gauss-Jordan for what is left: none or a few of most inverses.  (Onsite
+        // levels all at resonance leave every unit to the first inverse; a count read back
+        // with the polls comes too late to tell, and those after it then paid for empty tiles.)
         CU(eng.refine_steps(X, M, b, NU, T[0], T[1], 2, redo));
         launch_pdl(refine_check_kernel, NU, book_threads(b), 0, s, T[0], b, redo, 1e-7, redo);
         KCHECK();

@@ -189,7 +189,9 @@ cudaError_t zgemm_ozt_variant(const GemmArgs& g, void* scratch, int* err, cudaSt
 // complex of the working precision).  status[u] (nullable, indexed status_base+u)
 // gets NEGF_ERR_SINGULAR on an exactly zero pivot.
 // `lent` (lent_bytes, nullable): 16-byte aligned scratch the caller does not need meanwhile.
-// few: some tens of the mask's units are set at most.
+// few: the mask is expected to be empty or nearly so.  With more units set the result is the same and
+// the time above the launches' (n = 128, FP64: none of 384 set 6 us against 110, 4 414 : 429, 16
+// 680 : 538, 400 8.9 : 5.7 ms).
 cudaError_t zinv(BMat X, BMat M, int n, int units, const int* active, int single, void* scratch,
                  int32_t* status, cudaStream_t s, void* lent = nullptr, size_t lent_bytes = 0, bool few = false);
 size_t zinv_scratch_bytes(int n, int units, int single);
