@@ -401,7 +401,7 @@ negf_status negf_block_gemm_noalloc(int32_t n, int32_t units, int32_t opA, int32
 /* Autotuner of the NEGF_MIXED block products' tile shapes.  Variants:
  *   1 = tiles of 128 rows x 16 complex columns (n <= 128),
  *   2 = tiles of 128 x 32 (n <= 128),
- *   3 = tiles of 128 x 32 (any n, K in exact passes of 128),
+ *   3 = tiles of 128 x 32 (any n, K in passes of 128): where 2 is supported, 2,
  *   0 = the built-in rule (the narrow tiles where they take fewer or no more rounds of the
  *       GPU's SMs, else the wide ones).
  * negf_tune_products times every variant that supports n on `units` random n x n

@@ -3344,6 +3344,10 @@ negf_status negf_tune_products(negf_ctx* c, int32_t n, int32_t units, int32_t* c
   for (int v = OZ_HALF; v < OZ_NVARIANT; ++v) {
     if (ms) ms[v] = -1.0;
     if (!oz_variant_supported(n, v)) continue;
+    if (v == OZ_FULL && oz_variant_supported(n, OZ_PERSISTENT)) {   // the same tiles: timed as 2
+      if (ms) ms[v] = ms[OZ_PERSISTENT];
+      continue;
+    }
     CU(zgemm_ozt_variant(g, scratch, ctx->d_err, s, v));   // warm-up
     CU(cudaEventRecord(e0, s));
     constexpr int reps = 3;

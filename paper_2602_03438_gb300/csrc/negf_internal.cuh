@@ -102,9 +102,9 @@ struct GemmArgs {
   int units;           // batch
   const int* active;   // per unit, nullable: 0 => unit skipped
   int plus_identity = 0;   // sliced kernels: D += I after the rest (the residual I - M X in one product)
-  // sliced kernels with n <= 128: op(A)'s scales and digit images are still in the scratch
-  // from the previous product on the same op(A) (same layout, units and mask), so that
-  // only op(B)'s column scales are made before the product
+  // byte-digit product: op(A)'s scales and digit images are still in the scratch from the
+  // previous product on the same op(A) (same layout, units, mask and variant), so that only
+  // op(B)'s column scales are made before the product
   int reuse_a = 0;
 };
 
@@ -178,7 +178,8 @@ size_t oz_scratch_bytes(int n, int units);
 bool oz_supported(int n);
 size_t ozt_scratch_bytes(int n, int units);
 // tile variants (the autotuner's choices): the default rule, tiles of 16 complex columns
-// (n <= 128), tiles of 32 (n <= 128), tiles of 32 (any n)
+// (n <= 128), tiles of 32 (n <= 128), tiles of 32 (any n).  The last two are one kernel: both
+// numbers stand in saved tunings.
 enum OzVariant { OZ_DEFAULT = 0, OZ_HALF = 1, OZ_PERSISTENT = 2, OZ_FULL = 3, OZ_NVARIANT = 4 };
 bool oz_variant_supported(int n, int variant);
 cudaError_t zgemm_ozt_variant(const GemmArgs& g, void* scratch, int* err, cudaStream_t s, int variant);

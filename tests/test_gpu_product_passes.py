@@ -64,3 +64,18 @@ def test_sums_past_63_bits(P, n, sign, value):
     want[1, 0] = 0.0
     want[1, :, 1] *= -1.0
     assert float((D - want).abs().max()) <= n * 2.0 ** -50
+
+
+def test_the_two_names_of_the_wide_tiles_are_timed_once(P):
+    import ctypes as C
+    ctx = P.Context(0, 1 << 28)
+    try:
+        for n, names in ((64, (1, 2, 3)), (200, (3,))):
+            choice, ms = C.c_int32(), (C.c_double * 4)()
+            ctx.check(ctx.lib.negf_tune_products(ctx.h, n, 32, C.byref(choice), ms, None))
+            assert [v for v in range(4) if ms[v] > 0.0] == list(names)
+            assert ms[choice.value] == min(ms[v] for v in names)
+            if n <= 128:
+                assert ms[2] == ms[3] and choice.value != 3
+    finally:
+        ctx.close()
