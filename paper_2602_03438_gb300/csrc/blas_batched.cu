@@ -34,7 +34,9 @@ cudaError_t once_per_device(int slot, const std::function<cudaError_t(int device
 // partitions, so the kernel is bound by 4 n FP64 FMAs per element and nothing else: the
 // one load pair per 256 clocks of the pipe needs no staging, while square tiles spent
 // the pipe on padding.  With C: 96 units of n = 40 206 -> 55 us, 20 of 100 473 -> 149 us, 512 of
-// 8 71 -> 14 us, 128 of 128 2117 -> 1776 us (1.21 TFLOP/s).
+// 8 71 -> 14 us, 128 of 128 2117 -> 1776 us (1.21 TFLOP/s), 8 of 256 1066 -> 882, 2 of 512 2117 ->
+// 1751, one of 1000 8158 -> 6517 us.  Conjugated operands, which a warp reads with a stride of n, take
+// the same time to 0.2% at every size from 8 to 1000 (the pipe hides them).
 // ---------------------------------------------------------------------------
 constexpr int kF64Threads = 128;
 __global__ void __launch_bounds__(kF64Threads) zgemm_f64_kernel(GemmArgs g) {
@@ -273,24 +275,30 @@ static cudaError_t launch_inv(BMat X, BMat M, int n, int units, const int* activ
 }
 
 // FP64 inverses run as column tiles over several CTAs per block (inv_tiles.cu) where there is
-// scratch for it and one CTA per block (a flat time up to 152 units) would leave SMs idle or
-// keep the matrix in global memory.  Measured (us, tiles : one CTA): n = 32, 96 blocks 124 :
-// 111; n = 40, 96 blocks 154 : 163, 400 349 : 476; n = 48, 152 blocks 251 : 228, 300 348 : 451; n = 56, 96
-// blocks 260 : 347; n = 64, 152 blocks 393 : 413, 600 1137 : 1634; n = 72, 80 blocks 444 : 553, 152 765 :
-// 554; n = 96, 80 blocks 736 : 1098, 300 2447 : 2189; n = 128, 16 blocks 538 : 2504, 400 5745 : 7629.
+// scratch for it and one CTA per block (a flat time up to kSms units, then the next round) would
+// leave SMs idle or keep the matrix in global memory.  Measured (us, tiles : one CTA) around the
+// lines: n = 40, 96 blocks 157 : 164, 104 158 : 165, 112 172 : 163, 160 201 : 318; n = 44, 76 178 : 194, 96
+// 200 : 195, 304 370 : 383; n = 48, 104 208 : 228, 112 223 : 230, 152 253 : 229; n = 52, 96 255 : 268, 112
+// 256 : 268, 152 320 : 269; n = 36, 64 136 : 137, 104 151 : 138; n = 56, 152 328 : 346; n = 64, 152 394 :
+// 415, 600 1139 : 1632; n = 72, 76 441 : 554, 112 575 : 554, 160 802 : 1095, 400 1879 : 1639; n = 96, 76
+// 676 : 1099, 152 1295 : 1099; n = 111, 152 1730 : 1667, 600 6591 : 6656; n = 128, 16 538 : 2504, 400
+// 5745 : 7629.  From 65 to 111 the line at 76 leaves the tiles' gain up to some 110 unused.
 static bool f64_tiles(int n, int units) {
-  if (n > 64) return n >= 112 || units <= 76;
-  return n >= 56 || (n >= 40 && (units <= 96 || units > 152));
+  if (n > 64) return n >= 112 || units <= kSms / 2;
+  return n >= 56 || (n >= 40 && (units <= 96 || units > kSms));
 }
 
 // FP32 blocks up to 128 are inverted in registers, one CTA per block and SM, in rounds of 120 us
 // at n = 128; tiles take about 100 us + 0.6 per block and win where the last round of the
-// registers is far from full (n = 128, us, tiles : registers: 152 blocks 187 : 125, 200 214 : 241,
-// 304 260 : 244, 400 324 : 359, 512 406 : 476, 1024 821 : 830; n = 100, 300 208 : 189; n = 96, 512 237 :
-// 246).  A mask may leave few of the units.
+// registers is far from full.  Measured (us, tiles : registers, with the refinement) at n = 97: 152
+// blocks 445 : 385, 153 484 : 509, 230 644 : 637, 304 759 : 735, 305 796 : 854, 456 1083 : 1070, 460 1117 :
+// 1186, 1024 2313 : 2330; n = 112: 152 469 : 414, 160 526 : 563, 260 718 : 723, 304 800 : 792, 400 1031 :
+// 1077, 1024 2447 : 2516; n = 128: 153 565 : 619, 230 745 : 763, 304 873 : 858, 305 908 : 1009, 456 1245 :
+// 1243, 512 1396 : 1475, 1024 2679 : 2700.  The line, drawn for n = 128, is within 1% of the better
+// side for 97 to 127 too; n = 96, 512 alone 237 : 246.  A mask may leave few of the units.
 bool f32_tiles(int n, int units, const int* active) {
   if (n <= 96 || n > 128) return n > 128;
-  return !active && units > 152 && 500 + 3ll * units < 600ll * ((units + 151) / 152);
+  return !active && units > kSms && 500 + 3ll * units < 600ll * ((units + kSms - 1) / kSms);
 }
 
 cudaError_t zinv(BMat X, BMat M, int n, int units, const int* active, int single, void* scratch,

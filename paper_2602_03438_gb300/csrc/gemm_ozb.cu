@@ -837,7 +837,6 @@ __global__ void __launch_bounds__(NT, 1) ozb_product_kernel(GemmArgs g, ImgArgs 
   }
 }
 
-constexpr long long kSms = 152;   // of a GB300, for the choice of the tile width
 int g_sms[kMaxDevices];   // multiprocessors per device (set with the kernels' attributes)
 
 template <int ND, int TNC>

@@ -25,6 +25,8 @@ enum InitSlot { INIT_OZ = 0, INIT_TC, INIT_MLP, INIT_SMALL, INIT_OBC_SMALL, INIT
 constexpr int kMaxDevices = 64;
 cudaError_t once_per_device(int slot, const std::function<cudaError_t(int device)>& init);
 
+constexpr int kSms = 152;   // multiprocessors of a GB300, for the rules that choose a kernel by rounds of them
+
 // Launches that may start while the kernel before them on the stream drains: `k` calls
 // pdl_begin() before it touches global memory (every thread, before any return), which waits
 // until that kernel has finished.  What is saved is the launch latency and the set-up behind a
