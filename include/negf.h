@@ -64,14 +64,16 @@ typedef enum {
 
 typedef enum {
   NEGF_FP64 = 0,       /* every product, inverse and reduction in FP64                      */
-  NEGF_MIXED = 1,      /* block products on the FP16 tensor cores with exact FP32
-                          accumulation of 8-bit digit slices (FP64-class: ~2^-54 of the
-                          row/column scales with the 7 digits of
-                          negf_sliced_digits; 16 <= b <= 512, K in exact passes of 128;
-                          FP64 FMA otherwise); block inverses in FP32 + two refinement
-                          steps whose residual uses the same product and whose correction
-                          a 5-digit one; devices with b < 16 run their sweeps in FP64 (one
-                          launch); I/O complex128                                           */
+  NEGF_MIXED = 1,      /* block products on the FP16 tensor cores from 8-bit digit slices
+                          accumulated in FP32 (FP64-class: ~2^-54 of the row/column scales
+                          with the 7 digits of negf_sliced_digits.  The sums are exact in
+                          the digit groups down to 2^-48 of the scales; the last two groups
+                          may round at 2^-56 and 2^-64, and results are kept in units of
+                          2^-56.  16 <= b <= 512, K in passes of 128 whose sums lose
+                          nothing; FP64 FMA otherwise); block inverses in FP32 + two
+                          refinement steps whose residual uses the same product and whose
+                          correction a 5-digit one; a device alone in its block size with
+                          b <= 16 runs its sweeps in FP64 (one launch); I/O complex128      */
   NEGF_MIXED_TF32 = 2  /* block products as 3-term TF32 splits (hi*hi + hi*lo + lo*hi) on
                           the tensor cores, FP32 accumulate in TMEM (~1e-6 relative per
                           128-wide product); inverses FP32 + refinement with an FP64
@@ -347,7 +349,7 @@ negf_status negf_observables(negf_ctx* ctx, const negf_system* sys, negf_precisi
  * by all units).  op: 0 = as stored, 2 = conjugate transpose.  alpha, beta: host
  * double[2] (re, im).  C may be NULL (beta ignored) or equal to D; D must not
  * overlap A or B.  NEGF_FP64: FP64 FMA; NEGF_MIXED: digit-sliced FP16 tensor-core
- * product for 16 <= n <= 512 (K in exact passes of 128); NEGF_MIXED_TF32: 3-term TF32 split for n >= 16
+ * product for 16 <= n <= 512 (K in passes of 128); NEGF_MIXED_TF32: 3-term TF32 split for n >= 16
  * (FP64 FMA outside those ranges).  In the digit-sliced product a row of op(A) or a
  * column of op(B) that holds an infinity or a NaN makes its whole row or column of the
  * product NaN, results past the range of a double are infinite, and results below the
@@ -418,7 +420,8 @@ negf_status negf_set_product_variant(negf_ctx* ctx, int32_t n, int32_t variant);
 /* Digits per value of the NEGF_MIXED block product (7, of 8 bits): ND digits give ND (ND +
  * 1) / 2 FP16 slice products per complex product and an error of ~2^-54 of the row x
  * column scales.  (negf_block_gemm_noalloc and calls whose workspace holds scales only
- * use 8 digits of 7 bits in BF16.)  Not a paper operation: introspection for measurement. */
+ * use 8 digits of 7 bits in BF16; NEGF_OZ_DIGITS at compile time, 6..8, sets the number
+ * for these alone.)  Not a paper operation: introspection for measurement. */
 int32_t negf_sliced_digits(void);
 
 /* Kernel timing (the tracing facility).  When enabled, every launch of the
