@@ -218,8 +218,10 @@ __global__ void __launch_bounds__(kInvThreads) zinv_kernel(BMat X, BMat M, int n
         } else {
           C w = (mc == k) ? zero : ((r == p) ? kr : W[i]);
           const C f = fcol[r];
-          w.x = fma(-f.x, pc.x, fma(f.y, pc.y, w.x));
-          w.y = fma(-f.x, pc.y, fma(-f.y, pc.x, w.y));
+          // (the product first: one rounding of the entry's own size; as two FMAs onto w, FP64 took a
+          // third less time and had a third more error)
+          w.x = w.x - (f.x * pc.x - f.y * pc.y);
+          w.y = w.y - (f.x * pc.y + f.y * pc.x);
           W[i] = w;
         }
       }
@@ -276,16 +278,16 @@ static cudaError_t launch_inv(BMat X, BMat M, int n, int units, const int* activ
 
 // FP64 inverses run as column tiles over several CTAs per block (inv_tiles.cu) where there is
 // scratch for it and one CTA per block (a flat time up to kSms units, then the next round) would
-// leave SMs idle or keep the matrix in global memory.  Measured (us, tiles : one CTA) around the
-// lines: n = 40, 96 blocks 157 : 164, 104 158 : 165, 112 172 : 163, 160 201 : 318; n = 44, 76 178 : 194, 96
-// 200 : 195, 304 370 : 383; n = 48, 104 208 : 228, 112 223 : 230, 152 253 : 229; n = 52, 96 255 : 268, 112
-// 256 : 268, 152 320 : 269; n = 36, 64 136 : 137, 104 151 : 138; n = 56, 152 328 : 346; n = 64, 152 394 :
-// 415, 600 1139 : 1632; n = 72, 76 441 : 554, 112 575 : 554, 160 802 : 1095, 400 1879 : 1639; n = 96, 76
-// 676 : 1099, 152 1295 : 1099; n = 111, 152 1730 : 1667, 600 6591 : 6656; n = 128, 16 538 : 2504, 400
-// 5745 : 7629.  From 65 to 111 the line at 76 leaves the tiles' gain up to some 110 unused.
+// leave SMs idle or keep the matrix in global memory.  Measured (us, tiles : one CTA): n = 16, 152
+// blocks 63 : 50, 160 63 : 92, 800 158 : 261; n = 20, 304 127 : 125; n = 24, 64 91 : 85, 160 101 : 159; n =
+// 28, 8 104 : 108, 90 111 : 107, 304 203 : 209; n = 32, 64 117 : 133, 96 128 : 132, 120 131 : 133, 152 143 :
+// 133, 160 144 : 256; n = 36, 96 153 : 169, 112 171 : 169, 152 199 : 170; n = 40, 1 137 : 206, 136 181 : 206,
+// 152 208 : 207, 400 364 : 603; n = 44, 152 255 : 252; n = 48, 152 263 : 303; n = 64, 8 213 : 586, 152 412 :
+// 588, 600 1200 : 2325; n = 72, 152 814 : 805, 400 1984 : 2391; n = 96, 60 675 : 1690, 300 2620 : 3363; n =
+// 111, 152 1826 : 2597; n = 128, 16 558 : 3818, 400 6115 : 11459.
 static bool f64_tiles(int n, int units) {
-  if (n > 64) return n >= 112 || units <= kSms / 2;
-  return n >= 56 || (n >= 40 && (units <= 96 || units > kSms));
+  if (n >= 40) return true;
+  return (n >= 32 && units <= 96) || (n >= 16 && units > kSms);
 }
 
 // FP32 blocks up to 128 are inverted in registers, one CTA per block and SM, in rounds of 120 us

@@ -20,7 +20,7 @@
 // the FP64 pipe at 64 clocks) of every warp of one CTA and one barrier, plus a launch per
 // panel; the updates (W and C from L2) run beside them.  Measured (GB300) against one CTA
 // per block: FP32 n = 512, 16 blocks 27.9 -> 0.88 ms; n = 256, 8 blocks 4.01 -> 0.27 ms; FP64
-// n = 128, one block 2.50 -> 0.41 ms, 400 blocks 7.6 -> 5.7 ms; n = 512, 2 blocks 138 -> 5.5 ms.
+// n = 128, one block 3.81 -> 0.43 ms, 400 blocks 11.5 -> 6.1 ms; n = 512, 2 blocks 223 -> 5.4 ms.
 // TW: a row's entries fit in 32 registers, and the update reads C once for TW columns.
 #include <algorithm>
 #include <type_traits>
@@ -205,6 +205,16 @@ __device__ __forceinline__ void tile_step(const TileInv<typename Tr<R>::C>& g, i
       for (int i = n - panel * TW + r / TW; i < TW; i += NT / TW) yk[i][r % TW] = czero<C>();
     }
     __syncthreads();
+    // FP64: the panel's share summed apart and added once, so that an entry takes one rounding of its
+    // own size per panel and not 16.  Error over the condition number, rms of 40 blocks, against one
+    // CTA per block with the product formed first: n = 40 5.7e-17 : 6.4e-17, 64 7.3e-17 : 9.0e-17, 100
+    // 7.9e-17 : 1.24e-16, 128 9.1e-17 : 1.21e-16.  Time 3% to 7% (n = 128, 400 blocks 5.73 -> 6.11 ms).
+    constexpr bool APART = sizeof(R) == 8;
+    C sum[APART ? TW : 1];
+    if (APART) {
+#pragma unroll
+      for (int c = 0; c < (APART ? TW : 1); ++c) sum[c] = czero<C>();
+    }
 #pragma unroll 2
     for (int k = 0; k < TW; k += V) {
       alignas(16) C f[V];
@@ -218,8 +228,15 @@ __device__ __forceinline__ void tile_step(const TileInv<typename Tr<R>::C>& g, i
           alignas(16) C y[V];
           *reinterpret_cast<uint4*>(y) = *reinterpret_cast<const uint4*>(&yk[k + x][c]);
 #pragma unroll
-          for (int z = 0; z < V; ++z) cfma(a[c + z], f[x], y[z]);
+          for (int z = 0; z < V; ++z) cfma(APART ? sum[APART ? c + z : 0] : a[c + z], f[x], y[z]);
         }
+    }
+    if (APART) {
+#pragma unroll
+      for (int c = 0; c < (APART ? TW : 1); ++c) {
+        a[c].x += sum[c].x;
+        a[c].y += sum[c].y;
+      }
     }
   }
 
